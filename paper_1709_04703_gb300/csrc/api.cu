@@ -625,12 +625,15 @@ void smooth2(pm_ctx* ctx, Grid u, Grid b, float h2, int per, float g, bool zero_
   }
 }
 
-// V(2,2) cycle on level-0 grids (u0, b0).  On levels of side >= FUSED_MIN
-// the two pre- and two post-smoothing sweeps are each one fused pass
-// (k_rbgs2): the pre-smoothing starts from zero on every level but, in the
-// plain path, the finest one, where it writes a scratch grid instead of u0;
-// the prolongation writes u + P uc to a second grid that the post-smoothing
-// reads back into u.  Smaller levels take four one-colour passes in place.
+// V(2,2) cycle on level-0 grids (u0, b0).  Every leg down that starts from
+// zero (all but the finest one's in the plain path and in later V-cycles on
+// one correction) is one fused launch (k_tile.cu) into the level's scratch
+// grid; the leg up from it is fused as well below side FUSED_MIN, and above
+// it the prolongation followed by the z-marching two-sweep pass (k_rbgs2),
+// which updates less halo.  A leg down that does not start from zero, and the
+// ball solve's masked levels, take k_rbgs2 from side FUSED_MIN (the
+// pre-smoothing writes a scratch grid instead of u0) or four one-colour
+// passes in place, and the separate transfers.
 pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
   const int per = ctx->periodic;
   const int L = (int)ctx->ls.size() - 1;
@@ -662,7 +665,34 @@ pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
   // thread-block cluster (k_cmg.cu)
   int Lc = 0;
   while (Lc < L && ctx->ls[Lc] > cmg_top_side(ball ? 1 : cmg_cluster())) ++Lc;
+  auto tiled = [&](int l) { return !ball && (l > 0 || zero0); };
+  auto tile_args = [&](int l) {
+    TileArgs a;
+    a.u = U[l];
+    a.b = B[l];
+    a.w = compact_view(ctx->lu2[l], ctx->ls[l]);
+    a.uc = U[l + 1];
+    a.bc = B[l + 1];
+    a.h2 = h2;
+    a.inv_h2 = 1.0f / h2;
+    a.gam = gam(l);
+    a.gam_c = gam(l + 1);
+    a.d0 = 6.0f + ctx->sig * h2;
+    a.periodic = per;
+    return a;
+  };
   for (int l = 0; l < Lc; ++l) {
+    if (tiled(l)) {
+      int e = l == 0 ? prof_begin(ctx) : -1;
+      Upre[l] = compact_view(ctx->lu2[l], ctx->ls[l]);
+      launch_tile(ctx->st, tile_args(l), false, tile_small(ctx->ls[l]));
+      if (l == 0) {
+        prof_end(ctx, PM_PROF_SMOOTH0, e, (24.0 + 9.0) * c0);
+        ec = prof_begin(ctx);
+      }
+      h2 *= 4.0f;
+      continue;
+    }
     int e = l == 0 ? prof_begin(ctx) : -1;
     // below level 0 the restriction zeroes the coarse iterate
     const bool zs = l == 0 ? zero0 : true;
@@ -698,6 +728,11 @@ pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
     if (l == 0) {
       prof_end(ctx, PM_PROF_COARSE, ec, (Lc > 0 ? 8.0 / 7.0 * 81.0 * c0 / 8.0 : 0.0));
       e = prof_begin(ctx);
+    }
+    if (tiled(l) && ctx->ls[l] < FUSED_MIN) {
+      launch_tile(ctx->st, tile_args(l), true, tile_small(ctx->ls[l]));
+      if (l == 0) prof_end(ctx, PM_PROF_SMOOTH0, e, (24.0 + 8.5) * c0);
+      continue;
     }
     const bool fused = ctx->ls[l] >= FUSED_MIN && (!ball || l == 0);
     const float d0 = 6.0f + ctx->sig * h2;
@@ -2478,7 +2513,8 @@ struct pm_batch {
   unsigned long long* h_cnt = nullptr;
   int* d_ovf = nullptr;
   BTab t_dep, t_src, t_bnd, t_pred, t_def, t_grad, t_gat, t_scan, t_scat;
-  std::vector<BTab> t_vc;  // V-cycle launch slots
+  std::vector<BTab> t_vc;  // V-cycle launch slots of the persistent solve
+  std::vector<BTab> t_leg; // the graph solve's fused legs: 2 l + (0 down, 1 up)
   int maxLc = 0;
   bool tables_stale = true;
   // the graph solve: init, defect, decision, a conditional while loop over
@@ -2486,8 +2522,7 @@ struct pm_batch {
   cudaGraphExec_t sgraph = nullptr;
   cudaStream_t st2 = nullptr;  // captures the loop's body
   long long loop_kernels = 0;  // kernels of one pass of the loop body
-  int rb_bx = 32, rb_by = 8;  // block shape of the batched colour pass (autotuned)
-  bool rb_tuned = false;
+  std::vector<char> leg_small;  // per level: its fused legs take the small tiles (autotuned)
   // the persistent solve: one cooperative launch per solve
   bool persistent = false;
   double wait_s = 2.0;         // longest wait at one grid barrier
@@ -2578,7 +2613,30 @@ int slot_bottom(int maxLc) { return 5 * maxLc; }
 int slot_up(int maxLc, int l, int k) { return 5 * maxLc + 1 + 5 * l + k; }  // k: 0 prolong, 1..4 sweeps
 int n_slots(int maxLc) { return 10 * maxLc + 1; }
 
-// Upload the descriptor tables of every V-cycle slot for the current cubes.
+// Upload the descriptor table of the bottom (every realisation's first level
+// small enough for one CTA or cluster).
+void upload_bottom_table(pm_batch* B) {
+  std::vector<CmgDesc> d;
+  std::vector<int> bl;
+  for (int r = 0; r < B->R; ++r) {
+    pm_ctx* c = B->ctx[r];
+    int Lc = first_small_level(c);
+    CmgDesc e{};
+    e.u = compact_view(c->lu[Lc], c->ls[Lc]);
+    e.b = compact_view(c->lb[Lc], c->ls[Lc]);
+    e.level = Lc;
+    e.periodic = c->periodic;
+    e.sweeps = COARSE_SWEEPS;
+    e.zero_top = 1;
+    set_dims(e, r, dim3(1, 1, 1));
+    d.push_back(e);
+    bl.push_back(1);
+  }
+  tab_upload(B, B->t_vc[slot_bottom(B->maxLc)], d, bl);
+}
+
+// Upload the descriptor tables of every V-cycle slot of the persistent solve
+// for the current cubes.
 void upload_vcycle_tables(pm_batch* B) {
   const int R = B->R, M = B->maxLc;
   for (int l = 0; l < M; ++l) {
@@ -2600,9 +2658,9 @@ void upload_vcycle_tables(pm_batch* B) {
           // the black one after it its own cells); coarser: the restriction
           // zeroed it
           e.zero_start = k == 0 ? 1 : (k == 1 ? 2 : 0);
-          set_dims(e, r, rbgs_grid_b(c->ls[l], B->rb_bx, B->rb_by));
+          set_dims(e, r, rbgs_grid_b(c->ls[l], 32, 8));
           d.push_back(e);
-          bl.push_back(nblocks(rbgs_grid_b(c->ls[l], B->rb_bx, B->rb_by)));
+          bl.push_back(nblocks(rbgs_grid_b(c->ls[l], 32, 8)));
         }
         tab_upload(B, B->t_vc[slot_down(l, k)], d, bl);
       } else {
@@ -2626,25 +2684,7 @@ void upload_vcycle_tables(pm_batch* B) {
       }
     }
   }
-  {  // bottom
-    std::vector<CmgDesc> d;
-    std::vector<int> bl;
-    for (int r = 0; r < R; ++r) {
-      pm_ctx* c = B->ctx[r];
-      int Lc = first_small_level(c);
-      CmgDesc e{};
-      e.u = compact_view(c->lu[Lc], c->ls[Lc]);
-      e.b = compact_view(c->lb[Lc], c->ls[Lc]);
-      e.level = Lc;
-      e.periodic = c->periodic;
-      e.sweeps = COARSE_SWEEPS;
-      e.zero_top = 1;
-      set_dims(e, r, dim3(1, 1, 1));
-      d.push_back(e);
-      bl.push_back(1);
-    }
-    tab_upload(B, B->t_vc[slot_bottom(M)], d, bl);
-  }
+  upload_bottom_table(B);
   for (int l = 0; l < M; ++l) {
     for (int k = 0; k < 5; ++k) {  // up
       std::vector<int> bl;
@@ -2676,9 +2716,9 @@ void upload_vcycle_tables(pm_batch* B) {
           e.color = (k - 1) & 1;
           e.periodic = c->periodic;
           e.zero_start = 0;
-          set_dims(e, r, rbgs_grid_b(c->ls[l], B->rb_bx, B->rb_by));
+          set_dims(e, r, rbgs_grid_b(c->ls[l], 32, 8));
           d.push_back(e);
-          bl.push_back(nblocks(rbgs_grid_b(c->ls[l], B->rb_bx, B->rb_by)));
+          bl.push_back(nblocks(rbgs_grid_b(c->ls[l], 32, 8)));
         }
         tab_upload(B, B->t_vc[slot_up(M, l, k)], d, bl);
       }
@@ -2686,78 +2726,89 @@ void upload_vcycle_tables(pm_batch* B) {
   }
 }
 
-// Launch the V-cycle slots (captured once into a graph, grids at their
-// largest; members and their grids come from the tables).
-void launch_vcycle_slots(pm_batch* B, cudaStream_t st) {
-  const int M = B->maxLc;
-  const int* act = B->d_active;
-  for (int l = 0; l < M; ++l) {
-    for (int k = 0; k < 4; ++k) {
-      BTab& t = B->t_vc[slot_down(l, k)];
-      launch_rbgs_b(st, t.grid_max, (const RbgsDesc*)t.d_desc, t.d_tab, act, B->rb_bx,
-                    B->rb_by);
+// Upload the descriptor tables of the graph solve's fused legs (and of the
+// bottom) for the current cubes: one launch per level and direction over
+// every realisation that has the level above its bottom.
+void upload_leg_tables(pm_batch* B) {
+  for (int l = 0; l < B->maxLc; ++l) {
+    std::vector<TileDesc> d;
+    std::vector<int> bl;
+    for (int r = 0; r < B->R; ++r) {
+      pm_ctx* c = B->ctx[r];
+      if (l >= first_small_level(c)) continue;
+      TileDesc e{};
+      e.a.u = compact_view(c->lu[l], c->ls[l]);
+      e.a.b = compact_view(c->lb[l], c->ls[l]);
+      e.a.w = compact_view(c->lu2[l], c->ls[l]);
+      e.a.uc = compact_view(c->lu[l + 1], c->ls[l + 1]);
+      e.a.bc = compact_view(c->lb[l + 1], c->ls[l + 1]);
+      e.a.h2 = (float)(1 << (2 * l));
+      e.a.inv_h2 = 1.0f / e.a.h2;
+      e.a.gam = level_gam(l);
+      e.a.gam_c = level_gam(l + 1);
+      e.a.d0 = 6.0f;
+      e.a.periodic = c->periodic;
+      const dim3 g = tile_grid(c->ls[l], B->leg_small[l] != 0);
+      set_dims(e, r, g);
+      d.push_back(e);
+      bl.push_back(nblocks(g));
     }
-    BTab& t = B->t_vc[slot_down(l, 4)];
-    launch_restrict_b(st, t.grid_max, (const RestrictDesc*)t.d_desc, t.d_tab, act);
+    for (int leg = 0; leg < 2; ++leg) tab_upload(B, B->t_leg[2 * l + leg], d, bl);
   }
-  BTab& tb = B->t_vc[slot_bottom(M)];
-  // one cluster per realisation, shared memory for the largest top level
-  launch_cmg_b(st, B->R, cmg_top_side(cmg_cluster()), (const CmgDesc*)tb.d_desc, act);
-  for (int l = M - 1; l >= 0; --l) {
-    BTab& tp = B->t_vc[slot_up(M, l, 0)];
-    launch_prolong_b(st, tp.grid_max, (const ProlongDesc*)tp.d_desc, tp.d_tab, act);
-    for (int k = 1; k < 5; ++k) {
-      BTab& t = B->t_vc[slot_up(M, l, k)];
-      launch_rbgs_b(st, t.grid_max, (const RbgsDesc*)t.d_desc, t.d_tab, act, B->rb_bx,
-                    B->rb_by);
-    }
-  }
+  upload_bottom_table(B);
 }
 
-// Autotuner of the batched colour pass: before the V-cycle graph is
-// captured, the down-sweep passes of every level run with each candidate
-// block shape on the batch's own grids (they only write the levels'
-// iterates, which every V-cycle restarts from zero) and the fastest shape
-// is kept.  Every shape computes the same cells with the same arithmetic:
-// the choice changes the time, not the bits.
-pm_status tune_rbgs(pm_batch* B) {
-  static const int shapes[4][2] = {{32, 8}, {32, 4}, {16, 8}, {64, 4}};
+// One fused leg of level l over the batch (active NULL: every realisation).
+void launch_leg(pm_batch* B, cudaStream_t st, int l, bool up, const int* active) {
+  BTab& t = B->t_leg[2 * l + (up ? 1 : 0)];
+  launch_tile_b(st, t.grid_max, (const TileDesc*)t.d_desc, t.d_tab, active, up,
+                B->leg_small[l] != 0);
+}
+
+// Launch the V-cycle (captured once into a graph, grids at their largest;
+// members and their grids come from the tables).
+void launch_vcycle_legs(pm_batch* B, cudaStream_t st) {
+  const int M = B->maxLc;
+  for (int l = 0; l < M; ++l) launch_leg(B, st, l, false, B->d_active);
+  BTab& tb = B->t_vc[slot_bottom(M)];
+  // one cluster per realisation, shared memory for the largest top level
+  launch_cmg_b(st, B->R, cmg_top_side(cmg_cluster()), (const CmgDesc*)tb.d_desc, B->d_active);
+  for (int l = M - 1; l >= 0; --l) launch_leg(B, st, l, true, B->d_active);
+}
+
+// Autotuner of the fused legs: before the V-cycle graph is captured, each
+// level's down leg runs with both tile shapes on the batch's own grids (it
+// writes only the level's scratch grid and the coarse right-hand side, which
+// every V-cycle rewrites) and the faster shape is kept.  Both compute the
+// same cells with the same arithmetic: the choice changes the time, not the
+// bits.
+pm_status tune_legs(pm_batch* B) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return bfail(B, PM_ECUDA, "pm_batch: event creation failed");
   const int M = B->maxLc;
-  float best = 1e30f;
-  int pick = 0;
-  for (int q = 0; q < 4; ++q) {
-    B->rb_bx = shapes[q][0];
-    B->rb_by = shapes[q][1];
-    upload_vcycle_tables(B);
-    float tot = 0.0f;
-    for (int rep = 0; rep < 3; ++rep) {  // the first pass warms up
-      cudaEventRecord(e0, B->st);
-      for (int l = 0; l < M; ++l)
-        for (int k = 0; k < 4; ++k) {
-          BTab& t = B->t_vc[slot_down(l, k)];
-          launch_rbgs_b(B->st, t.grid_max, (const RbgsDesc*)t.d_desc, t.d_tab, nullptr,
-                        B->rb_bx, B->rb_by);
-        }
-      cudaEventRecord(e1, B->st);
-      cudaEventSynchronize(e1);
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (rep > 0) tot += ms;
-    }
-    if (tot < best) {
-      best = tot;
-      pick = q;
-    }
+  std::vector<float> tot[2];
+  for (int q = 0; q < 2; ++q) {
+    B->leg_small.assign(M, (char)q);
+    for (auto& t : B->t_leg) t.grid_max = 0;
+    upload_leg_tables(B);
+    tot[q].assign(M, 0.0f);
+    for (int l = 0; l < M; ++l)
+      for (int rep = 0; rep < 3; ++rep) {  // the first pass warms up
+        cudaEventRecord(e0, B->st);
+        launch_leg(B, B->st, l, false, nullptr);
+        cudaEventRecord(e1, B->st);
+        cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (rep > 0) tot[q][l] += ms;
+      }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  B->rb_bx = shapes[pick][0];
-  B->rb_by = shapes[pick][1];
-  upload_vcycle_tables(B);
-  B->rb_tuned = true;
+  for (int l = 0; l < M; ++l) B->leg_small[l] = tot[1][l] < tot[0][l];
+  for (auto& t : B->t_leg) t.grid_max = 0;
+  upload_leg_tables(B);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? PM_OK : bfail(B, PM_ECUDA, cudaGetErrorString(e));
 }
@@ -2809,7 +2860,7 @@ pm_status build_solve_graph(pm_batch* B) {
                                         cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
         lb0 = g_launches.load();
-        launch_vcycle_slots(B, B->st2);
+        launch_vcycle_legs(B, B->st2);
         decide(B->st2);
         lb1 = g_launches.load();
         e = cudaStreamEndCapture(B->st2, &body);
@@ -2966,14 +3017,13 @@ pm_status batch_solve_persistent(pm_batch* B) {
 
 // One launch of the solve graph (captured at the first solve).
 pm_status batch_solve_graph(pm_batch* B) {
-  if (B->tables_stale) {
-    upload_vcycle_tables(B);
-    B->tables_stale = false;
-  }
-  if (!B->rb_tuned) {
-    pm_status st = tune_rbgs(B);
+  if (B->leg_small.empty() && B->maxLc > 0) {
+    pm_status st = tune_legs(B);
     if (st != PM_OK) return st;
+  } else if (B->tables_stale) {
+    upload_leg_tables(B);
   }
+  B->tables_stale = false;
   upload_defect_table(B, B->d_iters);
   upload_grad_table(B, B->d_iters);
   if (!B->sgraph) {
@@ -3173,6 +3223,11 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         size_t sz = std::max(std::max(sizeof(RbgsDesc), sizeof(RestrictDesc)),
                              std::max(sizeof(ProlongDesc), sizeof(CmgDesc)));
         pm_status st = tab_alloc(B, t, sz);
+        if (st != PM_OK) return st;
+      }
+      B->t_leg.resize(2 * M);
+      for (auto& t : B->t_leg) {
+        pm_status st = tab_alloc(B, t, sizeof(TileDesc));
         if (st != PM_OK) return st;
       }
     }
@@ -3442,10 +3497,6 @@ pm_status pm_batch_set_solve(pm_batch* B, int32_t persistent, double wait_second
                                "(coarse levels in a cluster, or grid not resident)");
   if (persistent != (int)B->persistent) {
     B->persistent = persistent != 0;
-    // block shape of the colour pass: the persistent kernel's, or autotuned
-    B->rb_bx = 32;
-    B->rb_by = 8;
-    B->rb_tuned = B->persistent;
     B->tables_stale = true;
     if (B->sgraph) {
       cudaStreamSynchronize(B->st);
@@ -3470,6 +3521,7 @@ void pm_batch_destroy(pm_batch* B) {
                   &B->t_gat, &B->t_scan, &B->t_scat})
     tab_free(*t);
   for (auto& t : B->t_vc) tab_free(t);
+  for (auto& t : B->t_leg) tab_free(t);
   if (B->d_active) cudaFree(B->d_active);
   if (B->d_bar) cudaFree(B->d_bar);
   if (B->h_bar) cudaFreeHost(B->h_bar);

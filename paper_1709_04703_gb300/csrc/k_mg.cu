@@ -761,35 +761,6 @@ void launch_sum_phi(cudaStream_t st, Grid ph, Grid pl, double* partial, unsigned
 // ---------------------------------------------------------------------------
 // Batched forms (one launch over the member realisations of a table).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) kb_rbgs(const RbgsDesc* d, const BTable* t,
-                                               const int* active) {
-  int q;
-  BI bi;
-  if (!batch_map(d, t, active, q, bi)) return;
-  const RbgsDesc& e = d[q];
-  each_plane(bi, e.u.s, [&](const BI& b) {
-    d_rbgs<false>(b, e.u, e.b, e.h2, e.color, e.periodic, e.gam, e.zero_start, 6.0f);
-  });
-}
-__global__ void __launch_bounds__(256) kb_restrict(const RestrictDesc* d, const BTable* t,
-                                                   const int* active) {
-  int q;
-  BI bi;
-  if (!batch_map(d, t, active, q, bi)) return;
-  const RestrictDesc& e = d[q];
-  each_plane(bi, e.uc.s, [&](const BI& b) {
-    d_resid_restrict<false>(b, e.u, e.b, e.inv_h2, e.uc, e.bc, e.periodic, e.gam, 6.0f);
-  });
-}
-__global__ void __launch_bounds__(256) kb_prolong(const ProlongDesc* d, const BTable* t,
-                                                  const int* active) {
-  int q;
-  BI bi;
-  if (!batch_map(d, t, active, q, bi)) return;
-  const ProlongDesc& e = d[q];
-  each_plane(bi, e.u.s,
-             [&](const BI& b) { d_prolong<false>(b, e.uc, e.u, e.periodic, e.gam_c); });
-}
 __global__ void __launch_bounds__(256, 4) kb_defect(const DefectDesc* d, const BTable* t,
                                                  const int* active) {
   int q;
@@ -865,24 +836,6 @@ __global__ void __launch_bounds__(256) kb_predict(const PredictDesc* d, const BT
   each_plane(bi, e.ph.s, [&](const BI& b) { d_predict(b, e.ph, e.pl, e.qh, e.ql, e.w, e.pair); });
 }
 
-void launch_rbgs_b(cudaStream_t st, int grid, const RbgsDesc* d, const BTable* t,
-                   const int* active, int bx, int by) {
-  if (grid <= 0) return;
-  kb_rbgs<<<grid, dim3(bx, by), 0, st>>>(d, t, active);
-  note_launch();
-}
-void launch_restrict_b(cudaStream_t st, int grid, const RestrictDesc* d, const BTable* t,
-                       const int* active) {
-  if (grid <= 0) return;
-  kb_restrict<<<grid, dim3(32, 8), 0, st>>>(d, t, active);
-  note_launch();
-}
-void launch_prolong_b(cudaStream_t st, int grid, const ProlongDesc* d, const BTable* t,
-                      const int* active) {
-  if (grid <= 0) return;
-  kb_prolong<<<grid, dim3(32, 8), 0, st>>>(d, t, active);
-  note_launch();
-}
 void launch_defect_b(cudaStream_t st, int grid, const DefectDesc* d, const BTable* t,
                      const int* active) {
   if (grid <= 0) return;

@@ -240,6 +240,26 @@ struct ProlongDesc {
   int periodic;
   int r, gx, gy, gz;
 };
+// k_tile.cu: the fused V-cycle legs of the mid levels.  Down: two sweeps
+// from zero on (w, b), residual restricted into bc (uc is not read and need
+// not be cleared: every coarser leg starts from zero).  Up: u = two sweeps
+// from w + P uc.  Interiors only; w and u distinct.
+struct TileArgs {
+  Grid u, b, w, uc, bc;
+  float h2, inv_h2, gam, gam_c, d0;
+  int periodic;
+};
+struct TileDesc {
+  TileArgs a;
+  int r, gx, gy, gz;
+};
+// levels up to this side take 8^3 tiles, larger ones 16 x 16 x 8
+constexpr int TILE_SMALL_MAX = 48;
+bool tile_small(int s);
+dim3 tile_grid(int s, bool small);
+void launch_tile(cudaStream_t st, const TileArgs& a, bool up, bool small);
+void launch_tile_b(cudaStream_t st, int grid, const TileDesc* d, const BTable* t,
+                   const int* active, bool up, bool small);
 struct CmgDesc {
   Grid u, b;
   int level, periodic, sweeps, zero_top;
@@ -342,12 +362,6 @@ struct ScatterDesc {
 
 // batched launchers: `grid` blocks (the members' total, or more), tables in
 // device memory, `active` (may be NULL) masks realisations by index
-void launch_rbgs_b(cudaStream_t st, int grid, const RbgsDesc* d, const BTable* t,
-                   const int* active, int bx, int by);
-void launch_restrict_b(cudaStream_t st, int grid, const RestrictDesc* d, const BTable* t,
-                       const int* active);
-void launch_prolong_b(cudaStream_t st, int grid, const ProlongDesc* d, const BTable* t,
-                      const int* active);
 // batched: cluster c solves entry c of d (n_desc entries, one per
 // realisation; entries whose realisation is inactive are skipped); shared
 // memory for tops up to max_top
