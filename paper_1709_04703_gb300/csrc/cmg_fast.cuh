@@ -1,4 +1,6 @@
 // The coarse levels of the multigrid V-cycle (Sec. 2.1, Eq. 3) in one CTA,
+// as the ball solve's masked levels and the persistent batched solve take
+// them (unmasked launches take cmg_col.cuh),
 // for tops of side <= 16 (16, 14, 12, 10, 8, 7, 6, 5, 4, 3, 2): the sides are template
 // constants, so every index is plain constant arithmetic, and each level's
 // unknowns carry a one-cell halo in shared memory that holds the open

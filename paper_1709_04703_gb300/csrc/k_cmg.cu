@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "cmg_dev.cuh"
+#include "cmg_col.cuh"
 #include "cmg_fast.cuh"
 
 namespace pm {
@@ -18,20 +19,16 @@ namespace {
 
 template <int CL>
 __global__ void __launch_bounds__(CC_NT, 1) k_cmg(Grid u, Grid b, int level, int periodic,
-                                                  int sweeps, int zero_top, float sig0,
-                                                  int fast) {
+                                                  int sweeps, int zero_top, float sig0) {
   pdl_wait();
   pdl_release();
   extern __shared__ float cc_sm[];
   __shared__ float red[CC_NT / 32];
-  if (CL == 1 && (fast || u.mbase) && fc_supported(u.s)) {
-    if (u.mbase)
+  if (u.mbase) {  // the ball solve: masked tops (q 2^j <= 16) are all supported
+    if (CL == 1 && fc_supported(u.s))
       fc_vcycle<CC_NT, true>(cc_sm, red, u, b, level, periodic, sweeps, zero_top, sig0);
-    else
-      fc_vcycle<CC_NT, false>(cc_sm, red, u, b, level, periodic, sweeps, zero_top, sig0);
     return;
   }
-  if (u.mbase) return;  // not reached: masked tops (q 2^j <= 16) are all supported
   __shared__ CcLevel lev[CC_MAXL];
   __shared__ int nlev;
   if (threadIdx.x == 0) Cc<CL>::init_levels(lev, nlev, u.s, level, periodic, sig0);
@@ -55,18 +52,13 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cmg(Grid u, Grid b, int level, int
 // (realisations whose solve has converged are skipped, by whole clusters)
 template <int CL>
 __global__ void __launch_bounds__(CC_NT, 1) kb_cmg(const CmgDesc* d, int n_desc,
-                                                   const int* active, int fast) {
+                                                   const int* active) {
   extern __shared__ float cc_sm[];
   __shared__ float red[CC_NT / 32];
   const int q = blockIdx.x / CL;
   if (q >= n_desc) return;
   const CmgDesc& e = d[q];
   if (active && !active[e.r]) return;
-  if (CL == 1 && fast && fc_supported(e.u.s)) {
-    fc_vcycle<CC_NT, false>(cc_sm, red, e.u, e.b, e.level, e.periodic, e.sweeps, e.zero_top,
-                            0.0f);
-    return;
-  }
   __shared__ CcLevel lev[CC_MAXL];
   __shared__ int nlev;
   if (threadIdx.x == 0) Cc<CL>::init_levels(lev, nlev, e.u.s, e.level, e.periodic, 0.0f);
@@ -86,8 +78,34 @@ __global__ void __launch_bounds__(CC_NT, 1) kb_cmg(const CmgDesc* d, int n_desc,
   c.run(e.zero_top, red);
 }
 
+// one CTA from an unmasked top <= 16 (cmg_col.cuh), and its batched form:
+// CTA c takes table entry c
+__device__ __forceinline__ void cmg_one(float* sm, const Grid& u, const Grid& b, int level,
+                                        int periodic, int sweeps, int zero_top, float sig0) {
+  if (cl_supported(u.s))
+    cl_vcycle(sm, u, b, level, periodic, sweeps, zero_top, sig0);
+  else if (threadIdx.x < 32)
+    cl_only_bottom(sm, u, b, level, periodic, sweeps, zero_top, sig0);
+}
+__global__ void __launch_bounds__(CL_NT) k_cmg_col(Grid u, Grid b, int level, int periodic,
+                                                   int sweeps, int zero_top, float sig0) {
+  extern __shared__ float cc_sm[];
+  pdl_wait();
+  pdl_release();
+  cmg_one(cc_sm, u, b, level, periodic, sweeps, zero_top, sig0);
+}
+__global__ void __launch_bounds__(CL_NT) kb_cmg_col(const CmgDesc* d, int n_desc,
+                                                    const int* active) {
+  extern __shared__ float cc_sm[];
+  const int q = blockIdx.x;
+  if (q >= n_desc) return;
+  const CmgDesc& e = d[q];
+  if (active && !active[e.r]) return;
+  cmg_one(cc_sm, e.u, e.b, e.level, e.periodic, e.sweeps, e.zero_top, 0.0f);
+}
+
 int g_cmg_cl = 1;  // CTAs per cluster of this process's launches (set by cmg_prepare)
-int g_cmg_fast = 1;  // one-CTA tops <= 16 take the constant-side form (cmg_fast.cuh)
+int g_cmg_fast = 1;  // unmasked one-CTA tops <= 16 take the column form (cmg_col.cuh)
 
 // dynamic shared memory of a coarse-level launch from tops up to `top`
 int cmg_smem(int top, int CL) {
@@ -164,6 +182,11 @@ cudaError_t cmg_prepare() {
   // the cluster of the coarse levels: 16 CTAs (levels <= 64^3), 8 (<= 32^3)
   // or one CTA (<= 16^3) when the GPU holds it; PM_NO_CLUSTER forces one CTA
   cudaError_t e = cmg_attrs<1>();
+  const int col = (int)sizeof(float) * CL_SMEM;
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_cmg_col, cudaFuncAttributeMaxDynamicSharedMemorySize, col);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kb_cmg_col, cudaFuncAttributeMaxDynamicSharedMemorySize, col);
   if (e != cudaSuccess) return e;
   g_cmg_cl = 1;
   // PM_CMG_GENERIC: the generic one-CTA form for every top (the same bits)
@@ -193,13 +216,17 @@ void launch_cmg(cudaStream_t st, Grid u, Grid b, int level, int periodic, int sw
   // the ball solve's masked levels take the one-CTA constant-side form
   switch (u.mbase ? 1 : g_cmg_cl) {
     case 16:
-      cmg_launch<16>(k_cmg<16>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0, 0);
+      cmg_launch<16>(k_cmg<16>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0);
       break;
     case 8:
-      cmg_launch<8>(k_cmg<8>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0, 0);
+      cmg_launch<8>(k_cmg<8>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0);
       break;
     default:
-      cmg_launch<1>(k_cmg<1>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0, g_cmg_fast);
+      if (!u.mbase && g_cmg_fast && fc_supported(u.s))
+        launch_pdl(k_cmg_col, dim3(1), dim3(cl_supported(u.s) ? cl_threads(u.s) : 32),
+                   sizeof(float) * CL_SMEM, st, u, b, level, periodic, sweeps, z, sig0);
+      else
+        cmg_launch<1>(k_cmg<1>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0);
       break;
   }
   note_launch();
@@ -207,10 +234,13 @@ void launch_cmg(cudaStream_t st, Grid u, Grid b, int level, int periodic, int sw
 
 void launch_cmg_b(cudaStream_t st, int n_desc, int max_top, const CmgDesc* d, const int* active) {
   switch (g_cmg_cl) {
-    case 16: cmg_launch<16>(kb_cmg<16>, n_desc, max_top, st, d, n_desc, active, 0); break;
-    case 8: cmg_launch<8>(kb_cmg<8>, n_desc, max_top, st, d, n_desc, active, 0); break;
+    case 16: cmg_launch<16>(kb_cmg<16>, n_desc, max_top, st, d, n_desc, active); break;
+    case 8: cmg_launch<8>(kb_cmg<8>, n_desc, max_top, st, d, n_desc, active); break;
     default:
-      cmg_launch<1>(kb_cmg<1>, n_desc, max_top, st, d, n_desc, active, g_cmg_fast);
+      if (g_cmg_fast)  // every top of an unclustered batch is at most 16: supported
+        kb_cmg_col<<<n_desc, CL_NT, sizeof(float) * CL_SMEM, st>>>(d, n_desc, active);
+      else
+        cmg_launch<1>(kb_cmg<1>, n_desc, max_top, st, d, n_desc, active);
       break;
   }
   note_launch();
