@@ -1923,13 +1923,15 @@ pm_status pm_sort_particles(const float* pos4_dev, const float* mom4_dev, int64_
 
 namespace {
 // Device work space of one P(k) call: CIC counts, contrast, its R2C
-// transform, bin accumulators (3 per bin + the escape counter) and slopes.
+// transform, bin accumulators (3 per bin + the escape counter), slopes and
+// the window's per-axis tables.
 struct PkWork {
   unsigned long long* rho = nullptr;
   float* delta = nullptr;
   cufftComplex* dk = nullptr;
   double* acc = nullptr;
   double* nu = nullptr;
+  void* axes = nullptr;
   cufftHandle plan = 0;
   bool have_plan = false;
   ~PkWork() {
@@ -1939,6 +1941,7 @@ struct PkWork {
     cudaFree(dk);
     cudaFree(acc);
     cudaFree(nu);
+    cudaFree(axes);
   }
 };
 
@@ -1952,7 +1955,8 @@ pm_status pk_transform(PkWork& w, const char* who, const float* pos4_dev, int64_
       cudaMalloc((void**)&w.delta, sizeof(float) * cells) != cudaSuccess ||
       cudaMalloc((void**)&w.dk, sizeof(cufftComplex) * modes) != cudaSuccess ||
       cudaMalloc((void**)&w.acc, sizeof(double) * (3 * n_bins + 1)) != cudaSuccess ||
-      cudaMalloc((void**)&w.nu, sizeof(double) * n_bins) != cudaSuccess)
+      cudaMalloc((void**)&w.nu, sizeof(double) * n_bins) != cudaSuccess ||
+      cudaMalloc(&w.axes, pk_axes_bytes(n_mesh)) != cudaSuccess)
     return fail(nullptr, PM_ENOMEM, std::string(who) + ": cudaMalloc failed");
   cudaMemsetAsync(w.rho, 0, sizeof(unsigned long long) * cells, st);
   cudaMemsetAsync(w.acc, 0, sizeof(double) * (3 * n_bins + 1), st);
@@ -2018,7 +2022,10 @@ pm_status pm_power_spectrum(const float* pos4_dev, int64_t n, double box, int32_
   pm_status ret = pk_transform(w, "pm_power_spectrum", pos4_dev, n, n_mesh, n_bins, st);
   if (ret != PM_OK) return ret;
   const double shot = subtract_shot ? box * box * box / (double)n : 0.0;
-  launch_pk_bin(st, (const float2*)w.dk, n_mesh, box, shot, n_bins, w.acc);
+  if (launch_pk_axes(st, w.axes, n_mesh, box, 0) != cudaSuccess ||
+      launch_pk_modes(st, (const float2*)w.dk, n_mesh, box, shot, n_bins, 0, w.axes, nullptr,
+                      w.acc) != cudaSuccess)
+    return fail(nullptr, PM_ECUDA, "pm_power_spectrum: launching the binning failed");
   return pk_read(w, "pm_power_spectrum", n_bins, st, k_out, pk_out, modes_out);
 }
 
@@ -2039,7 +2046,10 @@ pm_status pm_power_spectrum_jing(const float* pos4_dev, int64_t n, double box, i
   const double shot = subtract_shot ? box * box * box / (double)n : 0.0;
   std::vector<double> k(n_bins), p(n_bins), c(n_bins), nu(n_bins, -1.0);
   // first-order estimate for the starting slopes
-  launch_pk_bin(st, (const float2*)w.dk, n_mesh, box, shot, n_bins, w.acc);
+  if (launch_pk_axes(st, w.axes, n_mesh, box, alias_range) != cudaSuccess ||
+      launch_pk_modes(st, (const float2*)w.dk, n_mesh, box, shot, n_bins, 0, w.axes, nullptr,
+                      w.acc) != cudaSuccess)
+    return fail(nullptr, PM_ECUDA, std::string(who) + ": launching the binning failed");
   ret = pk_read(w, who, n_bins, st, k.data(), p.data(), c.data());
   if (ret != PM_OK) return ret;
   pk_slopes(k, p, nu);
@@ -2048,8 +2058,9 @@ pm_status pm_power_spectrum_jing(const float* pos4_dev, int64_t n, double box, i
     if (cudaMemcpyAsync(w.nu, nu.data(), sizeof(double) * n_bins, cudaMemcpyHostToDevice,
                         st) != cudaSuccess)
       return fail(nullptr, PM_ECUDA, std::string(who) + ": uploading slopes failed");
-    launch_pk_jing(st, (const float2*)w.dk, n_mesh, box, shot, n_bins, alias_range, w.nu,
-                   w.acc);
+    if (launch_pk_modes(st, (const float2*)w.dk, n_mesh, box, shot, n_bins, alias_range, w.axes,
+                        w.nu, w.acc) != cudaSuccess)
+      return fail(nullptr, PM_ECUDA, std::string(who) + ": launching the binning failed");
     ret = pk_read(w, who, n_bins, st, k.data(), p.data(), c.data());
     if (ret != PM_OK) return ret;
     std::vector<double> nn = nu;

@@ -208,10 +208,13 @@ void launch_record(cudaStream_t st, const float4* pos, float4* mom, long long N,
 // k_pk.cu
 void launch_pk_delta(cudaStream_t st, const unsigned long long* rho, float* delta, int n,
                      double inv_mean);
-void launch_pk_bin(cudaStream_t st, const float2* dk, int n, double box, double shot,
-                   int n_bins, double* acc);
-void launch_pk_jing(cudaStream_t st, const float2* dk, int n, double box, double shot,
-                    int n_bins, int m, const double* nu, double* acc);
+// the modes binned into acc (m = 0: first order; m > 0: alias range, slopes
+// nu), with the per-axis tables (pk_axes_bytes) that launch_pk_axes fills for
+// this m
+size_t pk_axes_bytes(int n);
+cudaError_t launch_pk_axes(cudaStream_t st, void* tab, int n, double box, int m);
+cudaError_t launch_pk_modes(cudaStream_t st, const float2* dk, int n, double box, double shot,
+                            int n_bins, int m, const void* tab, const double* nu, double* acc);
 
 }  // namespace pm
 
