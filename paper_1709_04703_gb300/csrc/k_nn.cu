@@ -7,8 +7,6 @@
 //                    K = 27 * input channels (im2col gathered into shared
 //                    memory), FP32 accumulation, bias + optional ReLU,
 //                    BF16 and/or FP32 output
-//   * k_conv_wgrad   weight gradient dW = sum_v in(v + tap) dY(v): M = 27 * Cin
-//                    rows, N = Cout, K = voxels split across blocks
 //   * elementwise    ReLU backward, 2x average pooling / nearest upsampling
 //                    (and their backward), channel concatenation, MSE, Adam
 // The input-gradient of a convolution is the forward convolution of the
@@ -277,111 +275,6 @@ __global__ void __launch_bounds__(128) k_conv_fwd(const bf16* __restrict__ in, V
   tc_end<NC>(c);
 }
 
-// Weight gradient, dw[co][tap*cin+ci] += sum_v in[v+tap][ci] dy[v][co]:
-// rows m = tap*cin + ci (128 per block), N >= cout, K = voxels, each block
-// folding `chunks` chunks of 64 voxels starting at its split.
-template <int N>
-__global__ void __launch_bounds__(128) k_conv_wgrad(const bf16* __restrict__ in, Vol g, int cin,
-                                                    const bf16* __restrict__ dy, int cout,
-                                                    float* __restrict__ dw, int chunks,
-                                                    int* err) {
-  constexpr int KC = 64;
-  __shared__ __align__(1024) uint8_t sA[tc::TM * KC * 2];
-  __shared__ __align__(1024) uint8_t sB[N * KC * 2];
-  __shared__ uint32_t tslot;
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ int vz[KC], vy[KC], vx[KC];
-  __shared__ long long vs[KC];
-  constexpr int NC = tc::tmem_cols(N);
-  TcCtx c = tc_begin<NC>(&tslot, &mbar);
-  const long long nvox = g.voxels();
-  const int m = blockIdx.x * tc::TM + threadIdx.x;  // this thread's row
-  const int rows = 27 * cin;
-  const int tap = m / cin, ci = m - (m / cin) * cin;
-  const int dz = tap / 9 - 1, dyy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-  const int coutp = (cout + 7) & ~7;
-  const long long k0 = (long long)blockIdx.y * chunks * KC;
-  uint32_t phase = 0;
-  auto fa = [&](int kt, uint8_t* s) {
-    // voxel coordinates of this chunk
-    if (threadIdx.x < KC) {
-      long long v = k0 + (long long)kt * KC + threadIdx.x;
-      long long t = v < nvox ? v : 0;
-      vx[threadIdx.x] = (int)(t % g.W); t /= g.W;
-      vy[threadIdx.x] = (int)(t % g.H); t /= g.H;
-      vz[threadIdx.x] = (int)(t % g.D);
-      vs[threadIdx.x] = v < nvox ? t / g.D : -1;
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int vv = 0; vv < KC / 8; ++vv) {
-      __align__(16) bf16 e[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        int kk = 8 * vv + q;
-        bf16 val = __float2bfloat16_rn(0.0f);
-        if (m < rows && vs[kk] >= 0) {
-          int zz = vz[kk] + dz, yy = vy[kk] + dyy, xx = vx[kk] + dx;
-          if (g.per) {
-            zz = zz < 0 ? zz + g.D : (zz >= g.D ? zz - g.D : zz);
-            yy = yy < 0 ? yy + g.H : (yy >= g.H ? yy - g.H : yy);
-            xx = xx < 0 ? xx + g.W : (xx >= g.W ? xx - g.W : xx);
-          }
-          if (zz >= 0 && zz < g.D && yy >= 0 && yy < g.H && xx >= 0 && xx < g.W)
-            val = in[(((vs[kk] * g.D + zz) * g.H + yy) * (long long)g.W + xx) * cin + ci];
-        }
-        e[q] = val;
-      }
-      *reinterpret_cast<uint4*>(s + tc::tile_offset(threadIdx.x, 8 * vv, KC)) =
-          *reinterpret_cast<const uint4*>(e);
-    }
-  };
-  auto fb = [&](int kt, uint8_t* s) {
-    for (int r = threadIdx.x; r < N; r += blockDim.x) {
-#pragma unroll 1
-      for (int vv = 0; vv < KC / 8; ++vv) {
-        __align__(16) bf16 e[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          long long v = k0 + (long long)kt * KC + 8 * vv + q;
-          e[q] = (r < cout && v < nvox) ? dy[v * coutp + r] : __float2bfloat16_rn(0.0f);
-        }
-        *reinterpret_cast<uint4*>(s + tc::tile_offset(r, 8 * vv, KC)) =
-            *reinterpret_cast<const uint4*>(e);
-      }
-    }
-  };
-  long long left = nvox - k0;
-  int kt_n = (int)((left + KC - 1) / KC);
-  if (kt_n > chunks) kt_n = chunks;
-  bool ok = kt_n > 0 ? tc_mainloop<N, KC>(fa, fb, kt_n, c.taddr, sA, sB, c.mbar, phase, err)
-                     : false;
-  if (ok) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * tc::TM + 32 * w + lane;
-#pragma unroll
-    for (int col = 0; col < N; col += 8) {
-      float val[8];
-      tc::tmem_ld8(c.taddr, w, col, val);
-      if (row < rows)
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (col + q < cout) atomicAdd(&dw[(long long)(col + q) * rows + row], val[q]);
-    }
-  }
-  tc_end<NC>(c);
-}
-
-#define PM_CONV_DISPATCH(KERNEL, N, ...)                                 \
-  switch (N) {                                                           \
-    case 16: KERNEL<16><<<__VA_ARGS__>>>; break;                         \
-    case 32: KERNEL<32><<<__VA_ARGS__>>>; break;                         \
-    case 48: KERNEL<48><<<__VA_ARGS__>>>; break;                         \
-    case 64: KERNEL<64><<<__VA_ARGS__>>>; break;                         \
-    case 96: KERNEL<96><<<__VA_ARGS__>>>; break;                         \
-    default: break;                                                      \
-  }
-
 void launch_conv_fwd(cudaStream_t st, const void* in, int B, int D, int H, int W, int per,
                      int cin, const void* wp, int n, int kp, const float* bias, int cout,
                      int relu, void* out_bf, float* out_f, int* err) {
@@ -393,31 +286,6 @@ void launch_conv_fwd(cudaStream_t st, const void* in, int B, int D, int H, int W
     case 48: k_conv_fwd<48><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)wp, kp, bias, cout, relu, (bf16*)out_bf, out_f, err); break;
     case 64: k_conv_fwd<64><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)wp, kp, bias, cout, relu, (bf16*)out_bf, out_f, err); break;
     case 96: k_conv_fwd<96><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)wp, kp, bias, cout, relu, (bf16*)out_bf, out_f, err); break;
-    default: return;
-  }
-  note_launch();
-}
-
-void launch_conv_wgrad(cudaStream_t st, const void* in, int B, int D, int H, int W, int per,
-                       int cin, const void* dy, int cout, int n, float* dw, int* err) {
-  Vol g{B, D, H, W, per};
-  const long long nvox = g.voxels();
-  const int rows = 27 * cin;
-  const int mt = (rows + tc::TM - 1) / tc::TM;
-  const long long kchunks = (nvox + 63) / 64;
-  // about 4 blocks per SM in total
-  long long splits = (608 + mt - 1) / mt;
-  if (splits > kchunks) splits = kchunks;
-  if (splits < 1) splits = 1;
-  const int chunks = (int)((kchunks + splits - 1) / splits);
-  splits = (kchunks + chunks - 1) / chunks;
-  dim3 grid((unsigned)mt, (unsigned)splits);
-  switch (n) {
-    case 16: k_conv_wgrad<16><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)dy, cout, dw, chunks, err); break;
-    case 32: k_conv_wgrad<32><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)dy, cout, dw, chunks, err); break;
-    case 48: k_conv_wgrad<48><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)dy, cout, dw, chunks, err); break;
-    case 64: k_conv_wgrad<64><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)dy, cout, dw, chunks, err); break;
-    case 96: k_conv_wgrad<96><<<grid, 128, 0, st>>>((const bf16*)in, g, cin, (const bf16*)dy, cout, dw, chunks, err); break;
     default: return;
   }
   note_launch();
@@ -687,21 +555,6 @@ __global__ void k_lap_grad(const float* __restrict__ q, Vol g, bf16* __restrict_
   }
 }
 
-// bias gradient: db[c] += sum_v dy[v][c] for c < cout (dy has coutp channels)
-__global__ void k_bias_grad(const bf16* __restrict__ dy, long long nvox, int cout, int coutp,
-                            float* __restrict__ db) {
-  __shared__ float sacc[64];
-  for (int c = threadIdx.x; c < 64; c += blockDim.x) sacc[c] = 0.0f;
-  __syncthreads();
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nvox * coutp;
-       t += (long long)gridDim.x * blockDim.x) {
-    int c = (int)(t % coutp);
-    if (c < cout) atomicAdd(&sacc[c], __bfloat162float(dy[t]));
-  }
-  __syncthreads();
-  for (int c = threadIdx.x; c < cout; c += blockDim.x) atomicAdd(&db[c], sacc[c]);
-}
-
 // Adam on FP32 master parameters
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, long long n, float lr, float b1, float b2, float eps,
@@ -793,11 +646,6 @@ void launch_resid_loss(cudaStream_t st, const float* y, const float* target, int
   k_lap_grad<<<ew_grid(n), 256, 0, st>>>(q, g, (bf16*)dy);
   note_launch();
   note_launch();
-  note_launch();
-}
-void launch_bias_grad(cudaStream_t st, const void* dy, long long nvox, int cout, int coutp,
-                      float* db) {
-  k_bias_grad<<<ew_grid(nvox * coutp), 256, 0, st>>>((const bf16*)dy, nvox, cout, coutp, db);
   note_launch();
 }
 void launch_adam(cudaStream_t st, float* w, const float* g, float* m, float* v, long long n,

@@ -454,11 +454,13 @@ namespace pm {
 void launch_wait_selftest(cudaStream_t st, int arrive, long long limit, int* gave_up);
 void launch_gemm_tc(cudaStream_t st, const void* A, const void* B, float* C, int M, int N,
                     int K, int* err);
+// k_wgrad.cu: weight and bias gradient of a convolution, accumulated into dw
+// [cout][27 cin] and db [cout]
+cudaError_t launch_wgrad(cudaStream_t st, const void* in, int B, int S, int per, int cin,
+                         const void* dy, int cout, float* dw, float* db);
 void launch_conv_fwd(cudaStream_t st, const void* in, int B, int D, int H, int W, int per,
                      int cin, const void* wp, int n, int kp, const float* bias, int cout,
                      int relu, void* out_bf, float* out_f, int* err);
-void launch_conv_wgrad(cudaStream_t st, const void* in, int B, int D, int H, int W, int per,
-                       int cin, const void* dy, int cout, int n, float* dw, int* err);
 void launch_resid_loss(cudaStream_t st, const float* y, const float* target, int B, int S,
                        int per, const float* tscale, float* d, float* q, void* dy, double* loss);
 void launch_pack_w(cudaStream_t st, const float* w, int cin, int cout, void* wp, int n, int kp,
@@ -477,8 +479,6 @@ void launch_nn_input(cudaStream_t st, const float* f, long long vps, const float
                      void* x);
 void launch_mse(cudaStream_t st, const float* y, const float* target, long long vps,
                 const float* tscale, int B, void* dy, double* loss);
-void launch_bias_grad(cudaStream_t st, const void* dy, long long nvox, int cout, int coutp,
-                      float* db);
 void launch_adam(cudaStream_t st, float* w, const float* g, float* m, float* v, long long n,
                  float lr, float b1, float b2, float eps, float c1, float c2);
 void launch_nn_output(cudaStream_t st, const float* y, long long vps, const float* scale, int B,
