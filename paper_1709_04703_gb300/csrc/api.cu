@@ -1795,11 +1795,18 @@ pm_status pm_potential(pm_ctx* ctx, const double* delta_dev, double a, int32_t b
   launch_source_f64(ctx->st, SRC_GRID, delta_dev, n, fh, fl, S, !per, ctx->partial,
                     ctx->counter, ctx->d_scal);
   // launch_source_f64 writes (||f||^2, q0, d, S_ab) to d_scal[0..10]
+  // both buffers from zero (the whole mesh with its ghost layer, in whole
+  // arrays), then the boundary values into both
   for (int q = 0; q < 2; ++q) {
-    Grid gh = full_view(ctx, ctx->phi_h[q], 0, n), gl = full_view(ctx, ctx->phi_l[q], 0, n);
-    if (!per) launch_boundary(ctx->st, gh, gl, n, 0, ctx->d_scal + 1, S, pair);
-    launch_fill(ctx->st, gh, 0.0f, false);
-    launch_fill(ctx->st, gl, 0.0f, false);
+    const size_t padded = sizeof(float) * (size_t)ctx->P * ctx->P * ctx->P;
+    CK(cudaMemsetAsync(ctx->phi_h[q], 0, padded, ctx->st));
+    CK(cudaMemsetAsync(ctx->phi_l[q], 0, padded, ctx->st));
+  }
+  if (!per) {
+    const Grid h2 = full_view(ctx, ctx->phi_h[1], 0, n), l2 = full_view(ctx, ctx->phi_l[1], 0, n);
+    launch_boundary(ctx->st, full_view(ctx, ctx->phi_h[0], 0, n),
+                    full_view(ctx, ctx->phi_l[0], 0, n), n, 0, ctx->d_scal + 1, S, pair, &h2,
+                    &l2);
   }
   CKL();
   const bool m64 = ctx->cfg.precision == PM_MIXED_FP64;

@@ -696,29 +696,51 @@ void launch_fill(cudaStream_t st, Grid g, float v, bool with_ghost) {
   note_launch();
 }
 
-// Potential output of pm_potential: phi32 = hi, phi64 = hi + lo (optional),
-// periodic results shifted by -mean (mean given as hi+lo sums).
-__global__ void k_phi_out(Grid ph, Grid pl, float* out32, double* out64, double shift) {
+// Potential output of pm_potential: phi64 = hi + lo - mean (optional), phi32
+// its FP32 rounding; without a mean (open) that is hi, the pair being
+// normalised.  A thread walks ZU planes; the conversions stay off the FP64
+// pipe (five FP64 operations per cell took 67 us at 192^3).
+__global__ void __launch_bounds__(256) k_phi_out(Grid ph, Grid pl, float* out32, double* out64,
+                                                 double shift) {
+  constexpr int ZU = 4;
   const int s = ph.s;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  int k = blockIdx.z;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= s || j >= s) return;
-  int c = gidx(ph, i, j, k);
-  double v = (double)ph.base[c] + (double)pl.base[c] - shift;
-  long long o = ((long long)k * s + j) * s + i;
-  out32[o] = (float)v;
-  if (out64) out64[o] = v;
+  float h[ZU], l[ZU];
+#pragma unroll
+  for (int u = 0; u < ZU; ++u) {
+    const int k = blockIdx.z * ZU + u, c = gidx(ph, i, j, k);
+    h[u] = k < s ? ph.base[c] : 0.0f;
+    l[u] = k < s ? pl.base[c] : 0.0f;
+  }
+#pragma unroll
+  for (int u = 0; u < ZU; ++u) {
+    const int k = blockIdx.z * ZU + u;
+    if (k >= s) break;
+    const long long o = ((long long)k * s + j) * s + i;
+    double v = double_of(h[u]) + double_of(l[u]);
+    if (shift != 0.0) {
+      v -= shift;
+      out32[o] = (float)v;
+    } else {
+      out32[o] = h[u];
+    }
+    if (out64) out64[o] = v;
+  }
 }
 
 void launch_phi_out(cudaStream_t st, Grid ph, Grid pl, float* out32, double* out64,
                     double shift) {
-  k_phi_out<<<grid_full(ph.s), dim3(32, 8), 0, st>>>(ph, pl, out32, out64, shift);
+  dim3 g = grid_full(ph.s);
+  g.z = (g.z + 3) / 4;
+  k_phi_out<<<g, dim3(32, 8), 0, st>>>(ph, pl, out32, out64, shift);
   note_launch();
 }
 
 // Sum of hi + lo over the interior (for the periodic zero-mean gauge); FP64
-// per thread, not on the step's hot path.
+// per thread, not on the step's hot path.  The last block folds the blocks'
+// sums, all its threads together.
 __global__ void k_sum_phi(Grid ph, Grid pl, double* __restrict__ partial,
                           unsigned int* counter, double* __restrict__ out) {
   const int s = ph.s;
@@ -727,10 +749,11 @@ __global__ void k_sum_phi(Grid ph, Grid pl, double* __restrict__ partial,
   double v = 0.0;
   for (int k = blockIdx.z; k < s && i < s && j < s; k += gridDim.z) {
     int c = gidx(ph, i, j, k);
-    v += (double)ph.base[c] + (double)pl.base[c];
+    v += double_of(ph.base[c]) + double_of(pl.base[c]);
   }
   __shared__ double sm[32];
-  int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int nth = blockDim.x * blockDim.y, nw = nth / 32;
   v = warp_sum(v);
   if ((tid & 31) == 0) sm[tid >> 5] = v;
   __syncthreads();
@@ -739,15 +762,21 @@ __global__ void k_sum_phi(Grid ph, Grid pl, double* __restrict__ partial,
   __shared__ bool last;
   if (tid == 0) {
     double tb = 0.0;
-    for (int w = 0; w < (int)(blockDim.x * blockDim.y) / 32; ++w) tb += sm[w];
+    for (int w = 0; w < nw; ++w) tb += sm[w];
     partial[bid] = tb;
     __threadfence();
     last = (atomicAdd(counter, 1u) == nblk - 1);
   }
   __syncthreads();
-  if (!last || tid != 0) return;
+  if (!last) return;
   double tt = 0.0;
-  for (unsigned q = 0; q < nblk; ++q) tt += __ldcg(partial + q);
+  for (unsigned q = tid; q < nblk; q += nth) tt += __ldcg(partial + q);
+  tt = warp_sum(tt);
+  if ((tid & 31) == 0) sm[tid >> 5] = tt;
+  __syncthreads();
+  if (tid != 0) return;
+  tt = 0.0;
+  for (int w = 0; w < nw; ++w) tt += sm[w];
   *out = tt;
   *counter = 0u;
 }

@@ -226,6 +226,32 @@ __device__ __forceinline__ df df_from_u64(unsigned long long v) {
   return fast_two_sum(t.hi, __fadd_rn(s.lo, t.lo));
 }
 
+// FP64 <-> FP32 without the FP64 pipe's conversions (its rate here is 1/64 of
+// FP32's, so at one conversion per cell they cost what 30 FP32 operations do).
+// x -> the double-float pair (RN(x), RN(x - hi)): the 53-bit significand in
+// three exact digits (21 + 16 + 16 bits), summed error-free.  Values outside
+// [2^-70, 2^90] take the conversions.
+__device__ __forceinline__ df df_from_double(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ffu) - 1023;
+  if (e < -70 || e > 90) {
+    const float hi = (float)x;
+    return df{hi, (float)(x - (double)hi)};
+  }
+  const float sc = __uint_as_float((unsigned)(e - 20 + 127) << 23 | (h & 0x80000000u));
+  const float a = __fmul_rn((float)((h & 0xfffffu) | 0x100000u), sc);
+  const float b = __fmul_rn((float)(l >> 16), __fmul_rn(sc, 1.52587890625e-05f));        // 2^-16
+  const float c = __fmul_rn((float)(l & 0xffffu), __fmul_rn(sc, 2.3283064365386963e-10f));  // 2^-32
+  const df s = fast_two_sum(a, b);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, c));
+}
+// the double of a float, exactly
+__device__ __forceinline__ double double_of(float v) {
+  const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+  if (m < 0x00800000u || m >= 0x7f800000u) return m ? (double)v : __hiloint2double((int)u, 0);
+  return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
 __device__ __forceinline__ float warp_sumf_all(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
