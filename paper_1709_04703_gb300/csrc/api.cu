@@ -9,7 +9,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -1213,6 +1215,78 @@ pm_status record_to(pm_ctx* ctx, double R, double a_cross) {
   return PM_OK;
 }
 
+// Work space of the calls without a context (particle order, spectra): stream
+// ordered allocations from one memory pool per device that the library owns.
+// cudaMalloc and cudaFree cost 40 us each here, 0.3 to 0.6 ms a call.  The
+// pool keeps at most KEEP bytes between calls and gives them back when an
+// allocation of the library fails; allocations follow the stream they are
+// made on, so any threads and streams may use it at once.
+struct WorkPool {
+  static constexpr unsigned long long KEEP = 1ull << 30;
+  std::mutex mu;
+  std::vector<std::pair<int, cudaMemPool_t>> pools;
+  cudaMemPool_t pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    for (auto& p : pools)
+      if (p.first == dev) return p.second;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    unsigned long long keep = KEEP;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return nullptr;
+    }
+    pools.push_back({dev, p});
+    return p;
+  }
+  // give the idle memory of this device's pool back; false if there is none
+  bool trim() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lk(mu);
+    for (auto& p : pools)
+      if (p.first == dev) return cudaMemPoolTrimTo(p.second, 0) == cudaSuccess;
+    return false;
+  }
+};
+WorkPool& work_pool() {
+  static WorkPool* w = new WorkPool();  // (not destroyed: the driver may be gone by then)
+  return *w;
+}
+// one call's allocations, freed on its stream when it ends
+struct WorkSpace {
+  cudaStream_t st;
+  std::vector<void*> ptrs;
+  explicit WorkSpace(cudaStream_t s) : st(s) {}
+  WorkSpace(const WorkSpace&) = delete;
+  ~WorkSpace() {
+    for (void* p : ptrs) cudaFreeAsync(p, st);
+  }
+  bool get(void** out, size_t bytes) {
+    cudaMemPool_t pool = work_pool().pool();
+    if (!pool) return false;
+    cudaError_t e = cudaMallocFromPoolAsync(out, bytes ? bytes : 1, pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      cudaStreamSynchronize(st);
+      if (work_pool().trim()) e = cudaMallocFromPoolAsync(out, bytes ? bytes : 1, pool, st);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      *out = nullptr;
+      return false;
+    }
+    ptrs.push_back(*out);
+    return true;
+  }
+};
+
 pm_status alloc(pm_ctx* ctx, void** p, size_t bytes) {
   // host-side fault injection for tests: PM_FAULT_ALLOC=k makes the k-th
   // device allocation of a context fail as if the device were full
@@ -1222,6 +1296,10 @@ pm_status alloc(pm_ctx* ctx, void** p, size_t bytes) {
     return fail(ctx, PM_ENOMEM, "cudaMalloc: allocation failure injected (PM_FAULT_ALLOC)");
   }
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && work_pool().trim()) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     *p = nullptr;
     return fail(ctx, PM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
@@ -1908,47 +1986,93 @@ pm_status pm_sort_particles(const float* pos4_dev, const float* mom4_dev, int64_
                           sizeof(unsigned) * (size_t)n, sizeof(unsigned) * (size_t)n,
                           sizeof(unsigned) * sort_counts_len(n),
                           sizeof(unsigned) * sort_ghist_len()};
-  auto release = [&]() {
-    for (void** b : bufs)
-      if (*b) cudaFree(*b);
-  };
-  for (int q = 0; q < 6; ++q) {
-    if (cudaMalloc(bufs[q], sizes[q]) != cudaSuccess) {
-      cudaGetLastError();
-      release();
-      return fail(ctx, PM_ENOMEM, "pm_sort_particles: cudaMalloc failed");
-    }
-  }
+  WorkSpace ws(st);
+  for (int q = 0; q < 6; ++q)
+    if (!ws.get(bufs[q], sizes[q]))
+      return fail(ctx, PM_ENOMEM, "pm_sort_particles: allocating work space failed");
   cudaError_t e = launch_sort_particles(st, (const float4*)pos4_dev, (const float4*)mom4_dev, n,
                                         n_mesh, w, (float4*)pos4_out, (float4*)mom4_out);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  release();
   if (e != cudaSuccess)
     return fail(ctx, PM_ECUDA, std::string("pm_sort_particles: ") + cudaGetErrorString(e));
   return PM_OK;
 }
 
 namespace {
+// FFT plans of the spectra, kept between calls: making one takes about as
+// long as a 256^3 transform and its binning.  A plan belongs to one call at a
+// time (take / put under a lock, any thread, any device); at most MAX idle
+// ones stay, the oldest is destroyed.  Plans hold no work area (the call's
+// work space gives it).
+struct PlanCache {
+  static constexpr size_t MAX = 4;
+  struct Plan {
+    int dev = 0, n = 0;
+    cufftHandle h = 0;
+    size_t work = 0;
+    bool ok = false;
+  };
+  std::mutex mu;
+  std::vector<Plan> idle;
+  Plan take(int n) {
+    Plan p;
+    if (cudaGetDevice(&p.dev) != cudaSuccess) return p;
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      for (size_t q = 0; q < idle.size(); ++q)
+        if (idle[q].dev == p.dev && idle[q].n == n) {
+          p = idle[q];
+          idle.erase(idle.begin() + q);
+          return p;
+        }
+    }
+    p.n = n;
+    if (cufftCreate(&p.h) != CUFFT_SUCCESS) return p;
+    if (cufftSetAutoAllocation(p.h, 0) != CUFFT_SUCCESS ||
+        cufftMakePlan3d(p.h, n, n, n, CUFFT_R2C, &p.work) != CUFFT_SUCCESS) {
+      cufftDestroy(p.h);
+      return p;
+    }
+    p.ok = true;
+    return p;
+  }
+  void put(const Plan& p) {
+    Plan old;
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      idle.push_back(p);
+      if (idle.size() > MAX) {
+        old = idle.front();
+        idle.erase(idle.begin());
+      }
+    }
+    if (old.ok) cufftDestroy(old.h);
+  }
+};
+PlanCache& plan_cache() {
+  static PlanCache* c = new PlanCache();  // (not destroyed: the driver may be gone by then)
+  return *c;
+}
+
 // Device work space of one P(k) call: CIC counts, contrast, its R2C
 // transform, bin accumulators (3 per bin + the escape counter), slopes and
 // the window's per-axis tables.
 struct PkWork {
+  WorkSpace ws;
   unsigned long long* rho = nullptr;
   float* delta = nullptr;
   cufftComplex* dk = nullptr;
   double* acc = nullptr;
   double* nu = nullptr;
   void* axes = nullptr;
-  cufftHandle plan = 0;
-  bool have_plan = false;
+  void* fft = nullptr;
+  PlanCache::Plan plan;
+  bool done = false;  // the call's work on the stream has completed
+  explicit PkWork(cudaStream_t st) : ws(st) {}
   ~PkWork() {
-    if (have_plan) cufftDestroy(plan);
-    cudaFree(rho);
-    cudaFree(delta);
-    cudaFree(dk);
-    cudaFree(acc);
-    cudaFree(nu);
-    cudaFree(axes);
+    if (!plan.ok) return;
+    if (done) plan_cache().put(plan);
+    else cufftDestroy(plan.h);
   }
 };
 
@@ -1958,13 +2082,18 @@ pm_status pk_transform(PkWork& w, const char* who, const float* pos4_dev, int64_
                        int n_mesh, int n_bins, cudaStream_t st) {
   const size_t cells = (size_t)n_mesh * n_mesh * n_mesh;
   const size_t modes = (size_t)n_mesh * n_mesh * (n_mesh / 2 + 1);
-  if (cudaMalloc((void**)&w.rho, sizeof(unsigned long long) * cells) != cudaSuccess ||
-      cudaMalloc((void**)&w.delta, sizeof(float) * cells) != cudaSuccess ||
-      cudaMalloc((void**)&w.dk, sizeof(cufftComplex) * modes) != cudaSuccess ||
-      cudaMalloc((void**)&w.acc, sizeof(double) * (3 * n_bins + 1)) != cudaSuccess ||
-      cudaMalloc((void**)&w.nu, sizeof(double) * n_bins) != cudaSuccess ||
-      cudaMalloc(&w.axes, pk_axes_bytes(n_mesh)) != cudaSuccess)
-    return fail(nullptr, PM_ENOMEM, std::string(who) + ": cudaMalloc failed");
+  if (!w.ws.get((void**)&w.rho, sizeof(unsigned long long) * cells) ||
+      !w.ws.get((void**)&w.delta, sizeof(float) * cells) ||
+      !w.ws.get((void**)&w.dk, sizeof(cufftComplex) * modes) ||
+      !w.ws.get((void**)&w.acc, sizeof(double) * (3 * n_bins + 1)) ||
+      !w.ws.get((void**)&w.nu, sizeof(double) * n_bins) ||
+      !w.ws.get(&w.axes, pk_axes_bytes(n_mesh)))
+    return fail(nullptr, PM_ENOMEM, std::string(who) + ": allocating work space failed");
+  w.plan = plan_cache().take(n_mesh);
+  if (!w.plan.ok)
+    return fail(nullptr, PM_ECUDA, std::string(who) + ": making the FFT plan failed");
+  if (w.plan.work && !w.ws.get(&w.fft, w.plan.work))
+    return fail(nullptr, PM_ENOMEM, std::string(who) + ": allocating work space failed");
   cudaMemsetAsync(w.rho, 0, sizeof(unsigned long long) * cells, st);
   cudaMemsetAsync(w.acc, 0, sizeof(double) * (3 * n_bins + 1), st);
   // positions are read-only here: no drift
@@ -1973,11 +2102,9 @@ pm_status pk_transform(PkWork& w, const char* who, const float* pos4_dev, int64_
                        (unsigned long long*)(w.acc + 3 * n_bins));
   const double mean = (double)n * 281474976710656.0 / (double)cells;
   launch_pk_delta(st, w.rho, w.delta, n_mesh, 1.0 / mean);
-  if (cufftPlan3d(&w.plan, n_mesh, n_mesh, n_mesh, CUFFT_R2C) != CUFFT_SUCCESS)
-    return fail(nullptr, PM_ECUDA, std::string(who) + ": cufftPlan3d failed");
-  w.have_plan = true;
-  cufftSetStream(w.plan, st);
-  if (cufftExecR2C(w.plan, w.delta, w.dk) != CUFFT_SUCCESS)
+  if (cufftSetStream(w.plan.h, st) != CUFFT_SUCCESS ||
+      (w.plan.work && cufftSetWorkArea(w.plan.h, w.fft) != CUFFT_SUCCESS) ||
+      cufftExecR2C(w.plan.h, w.delta, w.dk) != CUFFT_SUCCESS)
     return fail(nullptr, PM_ECUDA, std::string(who) + ": cufftExecR2C failed");
   return PM_OK;
 }
@@ -1991,6 +2118,7 @@ pm_status pk_read(PkWork& w, const char* who, int n_bins, cudaStream_t st, doubl
       cudaStreamSynchronize(st) != cudaSuccess)
     return fail(nullptr, PM_ECUDA,
                 std::string(who) + ": " + cudaGetErrorString(cudaGetLastError()));
+  w.done = true;  // the transform has run (what follows only reads its output)
   for (int b = 0; b < n_bins; ++b) {
     double c = h[3 * b];
     modes_out[b] = c;
@@ -2025,7 +2153,7 @@ pm_status pm_power_spectrum(const float* pos4_dev, int64_t n, double box, int32_
       !k_out || !pk_out || !modes_out)
     return fail(nullptr, PM_EINVAL, "pm_power_spectrum: bad argument");
   cudaStream_t st = (cudaStream_t)stream;
-  PkWork w;
+  PkWork w(st);
   pm_status ret = pk_transform(w, "pm_power_spectrum", pos4_dev, n, n_mesh, n_bins, st);
   if (ret != PM_OK) return ret;
   const double shot = subtract_shot ? box * box * box / (double)n : 0.0;
@@ -2047,7 +2175,7 @@ pm_status pm_power_spectrum_jing(const float* pos4_dev, int64_t n, double box, i
     return fail(nullptr, PM_EINVAL, "pm_power_spectrum_jing: bad argument");
   const char* who = "pm_power_spectrum_jing";
   cudaStream_t st = (cudaStream_t)stream;
-  PkWork w;
+  PkWork w(st);
   pm_status ret = pk_transform(w, who, pos4_dev, n, n_mesh, n_bins, st);
   if (ret != PM_OK) return ret;
   const double shot = subtract_shot ? box * box * box / (double)n : 0.0;
