@@ -37,6 +37,8 @@ constexpr int SRC_GRID = 1216;            // 152 SMs x 8 blocks
 constexpr int COARSE_SWEEPS = 6;
 constexpr int FUSED_MIN = 192;  // smallest level side smoothed by the fused pass
 constexpr int LEVEL_SWEEPS = 2;  // pre- and post-smoothing sweeps on levels below the finest
+constexpr int VC_SAME = 3;  // equal solves before a V-cycle is queued ahead (solve)
+constexpr size_t SCAL_BYTES = 16 * sizeof(double) + 4 * sizeof(unsigned long long);
 constexpr size_t BGW_OFF = 128;  // byte offset of the background weights in bgm
 
 // ---------------------------------------------------------------------------
@@ -169,7 +171,8 @@ struct pm_ctx {
   double* partial = nullptr;    // per-block FP64 partial sums
   void* partial_m = nullptr;    // per-block int128 moments
   unsigned int* counter = nullptr;
-  double* d_scal = nullptr;     // [0] ||f||^2, [1..10] moments, [11] ||r||^2, [12] sum phi
+  double* d_scal = nullptr;     // [0] ||f||^2, [1..10] moments, [11] ||r||^2 ([13] of the
+                                // start, [14] of a V-cycle queued ahead), [12] sum phi
   double* bgm = nullptr;        // background moments (10), then at BGW_OFF the weights
   df* bgw = nullptr;            // per-axis mean-density weights w_g, g in [0, n)
   float* ballw = nullptr;       // spherical keep region: mean-density image, n^3
@@ -247,6 +250,7 @@ struct pm_ctx {
 
   int vcycles_last = 0;
   int vc_prev = 0;          // V-cycles of the previous solve
+  int vc_same = 0;          // solves in a row, up to the previous one, that took vc_prev
   long long vcycles_total = 0;
   double resid_last = 0.0;
   double resid_start = 0.0, resid_guess = 0.0;  // of the last solve
@@ -495,6 +499,9 @@ pm_status set_cube(pm_ctx* ctx, int lo, int s, int periodic, double R) {
   if (same && ctx->ecorr && (ctx->mbase != mbase0 || ctx->mr != mr0))
     CK(cudaMemsetAsync(ctx->ecorr, 0, sizeof(float) * (size_t)(s + 2) * (s + 2) * (s + 2),
                        ctx->st));
+  // (periodic: the weights are ones and the moments the box's, as uploaded
+  // when this cube was set)
+  if (same && periodic) return PM_OK;
   // mean-density term of delta: per axis the image of the keep interval
   // [c - R, c + R] under the assignment kernel (CIC tent or TSC),
   // w_g = T(c + R - x_g) - T(c - R - x_g) at x_g = g + 1/2 with T the
@@ -607,10 +614,8 @@ void prof_end(pm_ctx* ctx, int cls, int e0, double bytes) {
 }
 
 pm_status sync_read(pm_ctx* ctx) {
-  CK(cudaMemcpyAsync(ctx->h_scal, ctx->d_scal, sizeof(double) * 16, cudaMemcpyDeviceToHost,
-                     ctx->st));
-  CK(cudaMemcpyAsync(ctx->h_cnt, ctx->d_cnt, sizeof(unsigned long long) * 4,
-                     cudaMemcpyDeviceToHost, ctx->st));
+  // d_cnt and h_cnt follow d_scal and h_scal in one block each
+  CK(cudaMemcpyAsync(ctx->h_scal, ctx->d_scal, SCAL_BYTES, cudaMemcpyDeviceToHost, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));
   if (ctx->prof_on) prof_flush(ctx);
   return PM_OK;
@@ -1102,6 +1107,26 @@ pm_status solve(pm_ctx* ctx) {
       }
       continue;
     }
+    // The last solves (VC_SAME of them) having taken the same number of
+    // V-cycles, this one is expected to take it too: where that is one more than have run, the
+    // V-cycle and its defect are queued before the residuals are read, both
+    // in one read (a host round trip leaves the GPU idle for 15 to 20 us).
+    // They write the correction, r and the other potential buffer, none of
+    // which is used if the solve turns out to have converged before: the same
+    // V-cycles, the same bits.
+    const bool ahead = mixed && !net_todo && !capture && ctx->vc_same >= VC_SAME &&
+                       it + 1 == ctx->vc_prev && it < ctx->cfg.max_vcycles;
+    if (ahead) {
+      pm_status v = vcycle_run(ctx, e0, r0, true);
+      if (v != PM_OK) return v;
+      const int c1 = ctx->cur;
+      e = prof_begin(ctx);
+      launch_defect(ctx->st, ph_of(c1), pl_of(c1), &e0, ph_of(c1 ^ 1), pl_of(c1 ^ 1), fh, fl,
+                    r0, per, true, ctx->partial, ctx->counter, ctx->d_scal + 14,
+                    6.0 + ctx->sig_d);
+      prof_end(ctx, PM_PROF_DEFECT, e, 32.0 * cells);
+      CKL();
+    }
     pm_status st = sync_read(ctx);
     if (st != PM_OK) return st;
     double f2 = ctx->h_scal[0], r2 = ctx->h_scal[slot];
@@ -1114,6 +1139,12 @@ pm_status solve(pm_ctx* ctx) {
       ctx->resid_guess = rel;  // after the network's correction
     }
     if (rel <= ctx->cfg.rtol || f2 == 0.0) break;
+    if (ahead) {  // take the V-cycle that has run
+      ++it;
+      ctx->cur ^= 1;
+      rel = std::sqrt(ctx->h_scal[14] / f2);
+      if (rel <= ctx->cfg.rtol) break;
+    }
     if (it >= ctx->cfg.max_vcycles) {
       ctx->vcycles_last = it;
       ctx->vcycles_total += it;
@@ -1156,6 +1187,7 @@ pm_status solve(pm_ctx* ctx) {
   ctx->vcycles_last = it;
   ctx->vcycles_total += it;
   ctx->resid_last = rel;
+  ctx->vc_same = it == ctx->vc_prev ? ctx->vc_same + 1 : 1;
   ctx->vc_prev = it;
   return PM_OK;
 }
@@ -1503,7 +1535,7 @@ pm_status pm_init(const pm_config* cfg, const float* pos4, const float* mom4,
   AL(ctx->partial, sizeof(double) * 16 * maxblk);
   AL(ctx->partial_m, 16 * 10 * (size_t)maxblk);
   AL(ctx->counter, sizeof(unsigned int) * 4);
-  AL(ctx->d_scal, sizeof(double) * 16);
+  AL(ctx->d_scal, SCAL_BYTES);
   AL(ctx->bgm, BGW_OFF + sizeof(df) * (size_t)n);
   ctx->bgw = (df*)((char*)ctx->bgm + BGW_OFF);
   if (cfg->domain != PM_DOMAIN_CUBE) {
@@ -1519,15 +1551,16 @@ pm_status pm_init(const pm_config* cfg, const float* pos4, const float* mom4,
     AL(ctx->sortw.ghist, sizeof(unsigned) * sort_ghist_len());
   }
   ctx->h_bg.assign(BGW_OFF + sizeof(df) * (size_t)n, 0);
-  AL(ctx->d_cnt, sizeof(unsigned long long) * 4);
+  ctx->d_cnt = (unsigned long long*)(ctx->d_scal + 16);
   ctx->d_overflow = (int*)(ctx->d_cnt + 3);  // read back with every sync_read
 #undef AL
-  if (cudaMallocHost((void**)&ctx->h_scal, sizeof(double) * 16) != cudaSuccess ||
-      cudaMallocHost((void**)&ctx->h_cnt, sizeof(unsigned long long) * 4) != cudaSuccess) {
+  if (cudaMallocHost((void**)&ctx->h_scal, SCAL_BYTES) != cudaSuccess) {
     g_err = "pm_init: cudaMallocHost failed";
     pm_destroy(ctx);
     return PM_ENOMEM;
   }
+  std::memset(ctx->h_scal, 0, SCAL_BYTES);
+  ctx->h_cnt = (unsigned long long*)(ctx->h_scal + 16);
   cudaStream_t s0 = ctx->st;
 #define Z(ptr, bytes)                                                        \
   if (cudaMemsetAsync((ptr), 0, (bytes), s0) != cudaSuccess) {               \
@@ -1545,8 +1578,7 @@ pm_status pm_init(const pm_config* cfg, const float* pos4, const float* mom4,
   if (ctx->prev64) Z(ctx->prev64, sizeof(double) * padded);
   if (ctx->ecorr) Z(ctx->ecorr, sizeof(float) * padded);
   Z(ctx->counter, sizeof(unsigned int) * 4);
-  Z(ctx->d_scal, sizeof(double) * 16);
-  Z(ctx->d_cnt, sizeof(unsigned long long) * 4);
+  Z(ctx->d_scal, SCAL_BYTES);
 #undef Z
   if (tune_fused(ctx) != cudaSuccess) {
     g_err = "pm_init: timing the fused smoother failed";
@@ -2524,6 +2556,7 @@ pm_status pm_load(pm_ctx* ctx, const char* path) {
   ctx->n_sol = h.n_sol;
   ctx->field_ready = h.field_ready != 0;
   ctx->vc_prev = h.vc_prev;
+  ctx->vc_same = 0;
   ctx->vcycles_last = h.vcycles_last;
   ctx->n_active = h.n_active;
   ctx->n_lc = h.n_lc;
@@ -2607,7 +2640,7 @@ void pm_destroy(pm_ctx* ctx) {
                   ctx->phi_h[0], ctx->phi_l[0], ctx->phi_h[1], ctx->phi_l[1], ctx->f_hi,
                   ctx->f_lo, ctx->prev_hi, ctx->prev_lo,
                   ctx->partial, ctx->partial_m,
-                  ctx->counter, ctx->d_scal, ctx->bgm, ctx->d_cnt, ctx->ballw,
+                  ctx->counter, ctx->d_scal, ctx->bgm, ctx->ballw,
                   ctx->nn_in, ctx->nn_out, ctx->grad, ctx->sortw.keys[0], ctx->sortw.keys[1],
                   ctx->sortw.vals[0], ctx->sortw.vals[1], ctx->sortw.counts, ctx->sortw.ghist};
   for (void* p : ptrs)
@@ -2624,7 +2657,6 @@ void pm_destroy(pm_ctx* ctx) {
   drop_graph(ctx);
   for (auto& e : ctx->ev) cudaEventDestroy(e);
   if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
-  if (ctx->h_cnt) cudaFreeHost(ctx->h_cnt);
   delete ctx;
 }
 

@@ -213,10 +213,13 @@ __device__ __forceinline__ void cl_vcycle(float* sm, const Grid& gu, const Grid&
     S = q ? C0 : S0;
     n = cl_threads(S);
     id = 1 + q;
-    const int H = S >> 1, seg = t / (S * H), r = t - seg * (S * H);
+    // lanes along x, then along z (two planes each): the shared rows of a
+    // warp then fall on different banks (16^3: 2 planes are 360 words, 8
+    // banks apart; along y the rows of 10 words would overlap)
+    const int H = S >> 1, r = t / H, seg = r % H;
     on = t < S * S * S / 4;
+    xp = t - r * H;
     j = r / H;
-    xp = r - j * H;
     k0 = 2 * seg;
     odd = j & 1;
     M = H + 2;
