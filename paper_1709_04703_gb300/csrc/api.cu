@@ -2676,6 +2676,19 @@ struct BTab {
   BTable* h_tab = nullptr;
   size_t desc_size = 0;
   int grid_max = 0;  // largest block total seen (graph launches use it)
+  bool uploaded = false;
+};
+
+// What a step of the batch reads back, in one block: one copy.
+struct BatchResult {
+  double scal[16 * MAX_REAL];  // 16 per realisation: [0] ||f||^2, [1..10] moments, [11] ||r||^2
+  double rel[MAX_REAL];        // last relative residual
+  double tol[MAX_REAL];        // relative tolerances (fixed for the run)
+  unsigned long long cnt[4 * MAX_REAL];  // 4 per realisation: [0] survivors
+  int iters[MAX_REAL];                   // V-cycles of the solve
+  int failed[MAX_REAL];                  // 1: not converged
+  int ovf[MAX_REAL];                     // 1: a cell's deposit overflowed
+  GridBar bar;                           // the persistent solve's barrier
 };
 
 }  // namespace
@@ -2685,12 +2698,9 @@ struct pm_batch {
   cudaStream_t st = nullptr;
   std::vector<pm_ctx*> ctx;
   int* d_active = nullptr;  // the graph solve's per-realisation activity
-  double* d_scal = nullptr;  // 16 per realisation: [0] ||f||^2, [1..10] moments, [11] ||r||^2
-  double* h_scal = nullptr;
-  unsigned long long* d_cnt = nullptr;  // 4 per realisation: [0] survivors
-  unsigned long long* h_cnt = nullptr;
-  int* d_ovf = nullptr;
-  BTab t_dep, t_src, t_bnd, t_pred, t_def, t_grad, t_gat, t_scan, t_scat;
+  BatchResult* d_res = nullptr;
+  BatchResult* h_res = nullptr;
+  BTab t_def, t_grad;
   std::vector<BTab> t_vc;  // V-cycle launch slots of the persistent solve
   std::vector<BTab> t_leg; // the graph solve's fused legs: 2 l + (0 down, 1 up)
   int maxLc = 0;
@@ -2705,12 +2715,6 @@ struct pm_batch {
   bool persistent = false;
   double wait_s = 2.0;         // longest wait at one grid barrier
   int extra = 0;               // barrier arrivals that never come (tests the wait limit)
-  GridBar* d_bar = nullptr;
-  GridBar* h_bar = nullptr;
-  int* d_iters = nullptr;      // [0, MAX_REAL): V-cycles, [MAX_REAL, 2 MAX_REAL): failed
-  int* h_iters = nullptr;
-  double* d_rel = nullptr;     // [0, MAX_REAL): last relative residual, then rtol
-  double* h_rel = nullptr;
   int* d_maxv = nullptr;
   SolveSlot* d_slots = nullptr;
   int n_slots_dev = 0;
@@ -2752,7 +2756,18 @@ void tab_free(BTab& t) {
 template <class D>
 int tab_upload(pm_batch* B, BTab& t, const std::vector<D>& d, const std::vector<int>& blocks) {
   const int m = std::min((int)d.size(), MAX_MEMBERS);  // callers add <= 2 per realisation
-  std::memcpy(t.h_desc, d.data(), sizeof(D) * m);
+  {
+    int tot = 0;
+    bool same = t.uploaded && m == t.h_tab->m &&
+                (m == 0 || std::memcmp(t.h_desc, d.data(), sizeof(D) * m) == 0);
+    for (int q = 0; q < m && same; ++q) same = t.h_tab->off[q + 1] == (tot += blocks[q]);
+    if (same) {  // the device has these members already
+      t.grid_max = std::max(t.grid_max, tot);
+      return tot;
+    }
+  }
+  t.uploaded = true;
+  if (m) std::memcpy(t.h_desc, d.data(), sizeof(D) * m);
   t.h_tab->m = m;
   t.h_tab->off[0] = 0;
   for (int q = 0; q < m; ++q) t.h_tab->off[q + 1] = t.h_tab->off[q] + blocks[q];
@@ -2761,6 +2776,18 @@ int tab_upload(pm_batch* B, BTab& t, const std::vector<D>& d, const std::vector<
   int tot = t.h_tab->off[m];
   if (tot > t.grid_max) t.grid_max = tot;
   return tot;
+}
+
+// The members of a launch as its argument; returns the block total.
+template <class D>
+int pack_args(BArgs<D>& a, const std::vector<D>& d, const std::vector<int>& blocks) {
+  a.m = (int)d.size();  // at most one entry per realisation
+  a.off[0] = 0;
+  for (int q = 0; q < a.m; ++q) {
+    a.off[q + 1] = a.off[q] + blocks[q];
+    a.d[q] = d[q];
+  }
+  return a.off[a.m];
 }
 
 int nblocks(dim3 g) { return (int)(g.x * g.y * g.z); }
@@ -3012,13 +3039,13 @@ pm_status build_solve_graph(pm_batch* B) {
   auto decide = [&](cudaStream_t st) {
     launch_defect_b(st, B->t_def.grid_max, (const DefectDesc*)B->t_def.d_desc, B->t_def.d_tab,
                     B->d_active);
-    launch_converged_b(st, R, B->d_scal, B->d_rel + MAX_REAL, B->d_maxv, B->d_active,
-                       B->d_iters, B->d_iters + MAX_REAL, B->d_rel, loop);
+    launch_converged_b(st, R, B->d_res->scal, B->d_res->tol, B->d_maxv, B->d_active,
+                       B->d_res->iters, B->d_res->failed, B->d_res->rel, loop);
   };
   cudaGraphNode_t wnode = nullptr;
   long long lb0 = 0, lb1 = 0;
   if (e == cudaSuccess) {
-    launch_solve_init_b(B->st, R, B->d_active, B->d_iters, B->d_iters + MAX_REAL);
+    launch_solve_init_b(B->st, R, B->d_active, B->d_res->iters, B->d_res->failed);
     decide(B->st);
     const cudaGraphNode_t* deps = nullptr;
     size_t nd = 0;
@@ -3112,10 +3139,9 @@ void upload_grad_table(pm_batch* B, const int* flip) {
     e.s = c->s;
     e.periodic = c->periodic;
     e.G = c->grad;
-    set_dims(e, r, dim3((unsigned)((c->s + 31) / 32), (unsigned)((c->s + 7) / 8), (unsigned)c->s));
+    set_dims(e, r, full_grid_b(c->s));
     d.push_back(e);
-    bl.push_back(nblocks(dim3((unsigned)((c->s + 31) / 32), (unsigned)((c->s + 7) / 8),
-                              (unsigned)c->s)));
+    bl.push_back(nblocks(full_grid_b(c->s)));
   }
   tab_upload(B, B->t_grad, d, bl);
 }
@@ -3143,7 +3169,7 @@ void upload_defect_table(pm_batch* B, const int* iters) {
     e.write_r = 1;
     e.partial = c->partial;
     e.counter = c->counter;
-    e.out = B->d_scal + 16 * r + 11;
+    e.out = B->d_res->scal + 16 * r + 11;
     e.iters = iters;
     set_dims(e, r, defect_grid(s));
     d.push_back(e);
@@ -3167,8 +3193,8 @@ pm_status batch_solve_persistent(pm_batch* B) {
   }
   upload_defect_table(B, nullptr);
   upload_grad_table(B, nullptr);
-  cudaMemsetAsync(B->d_bar, 0, sizeof(GridBar), B->st);
-  cudaMemsetAsync(B->d_iters + MAX_REAL, 0, sizeof(int) * R, B->st);
+  cudaMemsetAsync(&B->d_res->bar, 0, sizeof(GridBar), B->st);
+  cudaMemsetAsync(B->d_res->failed, 0, sizeof(int) * R, B->st);
   SolveArgs a{};
   a.grad = (const GradDesc*)B->t_grad.d_desc;
   a.grad_t = B->t_grad.d_tab;
@@ -3177,13 +3203,13 @@ pm_status batch_solve_persistent(pm_batch* B) {
   a.slots = B->d_slots;
   a.n_slots = B->n_slots_dev;
   a.R = R;
-  a.scal = B->d_scal;
-  a.rtol = B->d_rel + MAX_REAL;
+  a.scal = B->d_res->scal;
+  a.rtol = B->d_res->tol;
   a.maxv = B->d_maxv;
-  a.iters = B->d_iters;
-  a.failed = B->d_iters + MAX_REAL;
-  a.rel = B->d_rel;
-  a.bar = B->d_bar;
+  a.iters = B->d_res->iters;
+  a.failed = B->d_res->failed;
+  a.rel = B->d_res->rel;
+  a.bar = &B->d_res->bar;
   a.limit_ns = (unsigned long long)(B->wait_s * 1e9);
   a.extra = B->extra;
   a.fast_coarse = cmg_fast();
@@ -3202,8 +3228,8 @@ pm_status batch_solve_graph(pm_batch* B) {
     upload_leg_tables(B);
   }
   B->tables_stale = false;
-  upload_defect_table(B, B->d_iters);
-  upload_grad_table(B, B->d_iters);
+  upload_defect_table(B, B->d_res->iters);
+  upload_grad_table(B, B->d_res->iters);
   if (!B->sgraph) {
     pm_status st = build_solve_graph(B);
     if (st != PM_OK) return st;
@@ -3215,16 +3241,7 @@ pm_status batch_solve_graph(pm_batch* B) {
 }
 
 pm_status batch_sync(pm_batch* B) {
-  if (B->solved_on_device) {
-    cudaMemcpyAsync(B->h_iters, B->d_iters, sizeof(int) * 2 * MAX_REAL, cudaMemcpyDeviceToHost,
-                    B->st);
-    cudaMemcpyAsync(B->h_rel, B->d_rel, sizeof(double) * B->R, cudaMemcpyDeviceToHost, B->st);
-    cudaMemcpyAsync(B->h_bar, B->d_bar, sizeof(GridBar), cudaMemcpyDeviceToHost, B->st);
-  }
-  cudaMemcpyAsync(B->h_scal, B->d_scal, sizeof(double) * 16 * B->R, cudaMemcpyDeviceToHost,
-                  B->st);
-  cudaMemcpyAsync(B->h_cnt, B->d_cnt, sizeof(unsigned long long) * 4 * B->R,
-                  cudaMemcpyDeviceToHost, B->st);
+  cudaMemcpyAsync(B->h_res, B->d_res, sizeof(BatchResult), cudaMemcpyDeviceToHost, B->st);
   cudaError_t e = cudaStreamSynchronize(B->st);
   if (e != cudaSuccess) return bfail(B, PM_ECUDA, cudaGetErrorString(e));
   e = cudaGetLastError();
@@ -3237,35 +3254,35 @@ pm_status batch_sync(pm_batch* B) {
 pm_status batch_solve_done(pm_batch* B) {
   if (!B->solved_on_device) return PM_OK;
   B->solved_on_device = false;
-  if (B->h_bar->err) {
+  if (B->h_res->bar.err) {
     char buf[200];
     snprintf(buf, sizeof buf,
              "pm_batch_step: a grid barrier of the persistent solve waited longer than %.3g s "
              "(pass %d); the batch must be destroyed",
-             B->wait_s, B->h_bar->where);
+             B->wait_s, B->h_res->bar.where);
     return bfail(B, PM_ETIMEOUT, buf);
   }
   if (!B->persistent) {
     // the graph's kernels: init, defect, decision, gradient, and the loop's
     // body once per V-cycle of the realisation that took the most
     int most = 0;
-    for (int r = 0; r < B->R; ++r) most = std::max(most, B->h_iters[r]);
+    for (int r = 0; r < B->R; ++r) most = std::max(most, B->h_res->iters[r]);
     g_launches.fetch_add(4 + (long long)most * B->loop_kernels);
   }
   for (int r = 0; r < B->R; ++r) {
     pm_ctx* c = B->ctx[r];
-    const int it = B->h_iters[r];
-    if (B->h_iters[MAX_REAL + r]) {
+    const int it = B->h_res->iters[r];
+    if (B->h_res->failed[r]) {
       char buf[200];
       snprintf(buf, sizeof buf,
                "realisation %d: relative residual %.3e after %d V-cycles (rtol %.1e)", r,
-               B->h_rel[r], it, c->cfg.rtol);
+               B->h_res->rel[r], it, c->cfg.rtol);
       return bfail(B, PM_ENOCONV, buf);
     }
     c->cur ^= it & 1;
     c->vcycles_last = it;
     c->vcycles_total += it;
-    c->resid_last = B->h_rel[r];
+    c->resid_last = B->h_res->rel[r];
   }
   return PM_OK;
 }
@@ -3322,53 +3339,34 @@ pm_status pm_batch_init(int32_t n_real, const pm_config* cfgs, const float* cons
   }
   pm_status st = PM_OK;
   if (cudaMalloc((void**)&B->d_active, sizeof(int) * MAX_REAL) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_scal, sizeof(double) * 16 * MAX_REAL) != cudaSuccess ||
-      cudaMallocHost((void**)&B->h_scal, sizeof(double) * 16 * MAX_REAL) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_cnt, sizeof(unsigned long long) * 4 * MAX_REAL) != cudaSuccess ||
-      cudaMallocHost((void**)&B->h_cnt, sizeof(unsigned long long) * 4 * MAX_REAL) !=
-          cudaSuccess ||
-      cudaMalloc((void**)&B->d_ovf, sizeof(int) * MAX_REAL) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_bar, sizeof(GridBar)) != cudaSuccess ||
-      cudaMallocHost((void**)&B->h_bar, sizeof(GridBar)) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_iters, sizeof(int) * 2 * MAX_REAL) != cudaSuccess ||
-      cudaMallocHost((void**)&B->h_iters, sizeof(int) * 2 * MAX_REAL) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_rel, sizeof(double) * 2 * MAX_REAL) != cudaSuccess ||
-      cudaMallocHost((void**)&B->h_rel, sizeof(double) * MAX_REAL) != cudaSuccess ||
+      cudaMalloc((void**)&B->d_res, sizeof(BatchResult)) != cudaSuccess ||
+      cudaMallocHost((void**)&B->h_res, sizeof(BatchResult)) != cudaSuccess ||
       cudaMalloc((void**)&B->d_maxv, sizeof(int) * MAX_REAL) != cudaSuccess)
     st = bfail(B, PM_ENOMEM, "pm_batch_init: allocation failed");
   if (st == PM_OK) {
-    // per-realisation tolerances of the persistent solve (fixed for the run)
+    // per-realisation tolerances (fixed for the run)
     double tol[MAX_REAL];
     int mv[MAX_REAL];
     for (int r = 0; r < n_real; ++r) {
       tol[r] = cfgs[r].rtol;
       mv[r] = cfgs[r].max_vcycles;
     }
-    if (cudaMemcpy(B->d_rel + MAX_REAL, tol, sizeof(double) * n_real, cudaMemcpyHostToDevice) !=
-            cudaSuccess ||
+    // (zeroed first: the graph solve reads the barrier's state back as well)
+    if (cudaMemsetAsync(B->d_res, 0, sizeof(BatchResult), B->st) != cudaSuccess ||
+        cudaMemcpyAsync(B->d_res->tol, tol, sizeof(double) * n_real, cudaMemcpyHostToDevice,
+                        B->st) != cudaSuccess ||
         cudaMemcpy(B->d_maxv, mv, sizeof(int) * n_real, cudaMemcpyHostToDevice) != cudaSuccess)
       st = bfail(B, PM_ECUDA, "pm_batch_init: tolerance upload failed");
     // the graph solve by default (measured faster than the persistent
     // kernel, whose register budget is that of its heaviest phase)
     B->persistent = false;
   }
-  if (st == PM_OK) st = tab_alloc(B, B->t_dep, sizeof(DepositDesc));
-  if (st == PM_OK) st = tab_alloc(B, B->t_src, sizeof(SourceDesc));
-  if (st == PM_OK) st = tab_alloc(B, B->t_bnd, sizeof(BoundaryDesc));
-  if (st == PM_OK) st = tab_alloc(B, B->t_pred, sizeof(PredictDesc));
   if (st == PM_OK) st = tab_alloc(B, B->t_def, sizeof(DefectDesc));
   if (st == PM_OK) st = tab_alloc(B, B->t_grad, sizeof(GradDesc));
-  if (st == PM_OK) st = tab_alloc(B, B->t_gat, sizeof(GatherDesc));
-  if (st == PM_OK) st = tab_alloc(B, B->t_scan, sizeof(ScanDesc));
-  if (st == PM_OK) st = tab_alloc(B, B->t_scat, sizeof(ScatterDesc));
   if (st != PM_OK) {
     pm_batch_destroy(B);
     return st;
   }
-  cudaMemsetAsync(B->d_scal, 0, sizeof(double) * 16 * MAX_REAL, B->st);
-  cudaMemsetAsync(B->d_cnt, 0, sizeof(unsigned long long) * 4 * MAX_REAL, B->st);
-  cudaMemsetAsync(B->d_ovf, 0, sizeof(int) * MAX_REAL, B->st);
-  cudaMemsetAsync(B->d_iters, 0, sizeof(int) * 2 * MAX_REAL, B->st);
   *out = B;
   return PM_OK;
 }
@@ -3432,8 +3430,9 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         d.push_back(e);
         bl.push_back(nb);
       }
-      int g = tab_upload(B, B->t_dep, d, bl);
-      launch_deposit_b(B->st, g, (const DepositDesc*)B->t_dep.d_desc, B->t_dep.d_tab);
+      BArgs<DepositDesc> a;
+      const int g = pack_args(a, d, bl);
+      launch_deposit_b(B->st, g, a);
     }
     // 3. source (+ moments), boundary ghosts in both potential buffers, predict
     {
@@ -3461,16 +3460,17 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         e.partial_f2 = c->partial;
         e.partial_m = c->partial_m;
         e.counter = c->counter;
-        e.out = B->d_scal + 16 * r;
+        e.out = B->d_res->scal + 16 * r;
         e.bgm = c->bgm;
         e.invM_d = invM;
-        e.overflow = B->d_ovf + r;
+        e.overflow = B->d_res->ovf + r;
         set_dims(e, r, source_grid(s));
         d.push_back(e);
         bl.push_back(nblocks(source_grid(s)));
       }
-      int g = tab_upload(B, B->t_src, d, bl);
-      launch_source_b(B->st, g, (const SourceDesc*)B->t_src.d_desc, B->t_src.d_tab);
+      BArgs<SourceDesc> a;
+      const int g = pack_args(a, d, bl);
+      launch_source_b(B->st, g, a);
     }
     {
       std::vector<BoundaryDesc> d;
@@ -3478,23 +3478,24 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
       for (int r = 0; r < R; ++r) {
         pm_ctx* c = B->ctx[r];
         if (c->periodic) continue;
-        for (int qb = 0; qb < 2; ++qb) {
-          BoundaryDesc e{};
-          e.ph = full_view(c, c->phi_h[qb], c->lo, c->s);
-          e.pl = full_view(c, c->phi_l[qb], c->lo, c->s);
-          e.n = c->n;
-          e.lo = c->lo;
-          e.mom = B->d_scal + 16 * r + 1;
-          e.S = 1.5 * c->cfg.omega_m / c->a_half[k];
-          e.want_lo = 1;
-          int nb = boundary_blocks(c->s);
-          set_dims(e, r, dim3(nb, 1, 1));
-          d.push_back(e);
-          bl.push_back(nb);
-        }
+        BoundaryDesc e{};
+        e.ph = full_view(c, c->phi_h[0], c->lo, c->s);
+        e.pl = full_view(c, c->phi_l[0], c->lo, c->s);
+        e.ph2 = full_view(c, c->phi_h[1], c->lo, c->s);
+        e.pl2 = full_view(c, c->phi_l[1], c->lo, c->s);
+        e.n = c->n;
+        e.lo = c->lo;
+        e.mom = B->d_res->scal + 16 * r + 1;
+        e.S = 1.5 * c->cfg.omega_m / c->a_half[k];
+        e.want_lo = 1;
+        int nb = boundary_blocks(c->s);
+        set_dims(e, r, dim3(nb, 1, 1));
+        d.push_back(e);
+        bl.push_back(nb);
       }
-      int g = tab_upload(B, B->t_bnd, d, bl);
-      launch_boundary_b(B->st, g, (const BoundaryDesc*)B->t_bnd.d_desc, B->t_bnd.d_tab);
+      BArgs<BoundaryDesc> a;
+      const int g = pack_args(a, d, bl);
+      launch_boundary_b(B->st, g, a);
     }
     {
       std::vector<PredictDesc> d;
@@ -3520,8 +3521,9 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         d.push_back(e);
         bl.push_back(nblocks(full_grid_b(c->s)));
       }
-      int g = tab_upload(B, B->t_pred, d, bl);
-      launch_predict_b(B->st, g, (const PredictDesc*)B->t_pred.d_desc, B->t_pred.d_tab);
+      BArgs<PredictDesc> a;
+      const int g = pack_args(a, d, bl);
+      launch_predict_b(B->st, g, a);
     }
     // 4. solve every realisation to its rtol, decided on the device
     {
@@ -3573,8 +3575,9 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         flagged[r] = do_flag;
         any_flag |= do_flag;
       }
-      int g = tab_upload(B, B->t_gat, d, bl);
-      launch_gather_b(B->st, g, (const GatherDesc*)B->t_gat.d_desc, B->t_gat.d_tab);
+      BArgs<GatherDesc> a;
+      const int g = pack_args(a, d, bl);
+      launch_gather_b(B->st, g, a);
     }
     // 7. lightcone shrink of the flagged realisations
     if (any_flag) {
@@ -3589,7 +3592,7 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         e.cnt = c->block_keep;
         e.off = c->keep_off;
         e.nblk = nb;
-        e.n_keep = B->d_cnt + 4 * r;
+        e.n_keep = B->d_res->cnt + 4 * r;
         set_dims(e, r, dim3(1, 1, 1));
         ds.push_back(e);
         bs.push_back(1);
@@ -3609,10 +3612,12 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
         dc.push_back(f);
         bc.push_back(nb);
       }
-      int g = tab_upload(B, B->t_scan, ds, bs);
-      launch_scan_b(B->st, g, (const ScanDesc*)B->t_scan.d_desc, B->t_scan.d_tab);
-      g = tab_upload(B, B->t_scat, dc, bc);
-      launch_scatter_b(B->st, g, (const ScatterDesc*)B->t_scat.d_desc, B->t_scat.d_tab);
+      BArgs<ScanDesc> as;
+      int g = pack_args(as, ds, bs);
+      launch_scan_b(B->st, g, as);
+      BArgs<ScatterDesc> ac;
+      g = pack_args(ac, dc, bc);
+      launch_scatter_b(B->st, g, ac);
     }
     pm_status st = batch_sync(B);
     if (st != PM_OK) return st;
@@ -3622,7 +3627,7 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
       pm_ctx* c = B->ctx[r];
       c->particle_steps += c->n_active;
       if (flagged[r]) {
-        long long keep = (long long)B->h_cnt[4 * r];
+        long long keep = (long long)B->h_res->cnt[4 * r];
         std::swap(c->pos, c->pos2);
         std::swap(c->mom, c->mom2);
         c->n_lc += c->n_active - keep;
@@ -3630,11 +3635,8 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
       }
       c->step++;
     }
-    int ovf[MAX_REAL];
-    if (cudaMemcpy(ovf, B->d_ovf, sizeof(int) * R, cudaMemcpyDeviceToHost) != cudaSuccess)
-      return bfail(B, PM_ECUDA, "pm_batch_step: reading the overflow flags");
     for (int r = 0; r < R; ++r)
-      if (ovf[r]) return bfail(B, PM_EOVERFLOW, "deposit: a cell count exceeded 2^62");
+      if (B->h_res->ovf[r]) return bfail(B, PM_EOVERFLOW, "deposit: a cell count exceeded 2^62");
   }
   return PM_OK;
 }
@@ -3695,25 +3697,15 @@ void pm_batch_destroy(pm_batch* B) {
   if (B->sgraph) cudaGraphExecDestroy(B->sgraph);
   if (B->st2) cudaStreamDestroy(B->st2);
   for (pm_ctx* c : B->ctx) pm_destroy(c);
-  for (BTab* t : {&B->t_dep, &B->t_src, &B->t_bnd, &B->t_pred, &B->t_def, &B->t_grad,
-                  &B->t_gat, &B->t_scan, &B->t_scat})
-    tab_free(*t);
+  tab_free(B->t_def);
+  tab_free(B->t_grad);
   for (auto& t : B->t_vc) tab_free(t);
   for (auto& t : B->t_leg) tab_free(t);
   if (B->d_active) cudaFree(B->d_active);
-  if (B->d_bar) cudaFree(B->d_bar);
-  if (B->h_bar) cudaFreeHost(B->h_bar);
-  if (B->d_iters) cudaFree(B->d_iters);
-  if (B->h_iters) cudaFreeHost(B->h_iters);
-  if (B->d_rel) cudaFree(B->d_rel);
-  if (B->h_rel) cudaFreeHost(B->h_rel);
+  if (B->d_res) cudaFree(B->d_res);
+  if (B->h_res) cudaFreeHost(B->h_res);
   if (B->d_maxv) cudaFree(B->d_maxv);
   if (B->d_slots) cudaFree(B->d_slots);
-  if (B->d_scal) cudaFree(B->d_scal);
-  if (B->h_scal) cudaFreeHost(B->h_scal);
-  if (B->d_cnt) cudaFree(B->d_cnt);
-  if (B->h_cnt) cudaFreeHost(B->h_cnt);
-  if (B->d_ovf) cudaFree(B->d_ovf);
   delete B;
 }
 

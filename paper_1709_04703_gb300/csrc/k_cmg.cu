@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(CL_NT) kb_cmg_col(const CmgDesc* d, int n_desc
   if (q >= n_desc) return;
   const CmgDesc& e = d[q];
   if (active && !active[e.r]) return;
-  cmg_one(cc_sm, e.u, e.b, e.level, e.periodic, e.sweeps, e.zero_top, 0.0f);
+  cmg_one(cc_sm, in_global(e.u), in_global(e.b), e.level, e.periodic, e.sweeps, e.zero_top, 0.0f);
 }
 
 int g_cmg_cl = 1;  // CTAs per cluster of this process's launches (set by cmg_prepare)

@@ -1077,19 +1077,15 @@ cudaError_t launch_ade_sweep(cudaStream_t st, Grid ph, Grid pl, Grid fh, Grid fl
 // ---------------------------------------------------------------------------
 // Batched forms.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) kb_deposit(const DepositDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(256) kb_deposit(const __grid_constant__ BArgs<DepositDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const DepositDesc& e = d[q];
+  const DepositDesc& e = batch_arg(a, bi);
   d_drift_deposit<true>(bi, e.pos, e.mom, e.N, e.c0, e.n, e.lo, e.s, e.periodic, e.rho,
                         e.escaped);
 }
-__global__ void __launch_bounds__(256) kb_source(const SourceDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(256) kb_source(const __grid_constant__ BArgs<SourceDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const SourceDesc& e = d[q];
+  const SourceDesc& e = batch_arg(a, bi);
   if (e.moments)
     d_source<true>(bi, e.rho, e.n, e.lo, e.s, e.fh, e.fl, e.invM, e.S, e.bgw, nullptr,
                    e.partial_f2,
@@ -1099,27 +1095,25 @@ __global__ void __launch_bounds__(256) kb_source(const SourceDesc* d, const BTab
                     e.partial_f2, (__int128*)e.partial_m, e.counter, e.out, e.bgm, e.invM_d,
                     e.overflow);
 }
-__global__ void __launch_bounds__(256) kb_boundary(const BoundaryDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(256) kb_boundary(const __grid_constant__ BArgs<BoundaryDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const BoundaryDesc& e = d[q];
-  d_boundary(bi, e.ph, e.pl, e.n, e.lo, e.mom, e.S, e.want_lo, Grid{}, Grid{});
+  const BoundaryDesc& e = batch_arg(a, bi);
+  d_boundary(bi, e.ph, e.pl, e.n, e.lo, e.mom, e.S, e.want_lo, e.ph2, e.pl2);
 }
 
-void launch_deposit_b(cudaStream_t st, int grid, const DepositDesc* d, const BTable* t) {
+void launch_deposit_b(cudaStream_t st, int grid, const BArgs<DepositDesc>& a) {
   if (grid <= 0) return;
-  kb_deposit<<<grid, 256, 0, st>>>(d, t);
+  kb_deposit<<<grid, 256, 0, st>>>(a);
   note_launch();
 }
-void launch_source_b(cudaStream_t st, int grid, const SourceDesc* d, const BTable* t) {
+void launch_source_b(cudaStream_t st, int grid, const BArgs<SourceDesc>& a) {
   if (grid <= 0) return;
-  kb_source<<<grid, dim3(32, 8), 0, st>>>(d, t);
+  kb_source<<<grid, dim3(32, 8), 0, st>>>(a);
   note_launch();
 }
-void launch_boundary_b(cudaStream_t st, int grid, const BoundaryDesc* d, const BTable* t) {
+void launch_boundary_b(cudaStream_t st, int grid, const BArgs<BoundaryDesc>& a) {
   if (grid <= 0) return;
-  kb_boundary<<<grid, 256, 0, st>>>(d, t);
+  kb_boundary<<<grid, 256, 0, st>>>(a);
   note_launch();
 }
 int boundary_blocks(int s) { return (int)((6LL * (s + 2) * (s + 2) + 255) / 256); }

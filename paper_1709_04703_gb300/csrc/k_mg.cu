@@ -796,25 +796,20 @@ __global__ void __launch_bounds__(256, 4) kb_defect(const DefectDesc* d, const B
   BI bi;
   if (!batch_map(d, t, active, q, bi)) return;
   const DefectDesc& e = d[q];
-  if (e.iters) {
-    const int k = e.iters[e.r];
-    if (k == 0)
-      d_defect<false>(bi, e.ph, e.pl, e.e, e.ph, e.pl, e.fh, e.fl, e.rb, e.periodic, e.write_r,
-                      e.partial, e.counter, e.out, 6.0f, 0.0f);
-    else if (((k - 1) & 1) == 0)
-      d_defect<true>(bi, e.ph, e.pl, e.e, e.qh, e.ql, e.fh, e.fl, e.rb, e.periodic, e.write_r,
-                     e.partial, e.counter, e.out, 6.0f, 0.0f);
-    else
-      d_defect<true>(bi, e.qh, e.ql, e.e, e.ph, e.pl, e.fh, e.fl, e.rb, e.periodic, e.write_r,
-                     e.partial, e.counter, e.out, 6.0f, 0.0f);
-    return;
-  }
-  if (e.correct)
-    d_defect<true>(bi, e.ph, e.pl, e.e, e.qh, e.ql, e.fh, e.fl, e.rb, e.periodic, e.write_r,
-                   e.partial, e.counter, e.out, 6.0f, 0.0f);
+  // after V-cycle k >= 1 the correction moves the potential from the buffer
+  // of parity k - 1 into that of parity k
+  const int k = e.iters ? e.iters[e.r] : (e.correct ? 1 : 0);
+  const bool swap = k > 0 && ((k - 1) & 1);
+  const Grid ph = in_global(swap ? e.qh : e.ph), pl = in_global(swap ? e.ql : e.pl);
+  const Grid qh = in_global(swap ? e.ph : e.qh), ql = in_global(swap ? e.pl : e.ql);
+  const Grid ee = in_global(e.e), fh = in_global(e.fh), fl = in_global(e.fl);
+  const Grid rb = in_global(e.rb);
+  if (k == 0)
+    d_defect<false>(bi, ph, pl, ee, ph, pl, fh, fl, rb, e.periodic, e.write_r,
+                    in_global(e.partial), in_global(e.counter), in_global(e.out), 6.0f, 0.0f);
   else
-    d_defect<false>(bi, e.ph, e.pl, e.e, e.qh, e.ql, e.fh, e.fl, e.rb, e.periodic, e.write_r,
-                    e.partial, e.counter, e.out, 6.0f, 0.0f);
+    d_defect<true>(bi, ph, pl, ee, qh, ql, fh, fl, rb, e.periodic, e.write_r,
+                   in_global(e.partial), in_global(e.counter), in_global(e.out), 6.0f, 0.0f);
 }
 __global__ void kb_solve_init(int R, int* active, int* iters, int* failed) {
   const int r = (int)threadIdx.x;
@@ -857,11 +852,9 @@ void launch_converged_b(cudaStream_t st, int R, const double* scal, const double
   kb_converged<<<1, MAX_REAL, 0, st>>>(R, scal, rtol, maxv, active, iters, failed, rel, loop);
   note_launch();
 }
-__global__ void __launch_bounds__(256) kb_predict(const PredictDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(256) kb_predict(const __grid_constant__ BArgs<PredictDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const PredictDesc& e = d[q];
+  const PredictDesc& e = batch_arg(a, bi);
   each_plane(bi, e.ph.s, [&](const BI& b) { d_predict(b, e.ph, e.pl, e.qh, e.ql, e.w, e.pair); });
 }
 
@@ -871,9 +864,9 @@ void launch_defect_b(cudaStream_t st, int grid, const DefectDesc* d, const BTabl
   kb_defect<<<grid, dim3(32, 8), 0, st>>>(d, t, active);
   note_launch();
 }
-void launch_predict_b(cudaStream_t st, int grid, const PredictDesc* d, const BTable* t) {
+void launch_predict_b(cudaStream_t st, int grid, const BArgs<PredictDesc>& a) {
   if (grid <= 0) return;
-  kb_predict<<<grid, dim3(32, 8), 0, st>>>(d, t);
+  kb_predict<<<grid, dim3(32, 8), 0, st>>>(a);
   note_launch();
 }
 
@@ -1120,7 +1113,9 @@ __global__ void __launch_bounds__(SOLVE_NT, MINB) kb_solve(SolveArgs a) {
   // even number of V-cycles, in the other one after an odd number)
   each_block(a.grad, a.grad_t, (const int*)nullptr, s_off, [&](const GradDesc& e, const BI& bi) {
     const bool odd = (it[e.r] & 1) != 0;
-    d_grad(bi, odd ? e.ph_alt : e.ph, odd ? e.pl_alt : e.pl, e.n, e.lo, e.s, e.periodic, e.G);
+    each_plane(bi, e.s, [&](const BI& b) {
+      d_grad(b, odd ? e.ph_alt : e.ph, odd ? e.pl_alt : e.pl, e.n, e.lo, e.s, e.periodic, e.G);
+    });
   });
 }
 

@@ -661,30 +661,27 @@ __global__ void __launch_bounds__(256) kb_grad(const GradDesc* d, const BTable* 
   if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
   const GradDesc& e = d[q];
   const bool alt = e.flip && (e.flip[e.r] & 1);
-  d_grad(bi, alt ? e.ph_alt : e.ph, alt ? e.pl_alt : e.pl, e.n, e.lo, e.s, e.periodic, e.G);
+  const float *ph = in_global(alt ? e.ph_alt : e.ph), *pl = in_global(alt ? e.pl_alt : e.pl);
+  float4* G = in_global(e.G);
+  const int n = e.n, lo = e.lo, s = e.s, per = e.periodic;
+  each_plane(bi, s, [&](const BI& b) { d_grad(b, ph, pl, n, lo, s, per, G); });
 }
-__global__ void __launch_bounds__(KT) kb_gather(const GatherDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(KT) kb_gather(const __grid_constant__ BArgs<GatherDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const GatherDesc& e = d[q];
+  const GatherDesc& e = batch_arg(a, bi);
   d_gather_kick_drift<true>(bi, e.pos, e.mom, e.N, nullptr, nullptr, e.G, e.n, e.lo, e.s,
                              e.periodic, e.kick, e.c2, e.do_flag, e.klo, e.khi,
                              KeepBall{0, 0.0, 0.0}, e.flags,
                              e.block_keep, e.forces, e.escaped);
 }
-__global__ void __launch_bounds__(1024) kb_scan(const ScanDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(1024) kb_scan(const __grid_constant__ BArgs<ScanDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const ScanDesc& e = d[q];
+  const ScanDesc& e = batch_arg(a, bi);
   d_scan_blocks(bi, e.cnt, e.off, e.nblk, e.n_keep);
 }
-__global__ void __launch_bounds__(KT) kb_scatter(const ScatterDesc* d, const BTable* t) {
-  int q;
+__global__ void __launch_bounds__(KT) kb_scatter(const __grid_constant__ BArgs<ScatterDesc> a) {
   BI bi;
-  if (!batch_map(d, t, (const int*)nullptr, q, bi)) return;
-  const ScatterDesc& e = d[q];
+  const ScatterDesc& e = batch_arg(a, bi);
   d_scatter(bi, e.pos, e.mom, e.N, e.flags, e.keep_off, e.pos_out, e.mom_out, e.lc_pos,
             e.lc_mom, e.lc_base, e.a_cross);
 }
@@ -694,19 +691,19 @@ void launch_grad_b(cudaStream_t st, int grid, const GradDesc* d, const BTable* t
   kb_grad<<<grid, dim3(32, 8), 0, st>>>(d, t);
   note_launch();
 }
-void launch_gather_b(cudaStream_t st, int grid, const GatherDesc* d, const BTable* t) {
+void launch_gather_b(cudaStream_t st, int grid, const BArgs<GatherDesc>& a) {
   if (grid <= 0) return;
-  kb_gather<<<grid, KT, 0, st>>>(d, t);
+  kb_gather<<<grid, KT, 0, st>>>(a);
   note_launch();
 }
-void launch_scan_b(cudaStream_t st, int grid, const ScanDesc* d, const BTable* t) {
+void launch_scan_b(cudaStream_t st, int grid, const BArgs<ScanDesc>& a) {
   if (grid <= 0) return;
-  kb_scan<<<grid, 1024, 0, st>>>(d, t);
+  kb_scan<<<grid, 1024, 0, st>>>(a);
   note_launch();
 }
-void launch_scatter_b(cudaStream_t st, int grid, const ScatterDesc* d, const BTable* t) {
+void launch_scatter_b(cudaStream_t st, int grid, const BArgs<ScatterDesc>& a) {
   if (grid <= 0) return;
-  kb_scatter<<<grid, KT, 0, st>>>(d, t);
+  kb_scatter<<<grid, KT, 0, st>>>(a);
   note_launch();
 }
 

@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(T::NT, T::NT > 256 ? 2 : 4) kb_tile(const Tile
   int q;
   BI bi;
   if (!batch_map(d, tab, active, q, bi)) return;
-  const TileArgs a = d[q].a;  // (a batch solves Poisson's equation: d0 = 6)
+  TileArgs a = d[q].a;  // (a batch solves Poisson's equation: d0 = 6)
+  for (Grid* g : {&a.u, &a.b, &a.w, &a.uc, &a.bc}) *g = in_global(*g);
   if (a.periodic) tile_one<T, UP, true, true>(a, bi.x, bi.y, bi.z, sm);
   else if (a.gam == 0.0f) tile_open<T, UP, true>(a, bi.x, bi.y, bi.z, sm);
   else tile_open<T, UP, false>(a, bi.x, bi.y, bi.z, sm);

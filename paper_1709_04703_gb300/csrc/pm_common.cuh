@@ -328,7 +328,7 @@ struct BTable {
 };
 
 // Planes per block of the batched mesh passes (colour pass, restriction,
-// prolongation, warm-start prediction): a block's table lookup is shared by
+// prolongation, warm-start prediction, gradient field): a block's table lookup is shared by
 // BZ planes of its (x, y) tile.
 constexpr int BZ = 4;
 template <class F>
@@ -340,6 +340,46 @@ __device__ __forceinline__ void each_plane(const BI& bi, int nz, F&& f) {
     if (b.z >= nz) break;
     f(b);
   }
+}
+
+// The same table as a kernel argument, for the launches whose members are
+// known when they are made (all but the captured solve's): no upload before
+// the launch and no staging in the block, and the descriptor's fields come
+// from constant memory like any launch's arguments.  12 realisations, 7.1
+// million particles: gather 153 -> 112 us, deposit 152 -> 113, source 95 -> 63;
+// 65 uploads per five steps gone.
+template <class D>
+struct BArgs {
+  int m;
+  int off[MAX_REAL + 1];
+  D d[MAX_REAL];
+};
+template <class D>
+__device__ __forceinline__ const D& batch_arg(const BArgs<D>& a, BI& bi) {
+  static_assert(sizeof(BArgs<D>) <= 32764, "a kernel's arguments");
+  const int b = (int)blockIdx.x;
+  int lo = 0, hi = a.m - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.off[mid] <= b) lo = mid; else hi = mid - 1;
+  }
+  const D& e = a.d[lo];
+  const int lb = b - a.off[lo];
+  bi = BI{lb % e.gx, (lb / e.gx) % e.gy, lb / (e.gx * e.gy), e.gx, e.gy, e.gz};
+  return e;
+}
+// a pointer read from a descriptor in memory: it points to global memory,
+// which the compiler cannot see (it would use generic loads and stores: the
+// defect 85 us against 82, the gradient field 88 against 54 together with
+// the planes a block shares)
+template <class T>
+__device__ __forceinline__ T* in_global(T* p) {
+  __builtin_assume(__isGlobal((const void*)p));
+  return p;
+}
+__device__ __forceinline__ Grid in_global(Grid g) {
+  g.base = in_global(g.base);
+  return g;
 }
 
 // The block of a batched launch -> member q of the table and its block

@@ -314,7 +314,7 @@ struct SourceDesc {
   int r, gx, gy, gz;
 };
 struct BoundaryDesc {
-  Grid ph, pl;
+  Grid ph, pl, ph2, pl2;  // both potential buffers take the values
   int n, lo;
   const double* mom;
   double S;
@@ -425,14 +425,14 @@ int solve_grid_b();
 cudaError_t launch_solve_b(cudaStream_t st, const SolveArgs& a);
 void launch_defect_b(cudaStream_t st, int grid, const DefectDesc* d, const BTable* t,
                      const int* active);
-void launch_predict_b(cudaStream_t st, int grid, const PredictDesc* d, const BTable* t);
-void launch_deposit_b(cudaStream_t st, int grid, const DepositDesc* d, const BTable* t);
-void launch_source_b(cudaStream_t st, int grid, const SourceDesc* d, const BTable* t);
-void launch_boundary_b(cudaStream_t st, int grid, const BoundaryDesc* d, const BTable* t);
+void launch_predict_b(cudaStream_t st, int grid, const BArgs<PredictDesc>& a);
+void launch_deposit_b(cudaStream_t st, int grid, const BArgs<DepositDesc>& a);
+void launch_source_b(cudaStream_t st, int grid, const BArgs<SourceDesc>& a);
+void launch_boundary_b(cudaStream_t st, int grid, const BArgs<BoundaryDesc>& a);
 void launch_grad_b(cudaStream_t st, int grid, const GradDesc* d, const BTable* t);
-void launch_gather_b(cudaStream_t st, int grid, const GatherDesc* d, const BTable* t);
-void launch_scan_b(cudaStream_t st, int grid, const ScanDesc* d, const BTable* t);
-void launch_scatter_b(cudaStream_t st, int grid, const ScatterDesc* d, const BTable* t);
+void launch_gather_b(cudaStream_t st, int grid, const BArgs<GatherDesc>& a);
+void launch_scan_b(cudaStream_t st, int grid, const BArgs<ScanDesc>& a);
+void launch_scatter_b(cudaStream_t st, int grid, const BArgs<ScatterDesc>& a);
 
 // grid shapes of the single-realisation launches (blocks per dimension)
 dim3 rbgs_grid(int s);

@@ -106,6 +106,22 @@ def test_many_open_realisations():
     batch.close()
 
 
+@pytest.mark.parametrize("count", [1, 2, 64])
+def test_member_counts(count):
+    """One realisation, two, and the most a batch takes (the batched launches
+    carry their members as arguments, sized for 64), periodic and open, ragged
+    particle blocks: the same bits as separate contexts."""
+    from paper_1709_04703_gb300.sim import Batch
+    a0, a1, steps = 0.3, 1.0, 3
+    reals = [_realisation((16, 32, 24)[r % 3], 3000.0 + 2500.0 * (r % 4), 500 + r, a0)
+             for r in range(count)]
+    batch = Batch(reals, a0, a1, steps)
+    batch.step(steps)
+    for r in sorted({0, count // 2, count - 1}):
+        _compare(batch, r, _single(reals[r], a0, a1, steps, 1e-7))
+    batch.close()
+
+
 def test_fused_finest_level_matches_batched_passes():
     """At n = 192 a single context smooths its finest level with the fused
     two-sweep pass; the batched step uses one-colour passes: the same bits,
