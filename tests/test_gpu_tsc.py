@@ -45,6 +45,29 @@ def test_tsc_deposit_bitexact_periodic(n, N, seed):
     np.testing.assert_array_equal(rho.cpu().numpy(), ref)
 
 
+@pytest.mark.parametrize("n,N,periodic", [(16, 31, True), (16, 33, True), (4, 64, True),
+                                          (32, 32**3, True), (24, 40000, True),
+                                          (32, 32**3, False), (24, 40000, False)])
+def test_tsc_deposit_merged_lanes_bitexact(n, N, periodic):
+    """Particles in cell order along x, where neighbouring lanes merge their
+    rows: chains over the periodic edge, of one cell and of none, broken by a
+    row's end, by several particles in a cell and (open cube) by escapes."""
+    from paper_1709_04703_gb300.sim import deposit
+    rng = np.random.default_rng(N + n)
+    if N > n**3:  # several per cell, some cells empty
+        cell = np.sort(rng.integers(0, n**3, N))
+    else:
+        cell = (np.arange(N) + (n - 5)) % n**3
+    pos = np.stack([cell % n, cell // n % n, cell // n**2], 1) + rng.random((N, 3))
+    pos = np.minimum(pos.astype(np.float32), np.nextafter(np.float32(n), np.float32(0)))
+    lo, s = (0, n) if periodic else (3, n - 6)
+    p4, _ = _dev4(pos)
+    rho, esc = deposit(p4, n, lo, s, periodic=periodic, assignment="tsc")
+    ref, resc = opm.deposit_tsc(pos, n, lo, s, periodic)
+    assert esc == resc
+    np.testing.assert_array_equal(rho.cpu().numpy(), ref)
+
+
 @pytest.mark.parametrize("lo,s", [(4, 24), (10, 12)])
 def test_tsc_deposit_bitexact_open_cube_with_escapes(lo, s):
     from paper_1709_04703_gb300.sim import deposit
