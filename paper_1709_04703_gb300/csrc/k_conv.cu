@@ -1,4 +1,5 @@
-// The forward 3x3x3 "same" convolution of the learned guess as an implicit
+// The 3x3x3 "same" convolutions of the learned guess (forward, and the input
+// gradient with the taps reversed) as an implicit
 // GEMM on the 5th-generation tensor cores without an im2col copy.
 //
 // A CTA computes a T^3 block of output voxels of one sample.  It stages the
@@ -233,15 +234,22 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
   if (threadIdx.x < 32) tc::tmem_free(taddr, sh.ncols);
 }
 
-// wf[n][k] from the FP32 masters w[co][tap * cin + ci] (see the file head)
+// wf[n][k] from the FP32 masters w[co][tap * cin + ci] (see the file head).
+// bwd: the operand of the input gradient, a convolution of the output's
+// gradient (co channels in, ci out) with the taps reversed.
 __global__ void k_pack_wf(const float* __restrict__ w, int cin, int cout, int n, int kf,
-                          bf16* __restrict__ wf) {
-  const int cinp = cin == 8 ? 8 : (cin + 15) / 16 * 16;
+                          bool bwd, bf16* __restrict__ wf) {
+  const int c = bwd ? (cout + 7) / 8 * 8 : cin;  // channels of the convolved tensor
+  const int cinp = c == 8 ? 8 : (c + 15) / 16 * 16;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * kf; t += gridDim.x * blockDim.x) {
     const int r = t / kf, k = t - r * kf;
     const int tap = k / cinp, ci = k - tap * cinp;
     float v = 0.0f;
-    if (r < cout && tap < 27 && ci < cin) v = w[(long long)r * 27 * cin + tap * cin + ci];
+    if (!bwd) {
+      if (r < cout && tap < 27 && ci < cin) v = w[(long long)r * 27 * cin + tap * cin + ci];
+    } else if (r < cin && tap < 27 && ci < cout) {  // (row: input channel, ci: output channel)
+      v = w[(long long)ci * 27 * cin + (26 - tap) * cin + r];
+    }
     wf[t] = __float2bfloat16_rn(v);
   }
 }
@@ -274,9 +282,10 @@ int conv_fast_side(int cin, int cout) {
 
 int conv_fast_kf(int cin) { return cin == 8 ? 28 * 8 : 27 * ((cin + 15) / 16 * 16); }
 
-void launch_pack_wf(cudaStream_t st, const float* w, int cin, int cout, int n, void* wf) {
-  const int kf = conv_fast_kf(cin);
-  k_pack_wf<<<(n * kf + 255) / 256, 256, 0, st>>>(w, cin, cout, n, kf, (bf16*)wf);
+void launch_pack_wf(cudaStream_t st, const float* w, int cin, int cout, int n, bool bwd,
+                    void* wf) {
+  const int kf = conv_fast_kf(bwd ? (cout + 7) / 8 * 8 : cin);
+  k_pack_wf<<<(n * kf + 255) / 256, 256, 0, st>>>(w, cin, cout, n, kf, bwd, (bf16*)wf);
   note_launch();
 }
 

@@ -37,6 +37,8 @@ struct ConvL {
   void *wp = nullptr, *wt = nullptr;  // packed BF16 operands
   int fast_t = 0;          // output block side of the staged-input forward kernel (0: none)
   void* wf = nullptr;      // its packed weights
+  int fast_tt = 0;         // the same for the input gradient
+  void* wft = nullptr;
 };
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
@@ -69,7 +71,7 @@ struct pm_guess {
   double* rms_part = nullptr;  // block partial sums of the per-sample RMS
   double* loss = nullptr;
   int* err = nullptr;
-  bool packed = false;
+  bool packed = false, packed_t = false;
   std::string msg;
 };
 
@@ -134,9 +136,17 @@ pm_status ensure_shape(pm_guess* g, int B, int S) {
 void pack_all(pm_guess* g) {
   for (auto& c : g->conv) {
     launch_pack_w(g->st, g->w + c.w_off, c.cin, c.cout, c.wp, c.n, c.kp, c.wt, c.nt, c.kpt);
-    if (c.fast_t) launch_pack_wf(g->st, g->w + c.w_off, c.cin, c.cout, c.n, c.wf);
+    if (c.fast_t) launch_pack_wf(g->st, g->w + c.w_off, c.cin, c.cout, c.n, false, c.wf);
   }
   g->packed = true;
+  g->packed_t = false;
+}
+// the input gradients' operands: packed by the first backward pass after
+// pack_all (a forward-only user never pays for them)
+void pack_bwd(pm_guess* g) {
+  for (auto& c : g->conv)
+    if (c.fast_tt) launch_pack_wf(g->st, g->w + c.w_off, c.cin, c.cout, c.nt, true, c.wft);
+  g->packed_t = true;
 }
 
 // forward convolution of layer c on a B x s^3 input: the staged-input kernel
@@ -242,7 +252,8 @@ void conv_bwd(pm_guess* g, ConvL& c, const void* x, int B, int s, int per, const
               void* dx) {
   // (a failed launch is read with the others by GCK)
   launch_wgrad(g->st, x, B, s, per, c.cin, dy, c.cout, g->g + c.w_off, g->g + c.b_off);
-  if (dx)
+  if (dx && !(c.fast_tt && launch_conv_fast(g->st, dy, B, s, per, round_up(c.cout, 8), c.wft, c.nt,
+                                            c.fast_tt, nullptr, c.cin, 0, dx, nullptr, g->err)))
     launch_conv_fwd(g->st, dy, B, s, s, s, per, round_up(c.cout, 8), c.wt, c.nt, c.kpt,
                     nullptr /*no bias*/, c.cin, 0, dx, nullptr, g->err);
 }
@@ -252,6 +263,7 @@ void conv_bwd(pm_guess* g, ConvL& c, const void* x, int B, int s, int per, const
 pm_status backward(pm_guess* g, const float* phi, int B, int S, int per, int loss_kind) {
   const long long vps = (long long)S * S * S;
   const int L = g->L;
+  if (!g->packed_t) pack_bwd(g);
   cudaMemsetAsync(g->loss, 0, sizeof(double), g->st);
   cudaMemsetAsync(g->g, 0, sizeof(float) * g->n_params, g->st);
   void* G0 = g->act[SLOT_G0].p;
@@ -361,6 +373,12 @@ pm_status pm_guess_create(int32_t levels, void* stream, pm_guess** out) {
     c.fast_t = getenv("PM_NN_GATHER") ? 0 : conv_fast_side(c.cin, c.cout);
     if (c.fast_t)
       ok = ok && cudaMalloc(&c.wf, (size_t)c.n * conv_fast_kf(c.cin) * 2) == cudaSuccess;
+    // the input gradient likewise (the five of a 4-level net at 96^3 that
+    // fit: 490 us on the gathered tile, 286 staged)
+    const int co8 = round_up(c.cout, 8);
+    c.fast_tt = getenv("PM_NN_GATHER") ? 0 : conv_fast_side(co8, c.cin);
+    if (c.fast_tt)
+      ok = ok && cudaMalloc(&c.wft, (size_t)c.nt * conv_fast_kf(co8) * 2) == cudaSuccess;
   }
   size_t pb = sizeof(float) * g->n_params;
   ok = ok && cudaMalloc((void**)&g->w, pb) == cudaSuccess &&
@@ -464,6 +482,7 @@ void pm_guess_destroy(pm_guess* g) {
     if (c.wp) cudaFree(c.wp);
     if (c.wt) cudaFree(c.wt);
     if (c.wf) cudaFree(c.wf);
+    if (c.wft) cudaFree(c.wft);
   }
   for (auto& b : g->act)
     if (b.p) cudaFree(b.p);

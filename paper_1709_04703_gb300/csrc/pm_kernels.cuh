@@ -176,7 +176,8 @@ constexpr int PART_CHUNK = KT * KITEMS;
 // launch_conv_fast returns false if the kernel could not be configured.
 int conv_fast_side(int cin, int cout);
 int conv_fast_kf(int cin);
-void launch_pack_wf(cudaStream_t st, const float* w, int cin, int cout, int n, void* wf);
+void launch_pack_wf(cudaStream_t st, const float* w, int cin, int cout, int n, bool bwd,
+                    void* wf);
 bool launch_conv_fast(cudaStream_t st, const void* in, int B, int S, int per, int cin,
                       const void* wf, int n, int T, const float* bias, int cout, int relu,
                       void* out_bf, float* out_f, int* err);
