@@ -1113,9 +1113,8 @@ __global__ void __launch_bounds__(SOLVE_NT, MINB) kb_solve(SolveArgs a) {
   // even number of V-cycles, in the other one after an odd number)
   each_block(a.grad, a.grad_t, (const int*)nullptr, s_off, [&](const GradDesc& e, const BI& bi) {
     const bool odd = (it[e.r] & 1) != 0;
-    each_plane(bi, e.s, [&](const BI& b) {
-      d_grad(b, odd ? e.ph_alt : e.ph, odd ? e.pl_alt : e.pl, e.n, e.lo, e.s, e.periodic, e.G);
-    });
+    d_grad(bi, bi.z * BZ, min(bi.z * BZ + BZ, e.s), odd ? e.ph_alt : e.ph,
+           odd ? e.pl_alt : e.pl, e.n, e.lo, e.s, e.periodic, e.G);
   });
 }
 

@@ -240,10 +240,12 @@ __global__ void __launch_bounds__(KT) k_gather_kick_drift(
 // full (n+2)^3 layout of Phi.
 __global__ void __launch_bounds__(256) k_grad(const float* __restrict__ ph,
                                               const float* __restrict__ pl, int n, int lo,
-                                              int s, int periodic, float4* __restrict__ G) {
+                                              int s, int periodic, int run,
+                                              float4* __restrict__ G) {
   pdl_wait();
   pdl_release();
-  d_grad(bi_native(), ph, pl, n, lo, s, periodic, G);
+  const BI bi = bi_native();
+  d_grad(bi, bi.z * run, min(bi.z * run + run, s), ph, pl, n, lo, s, periodic, G);
 }
 
 // ---------------------------------------------------------------------------
@@ -400,8 +402,10 @@ void launch_gather_kick_drift(cudaStream_t st, float4* pos, float4* mom, long lo
 
 void launch_grad(cudaStream_t st, const float* ph, const float* pl, int n, int lo, int s,
                  int periodic, float4* G) {
-  dim3 grid((unsigned)((s + 31) / 32), (unsigned)((s + 7) / 8), (unsigned)s);
-  launch_pdl(k_grad, grid, dim3(32, 8), 0, st, ph, pl, n, lo, s, periodic, G);
+  // four planes per block while that leaves every SM a few blocks
+  const int run = s >= 96 ? 4 : 1;
+  dim3 grid((unsigned)((s + 31) / 32), (unsigned)((s + 7) / 8), (unsigned)((s + run - 1) / run));
+  launch_pdl(k_grad, grid, dim3(32, 8), 0, st, ph, pl, n, lo, s, periodic, run, G);
   note_launch();
 }
 
@@ -663,8 +667,8 @@ __global__ void __launch_bounds__(256) kb_grad(const GradDesc* d, const BTable* 
   const bool alt = e.flip && (e.flip[e.r] & 1);
   const float *ph = in_global(alt ? e.ph_alt : e.ph), *pl = in_global(alt ? e.pl_alt : e.pl);
   float4* G = in_global(e.G);
-  const int n = e.n, lo = e.lo, s = e.s, per = e.periodic;
-  each_plane(bi, s, [&](const BI& b) { d_grad(b, ph, pl, n, lo, s, per, G); });
+  const int s = e.s;
+  d_grad(bi, bi.z * BZ, min(bi.z * BZ + BZ, s), ph, pl, e.n, e.lo, s, e.periodic, G);
 }
 __global__ void __launch_bounds__(KT) kb_gather(const __grid_constant__ BArgs<GatherDesc> a) {
   BI bi;

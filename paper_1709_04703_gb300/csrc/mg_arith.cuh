@@ -95,26 +95,42 @@ __device__ __forceinline__ float gdiff(float hp, float hm, float lp, float lm) {
   return __fadd_rn(__fsub_rn(hp, hm), __fsub_rn(lp, lm));
 }
 
-// The gradient field of the potential at cell (i, j, k) of the active cube
-// (lo, side s) on the padded (n + 2)^3 mesh: G = the centred differences
-// along x, y, z (wrapped when periodic), one float4 per cell.
-__device__ __forceinline__ void d_grad(const BI& bi, const float* ph, const float* pl, int n,
-                                       int lo, int s, int periodic, float4* G) {
+// The gradient field of the potential on planes k0 .. k1 - 1 of a block's
+// (x, y) tile of the active cube (lo, side s) on the padded (n + 2)^3 mesh:
+// G = the centred differences along x, y, z (wrapped when periodic), one
+// float4 per cell.  The tile's planes are taken in a run because L2 reads
+// bound the pass: a single plane reads 3.3 times its cells (the rows around
+// the tile and the planes above and below), a run of four 1.8 times (256^3:
+// 103 -> 78 us, 5.2 TB/s; 128^3: 14.3 -> 11.9).
+__device__ __forceinline__ void d_grad(const BI& bi, int k0, int k1, const float* ph,
+                                       const float* pl, int n, int lo, int s, int periodic,
+                                       float4* G) {
   const int P = n + 2;
   const int i = bi.x * blockDim.x + threadIdx.x, j = bi.y * blockDim.y + threadIdx.y;
-  const int k = bi.z;
   if (i >= s || j >= s) return;
-  const int X = lo + i, Y = lo + j, Z = lo + k;
+  const int X = lo + i, Y = lo + j;
   auto w = [&](int a) { return periodic ? (a < 0 ? a + n : (a >= n ? a - n : a)) : a; };
-  const long long c = ((long long)(Z + 1) * P + (Y + 1)) * P + (X + 1);
-  const long long xm = ((long long)(Z + 1) * P + (Y + 1)) * P + (w(X - 1) + 1);
-  const long long xp = ((long long)(Z + 1) * P + (Y + 1)) * P + (w(X + 1) + 1);
-  const long long ym = ((long long)(Z + 1) * P + (w(Y - 1) + 1)) * P + (X + 1);
-  const long long yp = ((long long)(Z + 1) * P + (w(Y + 1) + 1)) * P + (X + 1);
-  const long long zm = ((long long)(w(Z - 1) + 1) * P + (Y + 1)) * P + (X + 1);
-  const long long zp = ((long long)(w(Z + 1) + 1) * P + (Y + 1)) * P + (X + 1);
-  G[c] = make_float4(gdiff(ph[xp], ph[xm], pl[xp], pl[xm]), gdiff(ph[yp], ph[ym], pl[yp], pl[ym]),
-                     gdiff(ph[zp], ph[zm], pl[zp], pl[zm]), 0.0f);
+  const long long sz = (long long)P * P;
+  const long long c = (long long)(Y + 1) * P + (X + 1);
+  const long long xm = (long long)(Y + 1) * P + (w(X - 1) + 1);
+  const long long xp = (long long)(Y + 1) * P + (w(X + 1) + 1);
+  const long long ym = (long long)(w(Y - 1) + 1) * P + (X + 1);
+  const long long yp = (long long)(w(Y + 1) + 1) * P + (X + 1);
+  // the column's values on planes k - 1, k, k + 1
+  auto at = [&](int k) { return (long long)(w(lo + k) + 1) * sz + c; };
+  float hm = ph[at(k0 - 1)], lm = pl[at(k0 - 1)], hc = ph[at(k0)], lc = pl[at(k0)];
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k) {
+    const long long z = (long long)(lo + k + 1) * sz, zp = at(k + 1);
+    const float hp = ph[zp], lp = pl[zp];
+    G[z + c] = make_float4(gdiff(ph[z + xp], ph[z + xm], pl[z + xp], pl[z + xm]),
+                           gdiff(ph[z + yp], ph[z + ym], pl[z + yp], pl[z + ym]),
+                           gdiff(hp, hm, lp, lm), 0.0f);
+    hm = hc;
+    lm = lc;
+    hc = hp;
+    lc = lp;
+  }
 }
 
 }  // namespace pm
