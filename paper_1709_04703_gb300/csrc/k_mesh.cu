@@ -489,14 +489,12 @@ __device__ __forceinline__ void d_source(const BI& bi,
     double* __restrict__ partial_f2,
     __int128* __restrict__ partial_m, unsigned int* counter, double* __restrict__ out,
     const double* __restrict__ bgm, double invM2_hi, int* __restrict__ overflow){
-  __int128 acc[SRC_NV];
-#pragma unroll
-  for (int q = 0; q < SRC_NV; ++q) acc[q] = 0;
-  // moments of the thread's column: sum c, c Z, c Z^2 with the count split
-  // c = c1 2^32 + c0 so that every partial sum is exact in int64 (at most
-  // 64 cells of |Z| < 2^11 per thread); the X, Y factors are constant along
-  // the column and applied once at the end in int128
-  long long m0[2] = {0, 0}, mz[2] = {0, 0}, mzz[2] = {0, 0};
+  // moments of the thread's column: sum c, c k, c k^2 with the count split
+  // c = c1 2^32 + c0 so that every product is one 32 x 32 -> 64-bit
+  // multiply-add and every partial sum exact in 64 bits (at most 64 cells of
+  // k < 2^11 per thread); Z = 2 k + 2 lo + 1 - n and the X, Y factors are
+  // constant or linear along the column and applied once at the end in int128
+  unsigned long long m0[2] = {0, 0}, mk[2] = {0, 0}, mkk[2] = {0, 0};
   float f2 = 0.f;
   // block (32, 8) covers an x-y tile; the grid's z dimension strides over
   // planes, ZU planes per round with all loads issued before any use
@@ -508,7 +506,7 @@ __device__ __forceinline__ void d_source(const BI& bi,
   // mean-density weight W = w_x w_y w_z (per-axis CIC image of the keep
   // interval, indexed by global cell; all ones in the periodic phase)
   df wxy{0.0f, 0.0f};
-  if (in_xy) wxy = df_mul(bgw[gi], bgw[gj]);
+  if (MOMENTS && in_xy) wxy = df_mul(bgw[gi], bgw[gj]);
   for (int k0 = bi.z; k0 < s && in_xy; k0 += ZU * bi.gz) {
     unsigned long long cnts[ZU];
 #pragma unroll
@@ -526,9 +524,11 @@ __device__ __forceinline__ void d_source(const BI& bi,
     if (cnt > (1ull << 62)) atomicOr(overflow, 1);
     long long c = (long long)cnt;
     df d = df_mul(df_from_u64(cnt), invM);
-    // ballw (spherical keep region): the mean density's image per cell
-    const df w = ballw ? df{ballw[((long long)gk * n + gj) * n + gi], 0.0f}
-                       : df_mul(wxy, bgw[gk]);
+    // ballw (spherical keep region): the mean density's image per cell;
+    // periodic (no moments): one
+    const df w = !MOMENTS ? df{1.0f, 0.0f}
+                 : ballw  ? df{ballw[((long long)gk * n + gj) * n + gi], 0.0f}
+                          : df_mul(wxy, bgw[gk]);
     d = df_add(d, df{-w.hi, -w.lo});
     df f = df_mul(d, S);
     int fi = gidx(fh, i, j, k);
@@ -536,32 +536,31 @@ __device__ __forceinline__ void d_source(const BI& bi,
     fl.base[fi] = f.lo;
     f2 = __fmaf_rn(f.hi, f.hi, f2);
     if (MOMENTS) {
-      const int Z = 2 * gk + 1 - n;
-      const long long c0 = (long long)(cnt & 0xffffffffull), c1 = (long long)(cnt >> 32);
+      const unsigned c0 = (unsigned)cnt, c1 = (unsigned)(cnt >> 32);
+      const unsigned ku = (unsigned)k, kk = ku * ku;
       m0[0] += c0;
       m0[1] += c1;
-      mz[0] += c0 * Z;
-      mz[1] += c1 * Z;
-      mzz[0] += c0 * (long long)(Z * Z);
-      mzz[1] += c1 * (long long)(Z * Z);
+      mk[0] += (unsigned long long)c0 * ku;
+      mk[1] += (unsigned long long)c1 * ku;
+      mkk[0] += (unsigned long long)c0 * kk;
+      mkk[1] += (unsigned long long)c1 * kk;
     }
     }
   }
-  if (MOMENTS && in_xy) {
-    const long long X = 2 * gi + 1 - n, Y = 2 * gj + 1 - n;
+  // sums over the warp, whose Y is the same: 1, X, Z, X^2, Z^2, Z X
+  __int128 acc[6];
+  if (MOMENTS) {
+    const long long X = 2 * gi + 1 - n, z0 = 2 * lo + 1 - n;
     const __int128 M0 = (__int128)m0[0] + ((__int128)m0[1] << 32);
-    const __int128 MZ = (__int128)mz[0] + ((__int128)mz[1] << 32);
-    const __int128 MZZ = (__int128)mzz[0] + ((__int128)mzz[1] << 32);
+    const __int128 MK = (__int128)mk[0] + ((__int128)mk[1] << 32);
+    const __int128 MKK = (__int128)mkk[0] + ((__int128)mkk[1] << 32);
+    const __int128 MZ = 2 * MK + z0 * M0;
     acc[0] = M0;
     acc[1] = M0 * X;
-    acc[2] = M0 * Y;
-    acc[3] = MZ;
-    acc[4] = M0 * (X * X);
-    acc[5] = M0 * (Y * Y);
-    acc[6] = MZZ;
-    acc[7] = M0 * (X * Y);
-    acc[8] = MZ * X;
-    acc[9] = MZ * Y;
+    acc[2] = MZ;
+    acc[3] = M0 * (X * X);
+    acc[4] = 4 * MKK + (4 * z0) * MK + (z0 * z0) * M0;
+    acc[5] = MZ * X;
   }
   // block reduction: ||f||^2 in double, moments in int128
   __shared__ double sf[32];
@@ -574,10 +573,21 @@ __device__ __forceinline__ void d_source(const BI& bi,
   if (lane == 0) sf[warp] = (double)wf;
   if (MOMENTS) {
 #pragma unroll
-    for (int q = 0; q < SRC_NV; ++q) {
-      __int128 v = acc[q];
-      for (int o = 16; o > 0; o >>= 1) v += shfl_xor_i128(v, o);
-      if (lane == 0) sm[warp * SRC_NV + q] = v;
+    for (int q = 0; q < 6; ++q)
+      for (int o = 16; o > 0; o >>= 1) acc[q] += shfl_xor_i128(acc[q], o);
+    if (lane == 0) {
+      const long long Y = 2 * (lo + bi.y * (int)blockDim.y + warp) + 1 - n;  // (a warp per row)
+      __int128* w = sm + warp * SRC_NV;
+      w[0] = acc[0];
+      w[1] = acc[1];
+      w[2] = acc[0] * Y;
+      w[3] = acc[2];
+      w[4] = acc[3];
+      w[5] = acc[0] * (Y * Y);
+      w[6] = acc[4];
+      w[7] = acc[1] * Y;
+      w[8] = acc[5];
+      w[9] = acc[2] * Y;
     }
   }
   __syncthreads();
@@ -663,8 +673,14 @@ __global__ void __launch_bounds__(256) k_source(
                     partial_m, counter, out, bgm, invM2_hi, overflow);
 }
 
+// Planes are strided over 16 blocks (8 from side 160 to 512: a thread's few
+// cells do not then pay for the block's reduction, which in the open phase
+// has ten int128 sums: open 192^3 90 us with the moments per cell and 16, 87
+// with 16, 70 with 8; periodic 256^3 97 -> 95 -> 90.  Above 512 a thread's
+// sums would pass 64 cells).
 dim3 source_grid(int s) {
-  return dim3((unsigned)((s + 31) / 32), (unsigned)((s + 7) / 8), (unsigned)(s < 16 ? s : 16));
+  const int gz = s >= 160 && s <= 512 ? 8 : 16;
+  return dim3((unsigned)((s + 31) / 32), (unsigned)((s + 7) / 8), (unsigned)(s < gz ? s : gz));
 }
 
 void launch_source(cudaStream_t st, int grid, unsigned long long* rho, int n, int lo,
