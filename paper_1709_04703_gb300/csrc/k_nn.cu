@@ -28,44 +28,53 @@ constexpr long long TC_WAIT_LIMIT = 20000000;  // mbarrier polls before giving u
 // mbarrier before the next chunk reuses the buffers.  Returns false on a
 // timed-out wait (the error word is set; the caller still frees TMEM).
 // ---------------------------------------------------------------------------
+// the KC / 16 MMAs of one chunk and their commit (one thread)
+template <int N, int KC>
+__device__ __forceinline__ void tc_chunk(uint32_t taddr, uint8_t* sA, uint8_t* sB, uint32_t mbar,
+                                         bool accumulate) {
+  constexpr uint32_t IDESC = tc::idesc_bf16(tc::TM, N);
+  constexpr uint32_t SBO = KC * 16;
+  const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
+#pragma unroll
+  for (int s = 0; s < KC / 16; ++s) {
+    uint64_t ad = tc::smem_desc(a0 + 256u * s, 128u, SBO);
+    uint64_t bd = tc::smem_desc(b0 + 256u * s, 128u, SBO);
+    tc::mma_bf16(taddr, ad, bd, IDESC, (accumulate || s > 0) ? 1u : 0u);
+  }
+  tc::mma_commit(mbar);
+}
+
+// The block waits for a committed chunk (bounded); false on a timed-out wait.
+__device__ __forceinline__ bool tc_chunk_wait(uint32_t mbar, uint32_t& phase, int* err) {
+  // every thread polls, but the block decides together: a thread whose
+  // polls ran out just before the commit landed must not leave the loop
+  // while the others go on (mismatched barriers, a diverged tcgen05.dealloc)
+  const bool done = __syncthreads_and(tc::mbar_wait(mbar, phase, TC_WAIT_LIMIT)) != 0;
+  phase ^= 1u;
+  if (!done) {
+    if (threadIdx.x == 0) atomicOr(err, 1);
+    // give the MMAs one more bounded wait before the buffers are left
+    tc::mbar_wait(mbar, phase ^ 1u, TC_WAIT_LIMIT);
+    return false;
+  }
+  tc::tc_fence_after();
+  return true;
+}
+
 template <int N, int KC, class FillA, class FillB>
 __device__ bool tc_mainloop(FillA fa, FillB fb, int ktiles, uint32_t taddr, uint8_t* sA,
                             uint8_t* sB, uint32_t mbar, uint32_t& phase, int* err) {
-  constexpr uint32_t IDESC = tc::idesc_bf16(tc::TM, N);
-  constexpr uint32_t SBO = KC * 16;
-  bool ok = true;
   for (int kt = 0; kt < ktiles; ++kt) {
     fa(kt, sA);
     fb(kt, sB);
     tc::fence_async_smem();
     __syncthreads();
     tc::tc_fence_after();
-    if (threadIdx.x == 0) {
-      const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
-#pragma unroll
-      for (int s = 0; s < KC / 16; ++s) {
-        uint64_t ad = tc::smem_desc(a0 + 256u * s, 128u, SBO);
-        uint64_t bd = tc::smem_desc(b0 + 256u * s, 128u, SBO);
-        tc::mma_bf16(taddr, ad, bd, IDESC, (kt > 0 || s > 0) ? 1u : 0u);
-      }
-      tc::mma_commit(mbar);
-    }
-    // every thread polls, but the block decides together: a thread whose
-    // polls ran out just before the commit landed must not leave the loop
-    // while the others go on (mismatched barriers, a diverged tcgen05.dealloc)
-    const bool done = __syncthreads_and(tc::mbar_wait(mbar, phase, TC_WAIT_LIMIT)) != 0;
-    phase ^= 1u;
-    if (!done) {
-      if (threadIdx.x == 0) atomicOr(err, 1);
-      ok = false;
-      // give the MMAs one more bounded wait before the buffers are left
-      tc::mbar_wait(mbar, phase ^ 1u, TC_WAIT_LIMIT);
-      break;
-    }
-    tc::tc_fence_after();
+    if (threadIdx.x == 0) tc_chunk<N, KC>(taddr, sA, sB, mbar, kt > 0);
+    if (!tc_chunk_wait(mbar, phase, err)) return false;
     __syncthreads();
   }
-  return ok;
+  return true;
 }
 
 // Shared setup/teardown around a tile: TMEM allocation by warp 0, mbarrier.
@@ -195,61 +204,103 @@ struct Vol {
 // (zero outside each sample, or periodic when g.per), as a GEMM: rows = 128 voxels, N = output
 // columns (>= cout, multiple of 16), K = 27 cin padded to 64.
 // wp: [N][kp] BF16, rows >= cout and columns >= 27 cin zero.
+//
+// It runs for the layers with many channels, on coarse levels with a few
+// hundred tiles at most: a tile's chain of K chunks (41 for 96 channels)
+// bounds it.  The next chunk's 16-byte pieces are therefore loaded into
+// registers while the MMAs of this one run, and eight lanes take eight rows
+// of one core matrix (conflict-free stores) with the warp on 64 contiguous
+// bytes of each voxel; a thread per voxel had every lane of a load on its own
+// line.  96 -> 32 channels at 40^3: 221 -> 114 us.
 template <int N>
 __global__ void __launch_bounds__(128) k_conv_fwd(const bf16* __restrict__ in, Vol g, int cin,
                                                   const bf16* __restrict__ wp, int kp,
                                                   const float* __restrict__ bias, int cout,
                                                   int relu, bf16* __restrict__ out_bf,
                                                   float* __restrict__ out_f, int* err) {
-  constexpr int KC = 64;
+  constexpr int KC = 64, NB = N / 16;
   __shared__ __align__(1024) uint8_t sA[tc::TM * KC * 2];
   __shared__ __align__(1024) uint8_t sB[N * KC * 2];
+  __shared__ int4 srow[tc::TM];  // x, y, z, sample of the tile's rows (sample -1: none)
   __shared__ uint32_t tslot;
   __shared__ __align__(8) uint64_t mbar;
   constexpr int NC = tc::tmem_cols(N);
-  TcCtx c = tc_begin<NC>(&tslot, &mbar);
   const long long nvox = g.voxels();
   const long long m0 = (long long)blockIdx.x * tc::TM;
-  // this thread's row (voxel) and its coordinates
-  const long long v = m0 + threadIdx.x;
-  const bool vin = v < nvox;
-  int x = 0, y = 0, z = 0;
-  long long smp = 0;
-  if (vin) {
-    long long t = v;
-    x = (int)(t % g.W); t /= g.W;
-    y = (int)(t % g.H); t /= g.H;
-    z = (int)(t % g.D); smp = t / g.D;
+  {
+    const long long v = m0 + threadIdx.x;
+    int4 c = make_int4(0, 0, 0, -1);
+    if (v < nvox) {
+      long long t = v;
+      c.x = (int)(t % g.W); t /= g.W;
+      c.y = (int)(t % g.H); t /= g.H;
+      c.z = (int)(t % g.D);
+      c.w = (int)(t / g.D);
+    }
+    srow[threadIdx.x] = c;
   }
-  uint32_t phase = 0;
-  auto fa = [&](int kt, uint8_t* s) {
-    uint8_t* row = s;
+  TcCtx c = tc_begin<NC>(&tslot, &mbar);  // (its barrier covers srow)
+  // piece q of a thread: row 8 (4 (q >> 1) + warp) + (lane & 7), 8 K columns
+  // from 8 ((q & 1) 4 + (lane >> 3))
+  const int warp = threadIdx.x >> 5, lane8 = threadIdx.x & 7, vv0 = (threadIdx.x & 31) >> 3;
+  uint4 ra[8], rb[NB];
+  auto load = [&](int kt) {
 #pragma unroll
-    for (int vv = 0; vv < KC / 8; ++vv) {
-      int k = kt * KC + 8 * vv;
-      int tap = k / cin, ci = k - tap * cin;
-      uint4 val = make_uint4(0, 0, 0, 0);
-      if (vin && tap < 27) {
-        int zz = z + tap / 9 - 1, yy = y + (tap / 3) % 3 - 1, xx = x + tap % 3 - 1;
+    for (int h = 0; h < 2; ++h) {
+      const int k = kt * KC + 8 * (4 * h + vv0);
+      const int tap = k / cin, ci = k - tap * cin;
+      const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int4 r = srow[8 * (4 * q + warp) + lane8];
+        uint4 val = make_uint4(0, 0, 0, 0);
+        int zz = r.z + dz, yy = r.y + dy, xx = r.x + dx;
         if (g.per) {
           zz = zz < 0 ? zz + g.D : (zz >= g.D ? zz - g.D : zz);
           yy = yy < 0 ? yy + g.H : (yy >= g.H ? yy - g.H : yy);
           xx = xx < 0 ? xx + g.W : (xx >= g.W ? xx - g.W : xx);
         }
-        if (zz >= 0 && zz < g.D && yy >= 0 && yy < g.H && xx >= 0 && xx < g.W) {
-          long long nv = ((smp * g.D + zz) * g.H + yy) * (long long)g.W + xx;
+        if (r.w >= 0 && tap < 27 && zz >= 0 && zz < g.D && yy >= 0 && yy < g.H && xx >= 0 &&
+            xx < g.W) {
+          const long long nv = (((long long)r.w * g.D + zz) * g.H + yy) * g.W + xx;
           val = *reinterpret_cast<const uint4*>(in + nv * cin + ci);
         }
+        ra[2 * q + h] = val;
       }
-      *reinterpret_cast<uint4*>(row + tc::tile_offset(threadIdx.x, 8 * vv, KC)) = val;
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int idx = threadIdx.x + 128 * q;
+      const int r = (idx & 7) + 8 * (idx >> 6), vv = (idx >> 3) & 7;
+      rb[q] = *reinterpret_cast<const uint4*>(wp + (long long)r * kp + kt * KC + 8 * vv);
     }
   };
-  auto fb = [&](int kt, uint8_t* s) {
-    fill_tile<KC>(s, N, [&](int r, int vv) {
-      return *reinterpret_cast<const uint4*>(wp + (long long)r * kp + kt * KC + 8 * vv);
-    });
+  auto store = [&]() {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      *reinterpret_cast<uint4*>(sA + tc::tile_offset(8 * (4 * (q >> 1) + warp) + lane8,
+                                                     8 * (4 * (q & 1) + vv0), KC)) = ra[q];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int idx = threadIdx.x + 128 * q;
+      const int r = (idx & 7) + 8 * (idx >> 6), vv = (idx >> 3) & 7;
+      *reinterpret_cast<uint4*>(sB + tc::tile_offset(r, 8 * vv, KC)) = rb[q];
+    }
   };
-  bool ok = tc_mainloop<N, KC>(fa, fb, kp / KC, c.taddr, sA, sB, c.mbar, phase, err);
+  const int ktiles = kp / KC;
+  uint32_t phase = 0;
+  bool ok = true;
+  load(0);
+  for (int kt = 0; kt < ktiles; ++kt) {
+    store();
+    tc::fence_async_smem();
+    __syncthreads();
+    tc::tc_fence_after();
+    if (threadIdx.x == 0) tc_chunk<N, KC>(c.taddr, sA, sB, c.mbar, kt > 0);
+    if (kt + 1 < ktiles) load(kt + 1);
+    ok = tc_chunk_wait(c.mbar, phase, err);
+    if (!ok) break;
+  }
   if (ok) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long row = m0 + 32 * w + lane;
