@@ -33,7 +33,12 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 constexpr long long CF_WAIT_LIMIT = 20000000;  // mbarrier polls before giving up
-constexpr int CF_NT = 128;                     // threads per CTA (one per TMEM lane)
+// Threads per CTA: two for each TMEM lane.  Staging and the epilogue, not the
+// MMAs, take most of a block's time (160^3, 8 -> 8: 98 MMAs, 2700
+// instructions a warp), and the layers of many channels have room for one
+// CTA per SM (the five layers of 16 columns of a 160^3 forward: 1283 us; 1451
+// with 128 threads).
+constexpr int CF_NT = 256;
 constexpr int CF_SLACK = 128;                  // rows past a block's end an M tile may touch
 constexpr int CF_MAXK = 192;                   // K slices of 16 a layer may have
 
@@ -96,6 +101,9 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
   // the A and B descriptors of every K slice for the first M tile (the
   // next tiles start 128 rows, i.e. 2048 bytes = 128 descriptor units, on)
   __shared__ uint64_t adesc[CF_MAXK], bdesc[CF_MAXK];
+  __shared__ float sbias[N];
+  if (threadIdx.x < N)
+    sbias[threadIdx.x] = bias && (int)threadIdx.x < cout ? bias[threadIdx.x] : 0.0f;
   // 1 KB-aligned start of the staged input; the weights follow the blocks
   uint8_t* sA = cf_sm + ((1024 - (tc::smem_u32(cf_sm) & 1023)) & 1023);
   uint8_t* sB = sA + sh.nbr * sh.cbs;
@@ -197,9 +205,11 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
     tc::mbar_wait(mbar, 0u, CF_WAIT_LIMIT);  // one more bounded wait before leaving
   } else {
     tc::tc_fence_after();
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a warp reads the TMEM lanes 32 (w % 4) .. + 31; the two halves of the
+    // CTA take the M tiles in turn
+    const int w = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
     const int coutp = (cout + 7) & ~7;
-    for (int m = 0; m < sh.mt; ++m) {
+    for (int m = threadIdx.x >> 7; m < sh.mt; m += CF_NT / 128) {
       const int p = sh.p0 + 128 * m + 32 * w + lane;
       int x, y, z, r;
       cf_divmod(p, px, 1.0f / (float)px, r, x);
@@ -210,13 +220,14 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
       const long long row = sbase + ((long long)gz * S + gy) * S + gx;
 #pragma unroll
       for (int col = 0; col < N; col += 8) {
+        if (col >= coutp) break;
         float val[8];
         tc::tmem_ld8(taddr, w, m * N + col, val);
-        if (valid && col < coutp) {
+        if (valid) {
           __align__(16) bf16 ob[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
-            float o = col + q < cout ? val[q] + (bias ? bias[col + q] : 0.0f) : 0.0f;
+            float o = col + q < cout ? val[q] + sbias[col + q] : 0.0f;
             if (relu) o = fmaxf(o, 0.0f);
             ob[q] = __float2bfloat16_rn(o);
             if (out_f) out_f[row * coutp + col + q] = o;
