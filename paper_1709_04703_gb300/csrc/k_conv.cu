@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
             float o = col + q < cout ? val[q] + sbias[col + q] : 0.0f;
             if (relu) o = fmaxf(o, 0.0f);
             ob[q] = __float2bfloat16_rn(o);
-            if (out_f) out_f[row * coutp + col + q] = o;
+            if (out_f && col + q == 0) out_f[row] = o;  // (channel 0 only)
           }
           if (out_bf)
             *reinterpret_cast<uint4*>(out_bf + row * coutp + col) =

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(128) k_conv_fwd(const bf16* __restrict__ in, V
           float o = col + q < cout ? val[q] + (bias ? bias[col + q] : 0.0f) : 0.0f;
           if (relu) o = fmaxf(o, 0.0f);
           ob[q] = __float2bfloat16_rn(o);
-          if (out_f) out_f[row * coutp + col + q] = o;
+          if (out_f && col + q == 0) out_f[row] = o;  // (channel 0 only)
         }
         if (out_bf) *reinterpret_cast<uint4*>(out_bf + row * coutp + col) =
                         *reinterpret_cast<const uint4*>(ob);
@@ -376,49 +376,71 @@ void launch_pack_w(cudaStream_t st, const float* w, int cin, int cout, void* wp,
 // ---------------------------------------------------------------------------
 // Elementwise kernels (channels-last BF16 unless stated).
 // ---------------------------------------------------------------------------
-// dy <- dy * (y > 0)
-__global__ void k_relu_bwd(bf16* __restrict__ dy, const bf16* __restrict__ y, long long n) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x)
-    if (!(__bfloat162float(y[t]) > 0.0f)) dy[t] = __float2bfloat16_rn(0.0f);
+// dy <- dy * (y > 0), 8 values (16 bytes) per step (n: a multiple of 8)
+__global__ void k_relu_bwd(uint4* __restrict__ dy, const uint4* __restrict__ y, long long n8) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n8;
+       t += (long long)gridDim.x * blockDim.x) {
+    uint4 d = dy[t];
+    const uint4 v = y[t];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (!(__bfloat162float(reinterpret_cast<const bf16*>(&v)[q]) > 0.0f))
+        reinterpret_cast<bf16*>(&d)[q] = __float2bfloat16_rn(0.0f);
+    dy[t] = d;
+  }
 }
 
-// 2x2x2 average pooling: out [B][D/2][H/2][W/2][C]
-__global__ void k_pool2(const bf16* __restrict__ in, Vol g, int C, bf16* __restrict__ out) {
+// 2x2x2 average pooling: out [B][D/2][H/2][W/2][C], 8 channels (16 bytes) per
+// step (C a multiple of 8; I: 32-bit arithmetic below 2^31 pieces of the fine
+// grid).  A 160^3 forward's three: 18 us; two bytes per step
+// took 53.
+template <class I>
+__global__ void k_pool2_v8(const uint4* __restrict__ in, Vol g, int C8, uint4* __restrict__ out) {
   const int D2 = g.D / 2, H2 = g.H / 2, W2 = g.W / 2;
-  const long long n = (long long)g.B * D2 * H2 * W2 * C;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    int c = (int)(t % C);
-    long long r = t / C;
-    int x = (int)(r % W2); r /= W2;
-    int y = (int)(r % H2); r /= H2;
-    int z = (int)(r % D2);
-    long long b = r / D2;
-    float acc = 0.0f;
+  const I n = (I)g.B * D2 * H2 * W2 * C8;
+  for (I t = (I)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (I)gridDim.x * blockDim.x) {
+    const int c = (int)(t % C8);
+    I r = t / C8;
+    const int x = (int)(r % W2); r /= W2;
+    const int y = (int)(r % H2); r /= H2;
+    const int z = (int)(r % D2);
+    const I b = r / D2;
+    uint4 v[8];
 #pragma unroll
-    for (int d = 0; d < 8; ++d) {
-      long long v = ((b * g.D + 2 * z + (d >> 2)) * g.H + 2 * y + ((d >> 1) & 1)) * (long long)g.W +
-                    2 * x + (d & 1);
-      acc += __bfloat162float(in[v * C + c]);
+    for (int d = 0; d < 8; ++d)
+      v[d] = in[(((b * g.D + 2 * z + (d >> 2)) * g.H + 2 * y + ((d >> 1) & 1)) * g.W + 2 * x +
+                 (d & 1)) * C8 + c];
+    __align__(16) bf16 o[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      float acc = 0.0f;
+#pragma unroll
+      for (int d = 0; d < 8; ++d) acc += __bfloat162float(reinterpret_cast<const bf16*>(&v[d])[q]);
+      o[q] = __float2bfloat16_rn(0.125f * acc);
     }
-    out[t] = __float2bfloat16_rn(0.125f * acc);
+    out[t] = *reinterpret_cast<const uint4*>(o);
   }
 }
 
 // backward of pooling: din[v] = dout[parent] / 8 (din has the fine shape g)
-__global__ void k_pool2_bwd(const bf16* __restrict__ dout, Vol g, int C, bf16* __restrict__ din) {
-  const long long n = g.voxels() * C;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    int c = (int)(t % C);
-    long long r = t / C;
-    int x = (int)(r % g.W); r /= g.W;
-    int y = (int)(r % g.H); r /= g.H;
-    int z = (int)(r % g.D);
-    long long b = r / g.D;
-    long long p = ((b * (g.D / 2) + z / 2) * (g.H / 2) + y / 2) * (long long)(g.W / 2) + x / 2;
-    din[t] = __float2bfloat16_rn(0.125f * __bfloat162float(dout[p * C + c]));
+template <class I>
+__global__ void k_pool2_bwd_v8(const uint4* __restrict__ dout, Vol g, int C8,
+                               uint4* __restrict__ din) {
+  const I n = (I)(g.voxels() * C8);
+  for (I t = (I)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (I)gridDim.x * blockDim.x) {
+    const int c = (int)(t % C8);
+    I r = t / C8;
+    const int x = (int)(r % g.W); r /= g.W;
+    const int y = (int)(r % g.H); r /= g.H;
+    const int z = (int)(r % g.D);
+    const I b = r / g.D;
+    const I p = ((b * (g.D / 2) + z / 2) * (g.H / 2) + y / 2) * (g.W / 2) + x / 2;
+    const uint4 v = dout[p * C8 + c];
+    __align__(16) bf16 o[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      o[q] = __float2bfloat16_rn(0.125f * __bfloat162float(reinterpret_cast<const bf16*>(&v)[q]));
+    din[t] = *reinterpret_cast<const uint4*>(o);
   }
 }
 
@@ -517,12 +539,18 @@ __global__ void k_chan_copy(const bf16* __restrict__ src, long long nvox, int C,
 // zero padding turns it into a boundary indicator), channels 2..7 zero
 __global__ void k_nn_input(const float* __restrict__ f, long long vps, const float* __restrict__ scale,
                            int B, bf16* __restrict__ x) {
-  const long long n = (long long)B * vps * 8;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+  // a voxel (16 bytes) per thread; blockIdx.y: the sample (160^3: 11.5
+  // us; two bytes per thread took 68)
+  const float sc = scale[blockIdx.y];
+  const long long v0 = blockIdx.y * vps;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < vps;
        t += (long long)gridDim.x * blockDim.x) {
-    int c = (int)(t & 7);
-    long long v = t >> 3;
-    x[t] = __float2bfloat16_rn(c == 0 ? f[v] * scale[v / vps] : (c == 1 ? 1.0f : 0.0f));
+    __align__(16) bf16 o[8];
+    o[0] = __float2bfloat16_rn(f[v0 + t] * sc);
+    o[1] = __float2bfloat16_rn(1.0f);
+#pragma unroll
+    for (int c = 2; c < 8; ++c) o[c] = __float2bfloat16_rn(0.0f);
+    *reinterpret_cast<uint4*>(x + (v0 + t) * 8) = *reinterpret_cast<const uint4*>(o);
   }
 }
 
@@ -536,7 +564,7 @@ __global__ void k_mse(const float* __restrict__ y, const float* __restrict__ tar
   double acc = 0.0;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
        v += (long long)gridDim.x * blockDim.x) {
-    float d = y[v * 8] - target[v] * tscale[v / vps];
+    float d = y[v] - target[v] * tscale[v / vps];
     acc += (double)d * d;
 #pragma unroll
     for (int c = 0; c < 8; ++c) dy[v * 8 + c] = __float2bfloat16_rn(c == 0 ? 2.0f * d * inv : 0.0f);
@@ -557,7 +585,7 @@ __global__ void k_loss_diff(const float* __restrict__ y, const float* __restrict
   const long long n = (long long)B * vps;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
        v += (long long)gridDim.x * blockDim.x)
-    d[v] = y[v * 8] - target[v] * tscale[v / vps];
+    d[v] = y[v] - target[v] * tscale[v / vps];
 }
 
 __device__ __forceinline__ float lap7(const float* __restrict__ d, const Vol& g, long long v) {
@@ -627,7 +655,7 @@ __global__ void k_nn_output(const float* __restrict__ y, long long vps, const fl
   const long long n = (long long)B * vps;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
        v += (long long)gridDim.x * blockDim.x)
-    phi[v] = y[v * 8] * scale[v / vps];
+    phi[v] = y[v] * scale[v / vps];
 }
 
 static inline int ew_grid(long long n) {
@@ -636,18 +664,26 @@ static inline int ew_grid(long long n) {
 }
 
 void launch_relu_bwd(cudaStream_t st, void* dy, const void* y, long long n) {
-  k_relu_bwd<<<ew_grid(n), 256, 0, st>>>((bf16*)dy, (const bf16*)y, n);
+  k_relu_bwd<<<ew_grid(n / 8), 256, 0, st>>>((uint4*)dy, (const uint4*)y, n / 8);
   note_launch();
 }
 void launch_pool2(cudaStream_t st, const void* in, int B, int D, int H, int W, int C, void* out) {
   Vol g{B, D, H, W};
-  k_pool2<<<ew_grid(g.voxels() * C / 8), 256, 0, st>>>((const bf16*)in, g, C, (bf16*)out);
+  const int grid = ew_grid(g.voxels() * C / 64);
+  if (g.voxels() * C / 8 < (1LL << 31))
+    k_pool2_v8<int><<<grid, 256, 0, st>>>((const uint4*)in, g, C / 8, (uint4*)out);
+  else
+    k_pool2_v8<long long><<<grid, 256, 0, st>>>((const uint4*)in, g, C / 8, (uint4*)out);
   note_launch();
 }
 void launch_pool2_bwd(cudaStream_t st, const void* dout, int B, int D, int H, int W, int C,
                       void* din) {
   Vol g{B, D, H, W};
-  k_pool2_bwd<<<ew_grid(g.voxels() * C), 256, 0, st>>>((const bf16*)dout, g, C, (bf16*)din);
+  const int grid = ew_grid(g.voxels() * C / 8);
+  if (g.voxels() * C / 8 < (1LL << 31) - (1LL << 20))
+    k_pool2_bwd_v8<int><<<grid, 256, 0, st>>>((const uint4*)dout, g, C / 8, (uint4*)din);
+  else
+    k_pool2_bwd_v8<long long><<<grid, 256, 0, st>>>((const uint4*)dout, g, C / 8, (uint4*)din);
   note_launch();
 }
 void launch_up2(cudaStream_t st, const void* in, int B, int D, int H, int W, int C, void* out,
@@ -680,7 +716,7 @@ void launch_chan_copy(cudaStream_t st, const void* src, long long nvox, int C, i
 }
 void launch_nn_input(cudaStream_t st, const float* f, long long vps, const float* scale, int B,
                      void* x) {
-  k_nn_input<<<ew_grid((long long)B * vps * 8), 256, 0, st>>>(f, vps, scale, B, (bf16*)x);
+  k_nn_input<<<dim3(ew_grid(vps), B), 256, 0, st>>>(f, vps, scale, B, (bf16*)x);
   note_launch();
 }
 void launch_mse(cudaStream_t st, const float* y, const float* target, long long vps,

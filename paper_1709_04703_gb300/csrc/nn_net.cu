@@ -125,7 +125,7 @@ pm_status ensure_shape(pm_guess* g, int B, int S) {
     gmax = std::max(gmax, vox(B, S, l) * c);
   }
   ok = ok && alloc(SLOT_G0, gmax) && alloc(SLOT_G1, gmax) && alloc(SLOT_G2, gmax);
-  ok = ok && cudaMalloc((void**)&g->y, sizeof(float) * need * 8) == cudaSuccess;
+  ok = ok && cudaMalloc((void**)&g->y, sizeof(float) * need) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&g->ld, sizeof(float) * need) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&g->lq, sizeof(float) * need) == cudaSuccess;
   if (!ok) return gfail(g, PM_ENOMEM, "guess: activation allocation failed");
@@ -187,10 +187,11 @@ __global__ void k_rms_part(const float* __restrict__ f, long long vps, double* _
 __global__ void k_rms(const double* __restrict__ part, long long vps, int B, float out_scale,
                       float* __restrict__ sin_, float* __restrict__ sout,
                       float* __restrict__ tsc) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
+  const int b = blockIdx.x;  // a warp per sample
   double t = 0.0;
-  for (int q = 0; q < RMS_BLOCKS; ++q) t += part[(long long)b * RMS_BLOCKS + q];
+  for (int q = threadIdx.x; q < RMS_BLOCKS; q += 32) t += part[(long long)b * RMS_BLOCKS + q];
+  t = warp_sum(t);
+  if (threadIdx.x != 0) return;
   const double rms = sqrt(t / (double)vps);
   sin_[b] = rms > 0 ? (float)(1.0 / rms) : 0.0f;
   sout[b] = rms > 0 ? (float)(rms * out_scale) : 0.0f;
@@ -210,7 +211,7 @@ pm_status forward(pm_guess* g, const float* f, int B, int S, int per) {
   if (!g->packed) pack_all(g);
   const long long vps = (long long)S * S * S;
   k_rms_part<<<dim3(RMS_BLOCKS, B), 256, 0, g->st>>>(f, vps, g->rms_part);
-  k_rms<<<(B + 127) / 128, 128, 0, g->st>>>(g->rms_part, vps, B, g->out_scale, g->scale_in,
+  k_rms<<<B, 32, 0, g->st>>>(g->rms_part, vps, B, g->out_scale, g->scale_in,
                                             g->scale_out, g->tscale);
   note_launch();
   note_launch();
