@@ -141,11 +141,19 @@ void pack_all(pm_guess* g) {
   g->packed = true;
   g->packed_t = false;
 }
-// the input gradients' operands: packed by the first backward pass after
-// pack_all (a forward-only user never pays for them)
+// the input gradients' operands: allocated by the first backward pass and
+// packed by the first after pack_all (a forward-only user pays for neither);
+// without the memory a layer keeps the gathered tile
 void pack_bwd(pm_guess* g) {
-  for (auto& c : g->conv)
+  for (auto& c : g->conv) {
+    if (c.fast_tt && !c.wft &&
+        cudaMalloc(&c.wft, (size_t)c.nt * conv_fast_kf(round_up(c.cout, 8)) * 2) != cudaSuccess) {
+      cudaGetLastError();
+      c.wft = nullptr;
+      c.fast_tt = 0;
+    }
     if (c.fast_tt) launch_pack_wf(g->st, g->w + c.w_off, c.cin, c.cout, c.nt, true, c.wft);
+  }
   g->packed_t = true;
 }
 
@@ -376,10 +384,7 @@ pm_status pm_guess_create(int32_t levels, void* stream, pm_guess** out) {
       ok = ok && cudaMalloc(&c.wf, (size_t)c.n * conv_fast_kf(c.cin) * 2) == cudaSuccess;
     // the input gradient likewise (the five of a 4-level net at 96^3 that
     // fit: 490 us on the gathered tile, 286 staged)
-    const int co8 = round_up(c.cout, 8);
-    c.fast_tt = getenv("PM_NN_GATHER") ? 0 : conv_fast_side(co8, c.cin);
-    if (c.fast_tt)
-      ok = ok && cudaMalloc(&c.wft, (size_t)c.nt * conv_fast_kf(co8) * 2) == cudaSuccess;
+    c.fast_tt = getenv("PM_NN_GATHER") ? 0 : conv_fast_side(round_up(c.cout, 8), c.cin);
   }
   size_t pb = sizeof(float) * g->n_params;
   ok = ok && cudaMalloc((void**)&g->w, pb) == cudaSuccess &&
