@@ -2,15 +2,15 @@
 // gradient with the taps reversed) as an implicit
 // GEMM on the 5th-generation tensor cores without an im2col copy.
 //
-// A CTA computes a T^3 block of output voxels of one sample.  It stages the
-// (T+2)^3 input block once in shared memory, channel-blocked: block c holds
+// A CTA computes a tx x ty x tz block of output voxels of one sample.  It
+// stages the input block with its halo once in shared memory, channel-blocked: block c holds
 // channels 8c .. 8c+7 of every position as one 16-byte row, positions in
 // raster order of the padded block (x fastest).  In the K-major no-swizzle
 // canonical layout an MMA operand of 128 rows x 16 K-elements is two
 // 8-element core-matrix columns, each 128 rows of 16 bytes at a common row
 // stride of 16 bytes; so the A operand of tap (dz, dy, dx) for 128
 // consecutive positions is the staged block itself, started
-// ((dz-1) P_yx + (dy-1) P_x + (dx-1)) rows further on, with the second core
+// ((dz-1) P_y P_x + (dy-1) P_x + (dx-1)) rows further on, with the second core
 // column one channel block further (LBO = the block stride), or, for 8
 // input channels, at the next tap (LBO = that tap's extra shift).  Every
 // (tap, channel pair) is one tcgen05.mma issued straight from the staged
@@ -23,6 +23,8 @@
 // the 28th zero) or 27 taps x cinp (cinp = cin rounded up to 16; channels
 // beyond cin zero), tap-major, loaded whole into shared memory.
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "pm_kernels.cuh"
 #include "tc_gemm.cuh"
@@ -59,26 +61,31 @@ __device__ __forceinline__ void cf_cp16(uint8_t* smem, const void* gmem, int src
 }
 
 struct CfShape {
-  int T;      // output block side
-  int P;      // positions of the padded block, (T + 2)^3
-  int nbr;    // channel blocks staged (cin / 8)
-  int cbs;    // bytes between channel blocks (P + slack rows)
-  int mt;     // M tiles of 128 positions
-  int p0;     // position of the first output, (P_x + 1) P_x + 1 with P_x = T + 2
-  int kf;     // K of wf
-  int ncols;  // TMEM columns allocated (power of two >= mt N)
-  int smem;   // dynamic shared memory bytes
+  int tx, ty, tz;  // output block
+  int px, py;      // sides of the padded block, tx + 2 and ty + 2
+  int P;           // positions of the padded block
+  int nbr;         // channel blocks staged (cin / 8)
+  int cbs;         // bytes between channel blocks (P + slack rows)
+  int mt;          // M tiles of 128 positions
+  int p0;          // position of the first output
+  int kf;          // K of wf
+  int ncols;       // TMEM columns allocated (power of two >= mt N)
+  int smem;        // dynamic shared memory bytes
 };
 
-__host__ __device__ inline CfShape cf_shape(int T, int cin, int n) {
+__host__ __device__ inline CfShape cf_shape(int tx, int ty, int tz, int cin, int n) {
   CfShape s{};
-  const int px = T + 2;
-  s.T = T;
-  s.P = px * px * px;
+  const int px = tx + 2, py = ty + 2;
+  s.tx = tx;
+  s.ty = ty;
+  s.tz = tz;
+  s.px = px;
+  s.py = py;
+  s.P = px * py * (tz + 2);
   s.nbr = cin / 8;
   s.cbs = (s.P + CF_SLACK) * 16;
-  s.p0 = (px + 1) * px + 1;
-  const int last = (T * px + T) * px + T;  // position of the last output
+  s.p0 = (py + 1) * px + 1;
+  const int last = (tz * py + ty) * px + tx;  // position of the last output
   s.mt = (last - s.p0 + 1 + 127) / 128;
   s.kf = cin == 8 ? 28 * 8 : 27 * ((cin + 15) / 16 * 16);
   int need = s.mt * n, c = 32;
@@ -107,14 +114,15 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
   // 1 KB-aligned start of the staged input; the weights follow the blocks
   uint8_t* sA = cf_sm + ((1024 - (tc::smem_u32(cf_sm) & 1023)) & 1023);
   uint8_t* sB = sA + sh.nbr * sh.cbs;
-  const int T = sh.T, px = T + 2;
-  const int tiles = (S + T - 1) / T;
+  const int px = sh.px, py = sh.py;
   int bid = blockIdx.x;
-  const int tx = bid % tiles; bid /= tiles;
-  const int ty = bid % tiles; bid /= tiles;
-  const int tz = bid % tiles;
-  const int smp = bid / tiles;
-  const int x0 = tx * T - 1, y0 = ty * T - 1, z0 = tz * T - 1;  // sample coordinates of position 0
+  const int nx = (S + sh.tx - 1) / sh.tx, ny = (S + sh.ty - 1) / sh.ty;
+  const int nz = (S + sh.tz - 1) / sh.tz;
+  // sample coordinates of position 0
+  const int x0 = (bid % nx) * sh.tx - 1; bid /= nx;
+  const int y0 = (bid % ny) * sh.ty - 1; bid /= ny;
+  const int z0 = (bid % nz) * sh.tz - 1;
+  const int smp = bid / nz;
   const long long sbase = (long long)smp * S * S * S;
 
   if (threadIdx.x < 32) tc::tmem_alloc(&tslot, sh.ncols);
@@ -132,12 +140,12 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
   // (zero-filled outside an open sample, wrapped in a periodic one); the
   // slack rows are zeroed
   const int rows = sh.nbr * sh.P;
-  const float inv_px = 1.0f / (float)px, inv_p = 1.0f / (float)sh.P;
+  const float inv_px = 1.0f / (float)px, inv_py = 1.0f / (float)py, inv_p = 1.0f / (float)sh.P;
   for (int t = threadIdx.x; t < rows; t += CF_NT) {
     int c, p, x, y, z, r;
     cf_divmod(t, sh.P, inv_p, c, p);
     cf_divmod(p, px, inv_px, r, x);
-    cf_divmod(r, px, inv_px, z, y);
+    cf_divmod(r, py, inv_py, z, y);
     int gx = x0 + x, gy = y0 + y, gz = z0 + z;
     if (per) {
       gx = gx < 0 ? gx + S : (gx >= S ? gx - S : gx);
@@ -164,8 +172,8 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
       if (cin == 8) {
         // taps 2s and 2s + 1 (the 28th tap has zero weights: any rows)
         const int t0 = 2 * s, t1 = 2 * s + 1;
-        const int sh0 = (t0 / 9 - 1) * px * px + ((t0 / 3) % 3 - 1) * px + (t0 % 3 - 1);
-        const int sh1 = t1 < 27 ? (t1 / 9 - 1) * px * px + ((t1 / 3) % 3 - 1) * px + (t1 % 3 - 1)
+        const int sh0 = (t0 / 9 - 1) * px * py + ((t0 / 3) % 3 - 1) * px + (t0 % 3 - 1);
+        const int sh1 = t1 < 27 ? (t1 / 9 - 1) * px * py + ((t1 / 3) % 3 - 1) * px + (t1 % 3 - 1)
                                 : sh0;
         a = a0 + (uint32_t)(sh.p0 + sh0) * 16u;
         lbo = (uint32_t)(sh1 - sh0) * 16u;
@@ -174,7 +182,7 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
         // staged ones has zero weights: it re-reads block 2j)
         const int per_tap = cinp / 16;
         const int t = s / per_tap, j = s - t * per_tap;
-        const int sht = (t / 9 - 1) * px * px + ((t / 3) % 3 - 1) * px + (t % 3 - 1);
+        const int sht = (t / 9 - 1) * px * py + ((t / 3) % 3 - 1) * px + (t % 3 - 1);
         a = a0 + (uint32_t)(2 * j) * (uint32_t)sh.cbs + (uint32_t)(sh.p0 + sht) * 16u;
         lbo = 2 * j + 1 < sh.nbr ? (uint32_t)sh.cbs : 0u;
       }
@@ -212,11 +220,11 @@ __global__ void __launch_bounds__(CF_NT) k_conv_fast(const bf16* __restrict__ in
     for (int m = threadIdx.x >> 7; m < sh.mt; m += CF_NT / 128) {
       const int p = sh.p0 + 128 * m + 32 * w + lane;
       int x, y, z, r;
-      cf_divmod(p, px, 1.0f / (float)px, r, x);
-      cf_divmod(r, px, 1.0f / (float)px, z, y);
+      cf_divmod(p, px, inv_px, r, x);
+      cf_divmod(r, py, inv_py, z, y);
       const int gx = x0 + x, gy = y0 + y, gz = z0 + z;
-      const bool valid = x >= 1 && x <= T && y >= 1 && y <= T && z >= 1 && z <= T &&
-                         gx < S && gy < S && gz < S;
+      const bool valid = x >= 1 && x <= sh.tx && y >= 1 && y <= sh.ty && z >= 1 &&
+                         z <= sh.tz && gx < S && gy < S && gz < S;
       const long long row = sbase + ((long long)gz * S + gy) * S + gx;
 #pragma unroll
       for (int col = 0; col < N; col += 8) {
@@ -273,19 +281,69 @@ bool cf_set_attr(int smem) {
                               smem) == cudaSuccess;
 }
 
+long long cf_blocks(const CfShape& s, int B, int S) {
+  return (long long)B * ((S + s.tx - 1) / s.tx) * ((S + s.ty - 1) / s.ty) *
+         ((S + s.tz - 1) / s.tz);
+}
+
+// The block for B samples of side S.  An MMA of 128 rows takes 64 cycles
+// whatever its columns, and an M tile's rows on the halo are lost: 8^3 blocks
+// (57 % of the rows are outputs) against 16 x 16 x 2 or 20 x 10 x 2 (80 %).
+// So of the blocks that fit, the one whose busiest SM takes the fewest
+// cycles, counting MMAs, staged 16-byte pieces and a start per block, the two
+// overlapped where several blocks share an SM.  Every block gives a voxel the
+// same MMAs in the same order: the same bits.  160^3 forward, layers of 16
+// columns: 1283 us with 8^3 blocks, 996 so.
+CfShape cf_choose(int B, int S, int cin, int n, int T) {
+  struct Entry {
+    int B, S, cin, n;
+    CfShape sh;
+  };
+  thread_local Entry memo[16];  // (a function of its key alone)
+  thread_local int next = 0;
+  for (const Entry& e : memo)
+    if (e.B == B && e.S == S && e.cin == cin && e.n == n) return e.sh;
+  T = std::min(T, S);  // a block never larger than the sample
+  CfShape best{};
+  double best_cost = 0.0;
+  auto offer = [&](int x, int y, int z) {
+    const CfShape s = cf_shape(x, y, z, cin, n);
+    if (s.smem > CF_SMEM_MAX || s.mt * n > 128) return;
+    const int occ = std::min(512 / s.ncols, 227 * 1024 / (s.smem + 5 * 1024));
+    const double per_sm = (double)((cf_blocks(s, B, S) + 151) / 152);
+    const double mma = 64.0 * s.mt * (s.kf / 16);
+    const double stage = 1.2 * s.nbr * s.P + 1.2 * n * (s.kf / 8) + 2000.0;
+    const double one = occ >= 2 && per_sm >= 2.0
+                           ? std::max(mma, stage) + 0.25 * std::min(mma, stage)
+                           : mma + stage;
+    if (best.P == 0 || per_sm * one < best_cost) {
+      best = s;
+      best_cost = per_sm * one;
+    }
+  };
+  offer(T, T, T);
+  for (int x : {8, 10, 12, 14, 16, 20, 24, 32})
+    for (int y : {4, 6, 8, 10, 12, 14, 16})
+      for (int z : {1, 2, 4, 6, 8})
+        if (x <= S && y <= S && z <= S) offer(x, y, z);
+  memo[next] = Entry{B, S, cin, n, best};
+  next = (next + 1) % 16;
+  return best;
+}
+
 }  // namespace
 
 int conv_fast_kf(int cin);
 
-// The block side for a layer, or 0 when the staged block and the weights do
-// not fit in shared memory or the accumulators in 128 TMEM columns (four
+// The side of a cubic block for a layer (cf_choose starts from it), or 0 when
+// the staged block and the weights do not fit in shared memory or the accumulators in 128 TMEM columns (four
 // CTAs per SM) at any side >= 4.
 int conv_fast_side(int cin, int cout) {
   if (cin % 8 != 0 || conv_fast_kf(cin) / 16 > CF_MAXK) return 0;
   const int n = cout <= 16 ? 16 : (cout + 15) / 16 * 16;
   if (n != 16 && n != 32 && n != 48 && n != 64) return 0;
   for (int T = 14; T >= 4; --T) {
-    const CfShape s = cf_shape(T, cin, n);
+    const CfShape s = cf_shape(T, T, T, cin, n);
     if (s.smem <= CF_SMEM_MAX && s.mt * n <= 128) return T;
   }
   return 0;
@@ -303,10 +361,8 @@ void launch_pack_wf(cudaStream_t st, const float* w, int cin, int cout, int n, b
 bool launch_conv_fast(cudaStream_t st, const void* in, int B, int S, int per, int cin,
                       const void* wf, int n, int T, const float* bias, int cout, int relu,
                       void* out_bf, float* out_f, int* err) {
-  if (T > S) T = S;  // a block never larger than the sample
-  const CfShape sh = cf_shape(T, cin, n);
-  const int tiles = (S + T - 1) / T;
-  const dim3 grid((unsigned)(B * tiles * tiles * tiles));
+  const CfShape sh = cf_choose(B, S, cin, n, T);
+  const dim3 grid((unsigned)cf_blocks(sh, B, S));
 #define PM_CF(NN)                                                                       \
   if (!cf_set_attr<NN>(sh.smem)) return false;                                          \
   k_conv_fast<NN><<<grid, CF_NT, sh.smem, st>>>((const bf16*)in, B, S, per, cin,          \

@@ -111,3 +111,17 @@ def test_staged_input_gradient_matches_gathered(lib, S, B, per):
     for k, tol in ((0, 1e-2), (1, 2e-2)):
         err = np.sqrt(((a[k] - b[k]) ** 2).sum() / (b[k] ** 2).sum())
         assert err < tol, (k, err)
+
+
+@pytest.mark.parametrize("S,B,per", [(8, 1, 1), (48, 1, 0), (56, 1, 1), (72, 2, 0), (96, 1, 1)])
+def test_staged_block_shapes(lib, S, B, per):
+    """The staged kernel picks its block (x, y and z sides of their own) by
+    the sample side and count: sides that give long, flat, partial and
+    one-voxel blocks on the four levels, against the gathered kernel; the
+    tolerance is that of test_staged_forward_matches_gathered."""
+    g = torch.Generator().manual_seed(S + B + per)
+    src = torch.randn(B, S, S, S, generator=g).cuda()
+    a = _forward(src, S, per, gather=False)
+    b = _forward(src, S, per, gather=True)
+    err = np.sqrt(((a - b) ** 2).sum() / (b**2).sum())
+    assert err < 5e-3, err
