@@ -212,8 +212,9 @@ __global__ void k_rms(const double* __restrict__ part, long long vps, int B, flo
     if (e_ != cudaSuccess) return gfail(g, PM_ECUDA, cudaGetErrorString(e_));          \
   } while (0)
 
-// forward pass for B samples of side S starting from f (FP32, B*S^3)
-pm_status forward(pm_guess* g, const float* f, int B, int S, int per) {
+// forward pass for B samples of side S starting from f (FP32, B*S^3); keep:
+// a backward pass follows, which reads the decoder's concatenated inputs
+pm_status forward(pm_guess* g, const float* f, int B, int S, int per, bool keep) {
   pm_status st = ensure_shape(g, B, S);
   if (st != PM_OK) return st;
   if (!g->packed) pack_all(g);
@@ -242,10 +243,15 @@ pm_status forward(pm_guess* g, const float* f, int B, int S, int per) {
   for (int l = L - 2; l >= 0; --l) {
     int s = S >> l, cl = 8 << l, cu = 8 << (l + 1);
     const void* up = (l + 1 == L - 1) ? g->act[SLOT_E + l + 1].p : g->act[SLOT_D + l + 1].p;
+    ConvL& c = g->conv[ci++];
+    if (!keep && c.fast_t &&
+        launch_conv_fast(g->st, g->act[SLOT_E + l].p, B, s, per, c.cin, c.wf, c.n, c.fast_t,
+                         g->w + c.b_off, c.cout, 1, g->act[SLOT_D + l].p, nullptr, g->err, up,
+                         cu))
+      continue;
     launch_up2(g->st, up, B, s, s, s, cu, g->act[SLOT_C + l].p, cu + cl, 0);
     launch_chan_copy(g->st, g->act[SLOT_E + l].p, vox(B, S, l), cl, cl, 0, g->act[SLOT_C + l].p,
                      cu + cl, cu, false);
-    ConvL& c = g->conv[ci++];
     conv_fwd(g, c, g->act[SLOT_C + l].p, B, s, per, 1, g->act[SLOT_D + l].p, nullptr);
   }
   ConvL& c = g->conv[ci];
@@ -332,7 +338,7 @@ bool pm::guess_fits(const pm_guess* g, int S) {
 pm_status pm::guess_apply(pm_guess* g, cudaStream_t st, const float* src, int S, int per,
                           float* out) {
   g->st = st;
-  pm_status r = forward(g, src, 1, S, per);
+  pm_status r = forward(g, src, 1, S, per, false);
   if (r == PM_OK) launch_nn_output(st, g->y, (long long)S * S * S, g->scale_out, 1, out);
   g->st = g->st0;
   return r;
@@ -438,7 +444,7 @@ pm_status pm_guess_forward(pm_guess* g, const float* f_dev, int32_t B, int32_t S
                            int32_t periodic, float* phi_dev) {
   if (!g || !f_dev || !phi_dev || B < 1 || B > 4096 || S < 1) return PM_EINVAL;
   g->st = g->st0;
-  pm_status st = forward(g, f_dev, B, S, periodic ? 1 : 0);
+  pm_status st = forward(g, f_dev, B, S, periodic ? 1 : 0, false);
   if (st != PM_OK) return st;
   launch_nn_output(g->st, g->y, (long long)S * S * S, g->scale_out, B, phi_dev);
   int h = 0;
@@ -453,7 +459,7 @@ pm_status pm_guess_loss_grad(pm_guess* g, const float* f_dev, const float* phi_d
   if (!g || !f_dev || !phi_dev || B < 1 || B > 4096 || S < 1 || loss_kind < 0 || loss_kind > 1)
     return PM_EINVAL;
   g->st = g->st0;
-  pm_status st = forward(g, f_dev, B, S, periodic ? 1 : 0);
+  pm_status st = forward(g, f_dev, B, S, periodic ? 1 : 0, true);
   if (st != PM_OK) return st;
   st = backward(g, phi_dev, B, S, periodic ? 1 : 0, loss_kind);
   if (st != PM_OK) return st;

@@ -180,7 +180,8 @@ void launch_pack_wf(cudaStream_t st, const float* w, int cin, int cout, int n, b
                     void* wf);
 bool launch_conv_fast(cudaStream_t st, const void* in, int B, int S, int per, int cin,
                       const void* wf, int n, int T, const float* bias, int cout, int relu,
-                      void* out_bf, float* out_f, int* err);
+                      void* out_bf, float* out_f, int* err, const void* up = nullptr,
+                      int cup = 0);
 int gkd_blocks(long long N);
 // G: gradient field of k_grad (NULL: differences taken from Phi directly)
 void launch_gather_kick_drift(cudaStream_t st, float4* pos, float4* mom, long long N,
