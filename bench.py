@@ -165,14 +165,13 @@ ARITHMETIC = {
 # ncu dram__bytes_read.sum + dram__bytes_write.sum over the algorithmic bytes
 # of the kernel class's launches at 256^3 on the current kernels
 TRAFFIC_RATIO = {
-    # the smoother's algorithmic bytes are 12 B per cell and sweep, 48 B per
-    # pre + post pair of fused passes (the 256^3 level: 32 x 32 tiles)
-    "smooth0": ((93332224 + 187955712) / (48.0 * 256**3), "k_rbgs2<32> pre + post at 256^3, "
-                "profiles/rbgs2_pm256_level0.md"),
-    "defect": ((327600640 + 515282176) / (335.5e6 + 536.9e6), "k_defect<0> + k_defect<1> at "
-               "256^3, profiles/rbgs2_pm256_level0.md"),
-    "deposit": (1127.8e6 / 1073.7e6, "k_drift_deposit at 256^3, "
-                "profiles/defect_gather_deposit_pm256.md"),
+    # the smoother's algorithmic bytes are 12 B per cell and sweep and 9 for
+    # the residual and restriction in the leg down: 57 B per pair of legs
+    "smooth0": ((71951616 + 31623424 + 152123904 + 36274176) / (57.0 * 256**3),
+                "k_tile down + k_rbgs2 at 256^3, profiles/kernels_pm256.md"),
+    "defect": ((273779712 + 50797824 + 347053312 + 169682688) / (335.5e6 + 536.9e6),
+               "k_defect<0> + k_defect<1> at 256^3, profiles/kernels_pm256.md"),
+    "deposit": (1127.9e6 / 1073.7e6, "k_drift_deposit at 256^3, profiles/kernels_pm256.md"),
     "gather": (1294.6e6 / 1342.2e6, "k_gather_kick_drift at 256^3, "
                "profiles/defect_gather_deposit_pm256.md"),
 }

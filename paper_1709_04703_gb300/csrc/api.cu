@@ -1107,10 +1107,11 @@ pm_status solve(pm_ctx* ctx) {
       }
       continue;
     }
-    // The last solves (VC_SAME of them) having taken the same number of
-    // V-cycles, this one is expected to take it too: where that is one more than have run, the
-    // V-cycle and its defect are queued before the residuals are read, both
-    // in one read (a host round trip leaves the GPU idle for 15 to 20 us).
+    // The last VC_SAME solves having taken the same number of V-cycles, this
+    // one is expected to take it too: where that is one more than have run,
+    // the V-cycle and its defect are queued before the residuals are read,
+    // both in one read (a host round trip leaves the GPU idle for 15 to 20
+    // us).
     // They write the correction, r and the other potential buffer, none of
     // which is used if the solve turns out to have converged before: the same
     // V-cycles, the same bits.
