@@ -266,7 +266,10 @@ __device__ __forceinline__ void tsc_axis_f(float u, int& i, float w[3]) {
   w[2] = (float)w2 * sc;
 }
 
-__global__ void __launch_bounds__(KT) k_gather_tsc(
+// (Three blocks per SM, 85 registers: 2.1 million particles 60 us; two, 92
+// registers, 65; four, 62, and the CIC gather loses from more warps, whose
+// nodes share less of L1.)
+__global__ void __launch_bounds__(KT, 3) k_gather_tsc(
     float4* __restrict__ pos, float4* __restrict__ mom, long long N,
     const float4* __restrict__ G, int n, int lo, int s, int periodic, float kick, float c2,
     int do_flag, float klo, float khi, unsigned char* __restrict__ flags,
