@@ -349,8 +349,8 @@ CfShape cf_choose(int B, int S, int cin, int n, int T) {
 int conv_fast_kf(int cin);
 
 // The side of a cubic block for a layer (cf_choose starts from it), or 0 when
-// the staged block and the weights do not fit in shared memory or the accumulators in 128 TMEM columns (four
-// CTAs per SM) at any side >= 4.
+// the staged block and the weights do not fit in shared memory or the
+// accumulators in 128 TMEM columns (four CTAs per SM) at any side >= 4.
 int conv_fast_side(int cin, int cout) {
   if (cin % 8 != 0 || conv_fast_kf(cin) / 16 > CF_MAXK) return 0;
   const int n = cout <= 16 ? 16 : (cout + 15) / 16 * 16;
