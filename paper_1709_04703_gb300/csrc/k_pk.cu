@@ -53,8 +53,12 @@ void launch_pk_delta(cudaStream_t st, const unsigned long long* rho, float* delt
 //  - what depends on one axis alone is tabulated once, in FP64 (k_pk_axes);
 //  - the up to four stored modes that share |kx|, |ky|, |kz| share W, C1, C2
 //    and the bin, so they are added up first;
-//  - C2 and the bin sums are double-float (error below 2^-45, the FFT's own
-//    rounding 2^-24); the bin comes from integers: |k|/k_f >= b + 1/2 iff
+//  - C2 and the sums of P are double-float (error below 2^-45; the FFT rounds
+//    at 2^-24, and P's distance from 64 bits, 2e-7 and up, is what it was with
+//    FP64 sums).  |k| knows no FFT: its values and sums are three floats, exact
+//    beyond 64 bits (with pairs the mean |k| of a 32^3 mesh's bins was 3.5e-16
+//    off in the mean, 2.5 times as far as with FP64 sums);
+//  - the bin comes from integers: |k|/k_f >= b + 1/2 iff
 //    b (b + 1) < kx^2 + ky^2 + kz^2 in units of k_f;
 //  - along a row of kx the bin does not fall, so a warp sums runs of one bin
 //    by shuffles and their first lanes add to the warp's own bins without
@@ -107,6 +111,31 @@ __device__ __forceinline__ df df_of2(float2 v) { return df{v.x, v.y}; }
 __device__ __forceinline__ df df_scale(df a, float p) {  // by a power of two
   return df{__fmul_rn(a.hi, p), __fmul_rn(a.lo, p)};
 }
+// hi + lo + c: a pair and a float that takes what a pair rounds away
+struct tf {
+  float hi, lo, c;
+};
+__device__ __forceinline__ tf tf_add(tf a, tf b) {
+  const df s = two_sum(a.hi, b.hi), t = two_sum(a.lo, b.lo), m = two_sum(s.lo, t.hi);
+  const df r = fast_two_sum(s.hi, m.hi);
+  return tf{r.hi, r.lo, __fadd_rn(__fadd_rn(a.c, b.c), __fadd_rn(m.lo, t.lo))};
+}
+__device__ __forceinline__ tf tf_scale(tf a, float p) {  // by a power of two
+  return tf{__fmul_rn(a.hi, p), __fmul_rn(a.lo, p), __fmul_rn(a.c, p)};
+}
+__device__ __forceinline__ tf tf_shfl_down(tf a, int o) {
+  return tf{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o),
+            __shfl_down_sync(0xffffffffu, a.c, o)};
+}
+// the root of an integer q = s^2 (1 + d) < 2^24 from its FP32 root s: two
+// corrections, whose remainders are exact (errors of order d^2, then d^3)
+__device__ __forceinline__ tf tf_sqrt(float q, float s) {
+  const float d2 = 2.0f * s;
+  const float r = __fmaf_rn(-s, s, q), c = __fdiv_rn(r, d2);
+  const float e = __fdiv_rn(__fmaf_rn(-c, c, __fmaf_rn(-d2, c, r)), d2);
+  const df h = fast_two_sum(s, c);
+  return tf{h.hi, h.lo, e};
+}
 __device__ __forceinline__ df df_div(df a, df b) {
   const float q = __fdiv_rn(a.hi, b.hi);
   const df r = df_add(a, df_mul(df{-q, 0.0f}, b));
@@ -117,10 +146,10 @@ __device__ __forceinline__ df df_shfl_down(df a, int o) {
 }
 
 constexpr int PK_NT = 256, PK_WARPS = PK_NT / 32;
-// shared floats of a warp: per bin the count, sum |k|, sum P (and sum C1/C2)
-// as pairs; with aliases each lane's x factors
+// shared floats of a warp: per bin the count, sum |k| (three floats), sum P
+// (and sum C1/C2) as pairs; with aliases each lane's x factors
 __host__ __device__ constexpr int pk_warp_floats(int n_bins, int m) {
-  return n_bins * (m ? 7 : 5) + (m ? 2 * (2 * m + 1) * 32 : 0);
+  return n_bins * (m ? 8 : 6) + (m ? 2 * (2 * m + 1) * 32 : 0);
 }
 
 template <int m>
@@ -130,7 +159,7 @@ __global__ void __launch_bounds__(PK_NT) k_pk_modes(const float2* __restrict__ d
                                                     const double* __restrict__ nu,
                                                     double* __restrict__ acc) {
   constexpr unsigned FULL = 0xffffffffu;
-  constexpr int NA = 2 * m + 1, NF = m ? 7 : 5;
+  constexpr int NA = 2 * m + 1, NF = m ? 8 : 6;
   extern __shared__ float sm[];
   const PkAxes T = pk_axes(const_cast<void*>(tab), n);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -176,13 +205,14 @@ __global__ void __launch_bounds__(PK_NT) k_pk_modes(const float2* __restrict__ d
       const int key = in ? r - 1 : -1;
       if (!__any_sync(FULL, in)) continue;
       float cnt = 0.0f;
-      df K{0.0f, 0.0f}, A{0.0f, 0.0f}, C{0.0f, 0.0f};
+      tf K{0.0f, 0.0f, 0.0f};
+      df A{0.0f, 0.0f}, C{0.0f, 0.0f};
       if (in) {
         const float w = (ix == 0 || 2 * ix == n) ? 1.0f : 2.0f;
         cnt = w * (float)(ny * nz);
-        // sqrt(m2) = sq + (m2 - sq^2) / (2 sq); m2 <= 3 (n/2)^2 < 2^24 is exact
-        // in FP32 up to n = 4729, past any mesh that fits in memory
-        K = fast_two_sum(sq, __fdiv_rn(__fmaf_rn(-sq, sq, (float)m2), 2.0f * sq));
+        // (m2 <= 3 (n/2)^2 < 2^24 is exact in FP32 up to n = 4729, past any mesh
+        // that fits in memory)
+        K = tf_sqrt((float)m2, sq);
         df o{0.0f, 0.0f};
         for (int q = 0; q < 4; ++q) {
           if ((q & 1) >= ny || (q >> 1) >= nz) continue;
@@ -228,7 +258,7 @@ __global__ void __launch_bounds__(PK_NT) k_pk_modes(const float2* __restrict__ d
           C = df_scale(df_div(df_mul(cyz, df_of2(T.c1[ix])), c2), cnt);
         }
         A = df_scale(A, w);
-        K = df_scale(K, cnt);
+        K = tf_scale(K, cnt);
       }
       // sum each run of one bin onto its first lane
       const int prev = __shfl_up_sync(FULL, key, 1);
@@ -240,12 +270,13 @@ __global__ void __launch_bounds__(PK_NT) k_pk_modes(const float2* __restrict__ d
         const bool add = lane + o <= rend;
         if (!__any_sync(FULL, add)) break;
         const float ct = __shfl_down_sync(FULL, cnt, o);
-        const df kt = df_shfl_down(K, o), at = df_shfl_down(A, o);
+        const tf kt = tf_shfl_down(K, o);
+        const df at = df_shfl_down(A, o);
         df cc{0.0f, 0.0f};
         if (m) cc = df_shfl_down(C, o);
         if (add) {
           cnt += ct;
-          K = df_add(K, kt);
+          K = tf_add(K, kt);
           A = df_add(A, at);
           if (m) C = df_add(C, cc);
         }
@@ -253,15 +284,17 @@ __global__ void __launch_bounds__(PK_NT) k_pk_modes(const float2* __restrict__ d
       if (in && !same) {  // the runs of a row have different bins
         float* e = bins + key * NF;
         e[0] += cnt;
-        const df k = df_add(df{e[1], e[2]}, K), a = df_add(df{e[3], e[4]}, A);
+        const tf k = tf_add(tf{e[1], e[2], e[3]}, K);
+        const df a = df_add(df{e[4], e[5]}, A);
         e[1] = k.hi;
         e[2] = k.lo;
-        e[3] = a.hi;
-        e[4] = a.lo;
+        e[3] = k.c;
+        e[4] = a.hi;
+        e[5] = a.lo;
         if (m) {
-          const df c = df_add(df{e[5], e[6]}, C);
-          e[5] = c.hi;
-          e[6] = c.lo;
+          const df c = df_add(df{e[6], e[7]}, C);
+          e[6] = c.hi;
+          e[7] = c.lo;
         }
       }
       __syncwarp();
@@ -276,9 +309,9 @@ __global__ void __launch_bounds__(PK_NT) k_pk_modes(const float2* __restrict__ d
       const float* e = sm + (size_t)w * pk_warp_floats(n_bins, m) + b * NF;
       if (e[0] == 0.0f) continue;
       c += (double)e[0];
-      k += (double)e[1] + (double)e[2];
-      p += (double)e[3] + (double)e[4];
-      if (m) q += (double)e[5] + (double)e[6];
+      k += (double)e[1] + ((double)e[2] + (double)e[3]);
+      p += (double)e[4] + (double)e[5];
+      if (m) q += (double)e[6] + (double)e[7];
     }
     if (c == 0.0) continue;
     atomicAdd(&acc[3 * b + 0], c);
