@@ -246,8 +246,8 @@ pm_status pm_potential(pm_ctx* ctx, const double* delta_dev, double a, int32_t b
  * prod_d sinc^2(k_d h/2), minus the shot noise L^3/n (Sec. 2.4: power
  * spectrum with discreteness correction).  Linear bins of width
  * k_f = 2 pi/L: bin b holds |k|/k_f in [b+.5, b+1.5).  Host outputs of n_bins
- * entries: mean |k| (h/Mpc), mean P ((Mpc/h)^3), number of modes.  Allocates
- * its own scratch; synchronises stream.  subtract_shot = 0 omits the L^3/n
+ * entries: mean |k| (h/Mpc), mean P ((Mpc/h)^3), number of modes.  Work
+ * space comes from the library's pool (pm_release_work); synchronises stream.  subtract_shot = 0 omits the L^3/n
  * term (lattice-based particle sets). */
 pm_status pm_power_spectrum(const float* pos4_dev, int64_t n, double box,
                             int32_t n_mesh, int32_t n_bins, int32_t subtract_shot,
@@ -309,11 +309,18 @@ pm_status pm_deposit_tsc(float* pos4_dev, const float* mom4_dev, int64_t n,
  * mom4_out (device, n float4 each, caller-owned, not overlapping the inputs)
  * receive the records in that order; mom4_dev may be NULL (then mom4_out is
  * not written).  An order of the data only: the deposit of the particles is
- * unchanged (its integer sums do not depend on the order).  Work space is
- * allocated and freed inside the call.  n_mesh in [1, 1024], n in
+ * unchanged (its integer sums do not depend on the order).  Work space comes
+ * from the library's pool (pm_release_work).  n_mesh in [1, 1024], n in
  * [0, 2^31).  Synchronises stream. */
 pm_status pm_sort_particles(const float* pos4_dev, const float* mom4_dev, int64_t n,
                             int32_t n_mesh, float* pos4_out, float* mom4_out, void* stream);
+
+/* The work space of pm_sort_particles and of the power spectra stays with the
+ * library between calls, at most 1 GiB a device, with up to four FFT plans.
+ * It goes back to the device when an allocation of the library is refused,
+ * and by this call, for a program that needs the memory itself; the next
+ * call takes it anew.  Synchronises the current device.  Errors: PM_ECUDA. */
+pm_status pm_release_work(void);
 
 typedef struct {
   int32_t step;          /* steps completed */

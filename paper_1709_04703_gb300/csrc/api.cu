@@ -131,6 +131,178 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// Work space of the calls without a context (particle order, spectra): stream
+// ordered allocations from one memory pool per device that the library owns.
+// cudaMalloc and cudaFree cost 40 us each here, 0.3 to 0.6 ms a call.  The
+// pool keeps at most KEEP bytes between calls; they go back when an
+// allocation of the library is refused (with_room) and by pm_release_work.
+// Allocations follow the stream they are made on, so any threads and streams
+// may use it at once.
+struct WorkPool {
+  static constexpr unsigned long long KEEP = 1ull << 30;
+  std::mutex mu;
+  std::vector<std::pair<int, cudaMemPool_t>> pools;
+  cudaMemPool_t pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    for (auto& p : pools)
+      if (p.first == dev) return p.second;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    unsigned long long keep = KEEP;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return nullptr;
+    }
+    pools.push_back({dev, p});
+    return p;
+  }
+  // give the idle memory of this device's pool back
+  cudaError_t trim() {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    for (auto& p : pools)
+      if (p.first == dev) return cudaMemPoolTrimTo(p.second, 0);
+    return cudaSuccess;
+  }
+};
+WorkPool& work_pool() {
+  static WorkPool* w = new WorkPool();  // (not destroyed: the driver may be gone by then)
+  return *w;
+}
+void drop_idle_plans();
+// What idles between calls on this device goes back to it.  The pool only
+// gives up memory whose cudaFreeAsync is known to have run (a call queues its
+// frees after its last synchronisation), hence the wait.
+cudaError_t release_idle_work() {
+  drop_idle_plans();
+  const cudaError_t e = cudaDeviceSynchronize();
+  return e != cudaSuccess ? e : work_pool().trim();
+}
+// Host-side fault injection for tests: PM_FAULT_FULL=1 refuses the first
+// attempt of every device allocation as a full device would, PM_FAULT_FULL=2
+// the second one too.
+int fault_full() {
+  const char* f = getenv("PM_FAULT_FULL");
+  return f ? atoi(f) : 0;
+}
+// Run `attempt`, which takes device memory; where it is refused, once more
+// after the idle work space has gone back.  Leaves no error behind for a
+// later cudaGetLastError.
+template <class F>
+cudaError_t with_room(F&& attempt, int full = fault_full()) {
+  cudaError_t e = full >= 1 ? cudaErrorMemoryAllocation : attempt();
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (release_idle_work() == cudaSuccess && full < 2) e = attempt();
+  }
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+// one call's allocations, freed on its stream when it ends
+struct WorkSpace {
+  cudaStream_t st;
+  std::vector<void*> ptrs;
+  const int full = fault_full();  // (once a call: half a microsecond)
+  explicit WorkSpace(cudaStream_t s) : st(s) {}
+  WorkSpace(const WorkSpace&) = delete;
+  ~WorkSpace() {
+    for (void* p : ptrs) cudaFreeAsync(p, st);
+  }
+  bool get(void** out, size_t bytes) {
+    cudaMemPool_t pool = work_pool().pool();
+    if (!pool) {
+      cudaGetLastError();
+      return false;
+    }
+    const cudaError_t e = with_room(
+        [&] { return cudaMallocFromPoolAsync(out, bytes ? bytes : 1, pool, st); }, full);
+    if (e != cudaSuccess) {
+      *out = nullptr;
+      return false;
+    }
+    ptrs.push_back(*out);
+    return true;
+  }
+};
+// FFT plans of the spectra, kept between calls: making one takes about as
+// long as a 256^3 transform and its binning.  A plan belongs to one call at a
+// time (take / put under a lock, any thread, any device); at most MAX idle
+// ones stay, the oldest is destroyed.  Plans hold no work area (the call's
+// work space gives it).
+struct PlanCache {
+  static constexpr size_t MAX = 4;
+  struct Plan {
+    int dev = 0, n = 0;
+    cufftHandle h = 0;
+    size_t work = 0;
+    bool ok = false;
+  };
+  std::mutex mu;
+  std::vector<Plan> idle;
+  Plan take(int n) {
+    Plan p;
+    if (cudaGetDevice(&p.dev) != cudaSuccess) return p;
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      for (size_t q = 0; q < idle.size(); ++q)
+        if (idle[q].dev == p.dev && idle[q].n == n) {
+          p = idle[q];
+          idle.erase(idle.begin() + q);
+          return p;
+        }
+    }
+    p.n = n;
+    p.ok = with_room([&] {
+             if (cufftCreate(&p.h) != CUFFT_SUCCESS) return cudaErrorMemoryAllocation;
+             if (cufftSetAutoAllocation(p.h, 0) == CUFFT_SUCCESS &&
+                 cufftMakePlan3d(p.h, n, n, n, CUFFT_R2C, &p.work) == CUFFT_SUCCESS)
+               return cudaSuccess;
+             cufftDestroy(p.h);
+             return cudaErrorMemoryAllocation;  // (or another failure, which stays one)
+           }) == cudaSuccess;
+    return p;
+  }
+  void clear() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::vector<Plan> mine;
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      for (size_t q = idle.size(); q-- > 0;)
+        if (idle[q].dev == dev) {
+          mine.push_back(idle[q]);
+          idle.erase(idle.begin() + q);
+        }
+    }
+    for (const Plan& p : mine) cufftDestroy(p.h);
+  }
+  void put(const Plan& p) {
+    Plan old;
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      idle.push_back(p);
+      if (idle.size() > MAX) {
+        old = idle.front();
+        idle.erase(idle.begin());
+      }
+    }
+    if (old.ok) cufftDestroy(old.h);
+  }
+};
+PlanCache& plan_cache() {
+  static PlanCache* c = new PlanCache();  // (not destroyed: the driver may be gone by then)
+  return *c;
+}
+void drop_idle_plans() { plan_cache().clear(); }
+
 }  // namespace
 
 // a pair of profiling events around a launch group of one kernel class
@@ -800,7 +972,7 @@ pm_status vcycle_run(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
     }
     if (e != cudaSuccess)
       return fail(ctx, PM_ECUDA, std::string("V-cycle capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&g.exec, graph, 0);
+    e = with_room([&] { return cudaGraphInstantiate(&g.exec, graph, 0); });
     cudaGraphDestroy(graph);
     if (e != cudaSuccess)
       return fail(ctx, PM_ECUDA, std::string("V-cycle instantiate: ") + cudaGetErrorString(e));
@@ -1248,78 +1420,6 @@ pm_status record_to(pm_ctx* ctx, double R, double a_cross) {
   return PM_OK;
 }
 
-// Work space of the calls without a context (particle order, spectra): stream
-// ordered allocations from one memory pool per device that the library owns.
-// cudaMalloc and cudaFree cost 40 us each here, 0.3 to 0.6 ms a call.  The
-// pool keeps at most KEEP bytes between calls and gives them back when an
-// allocation of the library fails; allocations follow the stream they are
-// made on, so any threads and streams may use it at once.
-struct WorkPool {
-  static constexpr unsigned long long KEEP = 1ull << 30;
-  std::mutex mu;
-  std::vector<std::pair<int, cudaMemPool_t>> pools;
-  cudaMemPool_t pool() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-    std::lock_guard<std::mutex> lk(mu);
-    for (auto& p : pools)
-      if (p.first == dev) return p.second;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t p = nullptr;
-    unsigned long long keep = KEEP;
-    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
-    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-      cudaMemPoolDestroy(p);
-      return nullptr;
-    }
-    pools.push_back({dev, p});
-    return p;
-  }
-  // give the idle memory of this device's pool back; false if there is none
-  bool trim() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    std::lock_guard<std::mutex> lk(mu);
-    for (auto& p : pools)
-      if (p.first == dev) return cudaMemPoolTrimTo(p.second, 0) == cudaSuccess;
-    return false;
-  }
-};
-WorkPool& work_pool() {
-  static WorkPool* w = new WorkPool();  // (not destroyed: the driver may be gone by then)
-  return *w;
-}
-// one call's allocations, freed on its stream when it ends
-struct WorkSpace {
-  cudaStream_t st;
-  std::vector<void*> ptrs;
-  explicit WorkSpace(cudaStream_t s) : st(s) {}
-  WorkSpace(const WorkSpace&) = delete;
-  ~WorkSpace() {
-    for (void* p : ptrs) cudaFreeAsync(p, st);
-  }
-  bool get(void** out, size_t bytes) {
-    cudaMemPool_t pool = work_pool().pool();
-    if (!pool) return false;
-    cudaError_t e = cudaMallocFromPoolAsync(out, bytes ? bytes : 1, pool, st);
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      cudaStreamSynchronize(st);
-      if (work_pool().trim()) e = cudaMallocFromPoolAsync(out, bytes ? bytes : 1, pool, st);
-    }
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      *out = nullptr;
-      return false;
-    }
-    ptrs.push_back(*out);
-    return true;
-  }
-};
-
 pm_status alloc(pm_ctx* ctx, void** p, size_t bytes) {
   // host-side fault injection for tests: PM_FAULT_ALLOC=k makes the k-th
   // device allocation of a context fail as if the device were full
@@ -1328,19 +1428,19 @@ pm_status alloc(pm_ctx* ctx, void** p, size_t bytes) {
     *p = nullptr;
     return fail(ctx, PM_ENOMEM, "cudaMalloc: allocation failure injected (PM_FAULT_ALLOC)");
   }
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation && work_pool().trim()) {
-    cudaGetLastError();
-    e = cudaMalloc(p, bytes);
-  }
-  if (e != cudaSuccess) {
-    *p = nullptr;
+  cudaError_t e = dev_malloc(p, bytes);
+  if (e != cudaSuccess)
     return fail(ctx, PM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  }
   return PM_OK;
 }
 
 }  // namespace
+
+cudaError_t pm::dev_malloc(void** p, size_t bytes) {
+  const cudaError_t e = with_room([&] { return cudaMalloc(p, bytes); });
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
 
 // Keep rule of pm_shrink for callers outside a context (see noalloc.cu).
 double pm::shrink_radius_cells(int n, double box, double om, double ol, double buffer,
@@ -1957,7 +2057,7 @@ pm_status deposit_any(bool tsc, const char* who, float* pos4_dev, const float* m
     return fail(nullptr, PM_EINVAL, std::string(who) + ": periodic needs the whole mesh");
   cudaStream_t st = (cudaStream_t)stream;
   unsigned long long* esc = nullptr;
-  CK(cudaMallocAsync((void**)&esc, sizeof(unsigned long long), st));
+  CK(with_room([&] { return cudaMallocAsync((void**)&esc, sizeof(unsigned long long), st); }));
   CK(cudaMemsetAsync(esc, 0, sizeof(unsigned long long), st));
   if (tsc)
     launch_drift_deposit_tsc(st, n, (float4*)pos4_dev, (const float4*)mom4_dev, drift_coef,
@@ -1992,6 +2092,13 @@ pm_status pm_deposit_tsc(float* pos4_dev, const float* mom4_dev, int64_t n, floa
                          int64_t* rho_dev, int64_t* escaped_out, void* stream) {
   return deposit_any(true, "pm_deposit_tsc", pos4_dev, mom4_dev, n, drift_coef, n_mesh, lo,
                      side, periodic, rho_dev, escaped_out, stream);
+}
+
+pm_status pm_release_work(void) {
+  const cudaError_t e = release_idle_work();
+  if (e == cudaSuccess) return PM_OK;
+  cudaGetLastError();
+  return fail(nullptr, PM_ECUDA, std::string("pm_release_work: ") + cudaGetErrorString(e));
 }
 
 pm_status pm_sort_particles(const float* pos4_dev, const float* mom4_dev, int64_t n,
@@ -2032,61 +2139,6 @@ pm_status pm_sort_particles(const float* pos4_dev, const float* mom4_dev, int64_
 }
 
 namespace {
-// FFT plans of the spectra, kept between calls: making one takes about as
-// long as a 256^3 transform and its binning.  A plan belongs to one call at a
-// time (take / put under a lock, any thread, any device); at most MAX idle
-// ones stay, the oldest is destroyed.  Plans hold no work area (the call's
-// work space gives it).
-struct PlanCache {
-  static constexpr size_t MAX = 4;
-  struct Plan {
-    int dev = 0, n = 0;
-    cufftHandle h = 0;
-    size_t work = 0;
-    bool ok = false;
-  };
-  std::mutex mu;
-  std::vector<Plan> idle;
-  Plan take(int n) {
-    Plan p;
-    if (cudaGetDevice(&p.dev) != cudaSuccess) return p;
-    {
-      std::lock_guard<std::mutex> lk(mu);
-      for (size_t q = 0; q < idle.size(); ++q)
-        if (idle[q].dev == p.dev && idle[q].n == n) {
-          p = idle[q];
-          idle.erase(idle.begin() + q);
-          return p;
-        }
-    }
-    p.n = n;
-    if (cufftCreate(&p.h) != CUFFT_SUCCESS) return p;
-    if (cufftSetAutoAllocation(p.h, 0) != CUFFT_SUCCESS ||
-        cufftMakePlan3d(p.h, n, n, n, CUFFT_R2C, &p.work) != CUFFT_SUCCESS) {
-      cufftDestroy(p.h);
-      return p;
-    }
-    p.ok = true;
-    return p;
-  }
-  void put(const Plan& p) {
-    Plan old;
-    {
-      std::lock_guard<std::mutex> lk(mu);
-      idle.push_back(p);
-      if (idle.size() > MAX) {
-        old = idle.front();
-        idle.erase(idle.begin());
-      }
-    }
-    if (old.ok) cufftDestroy(old.h);
-  }
-};
-PlanCache& plan_cache() {
-  static PlanCache* c = new PlanCache();  // (not destroyed: the driver may be gone by then)
-  return *c;
-}
-
 // Device work space of one P(k) call: CIC counts, contrast, its R2C
 // transform, bin accumulators (3 per bin + the escape counter), slopes and
 // the window's per-axis tables.
@@ -2732,8 +2784,8 @@ pm_status bfail(pm_batch* b, pm_status code, const std::string& msg) {
 
 pm_status tab_alloc(pm_batch* B, BTab& t, size_t desc_size) {
   t.desc_size = desc_size;
-  if (cudaMalloc(&t.d_desc, desc_size * MAX_MEMBERS) != cudaSuccess ||
-      cudaMalloc((void**)&t.d_tab, sizeof(BTable)) != cudaSuccess ||
+  if (dev_malloc(&t.d_desc, desc_size * MAX_MEMBERS) != cudaSuccess ||
+      dev_malloc((void**)&t.d_tab, sizeof(BTable)) != cudaSuccess ||
       cudaMallocHost(&t.h_desc, desc_size * MAX_MEMBERS) != cudaSuccess ||
       cudaMallocHost((void**)&t.h_tab, sizeof(BTable)) != cudaSuccess)
     return bfail(B, PM_ENOMEM, "pm_batch: table allocation failed");
@@ -3081,7 +3133,8 @@ pm_status build_solve_graph(pm_batch* B) {
   g_launches.fetch_sub(g_launches.load() - l0);
   B->loop_kernels = lb1 - lb0;
   if (e == cudaSuccess) e = e2;
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&B->sgraph, done, 0);
+  if (e == cudaSuccess)
+    e = with_room([&] { return cudaGraphInstantiate(&B->sgraph, done, 0); });
   if (done) cudaGraphDestroy(done);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -3097,7 +3150,7 @@ pm_status upload_solve_slots(pm_batch* B) {
     cudaFree(B->d_slots);
     B->d_slots = nullptr;
   }
-  if (!B->d_slots && cudaMalloc((void**)&B->d_slots, sizeof(SolveSlot) * n) != cudaSuccess)
+  if (!B->d_slots && dev_malloc((void**)&B->d_slots, sizeof(SolveSlot) * n) != cudaSuccess)
     return bfail(B, PM_ENOMEM, "pm_batch: solve slot allocation failed");
   B->n_slots_dev = n;
   std::vector<SolveSlot> v;
@@ -3339,10 +3392,10 @@ pm_status pm_batch_init(int32_t n_real, const pm_config* cfgs, const float* cons
     B->ctx.push_back(c);
   }
   pm_status st = PM_OK;
-  if (cudaMalloc((void**)&B->d_active, sizeof(int) * MAX_REAL) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_res, sizeof(BatchResult)) != cudaSuccess ||
+  if (dev_malloc((void**)&B->d_active, sizeof(int) * MAX_REAL) != cudaSuccess ||
+      dev_malloc((void**)&B->d_res, sizeof(BatchResult)) != cudaSuccess ||
       cudaMallocHost((void**)&B->h_res, sizeof(BatchResult)) != cudaSuccess ||
-      cudaMalloc((void**)&B->d_maxv, sizeof(int) * MAX_REAL) != cudaSuccess)
+      dev_malloc((void**)&B->d_maxv, sizeof(int) * MAX_REAL) != cudaSuccess)
     st = bfail(B, PM_ENOMEM, "pm_batch_init: allocation failed");
   if (st == PM_OK) {
     // per-realisation tolerances (fixed for the run)
@@ -3795,7 +3848,7 @@ extern "C" pm_status pm_selftest_wait(int32_t arrive, int64_t polls, void* strea
     return fail(nullptr, PM_EINVAL, "pm_selftest_wait: polls in [1, 1e9]");
   cudaStream_t st = (cudaStream_t)stream;
   int* flag = nullptr;
-  if (cudaMallocAsync((void**)&flag, sizeof(int), st) != cudaSuccess)
+  if (with_room([&] { return cudaMallocAsync((void**)&flag, sizeof(int), st); }) != cudaSuccess)
     return fail(nullptr, PM_ENOMEM, "pm_selftest_wait: cudaMallocAsync");
   cudaMemsetAsync(flag, 0, sizeof(int), st);
   launch_wait_selftest(st, arrive ? 1 : 0, polls, flag);
@@ -3816,7 +3869,7 @@ extern "C" pm_status pm_nn_gemm_bf16(const void* A, const void* B, float* C, int
     return fail(nullptr, PM_EINVAL, "pm_nn_gemm_bf16: M % 128, K % 64, N in {16,32,64,128}");
   cudaStream_t st = (cudaStream_t)stream;
   int* err = nullptr;
-  if (cudaMallocAsync((void**)&err, sizeof(int), st) != cudaSuccess)
+  if (with_room([&] { return cudaMallocAsync((void**)&err, sizeof(int), st); }) != cudaSuccess)
     return fail(nullptr, PM_ENOMEM, "pm_nn_gemm_bf16: cudaMallocAsync");
   cudaMemsetAsync(err, 0, sizeof(int), st);
   launch_gemm_tc(st, A, B, C, M, N, K, err);

@@ -109,7 +109,7 @@ pm_status ensure_shape(pm_guess* g, int B, int S) {
   g->act.assign(SLOT_N, Buf());
   auto alloc = [&](int slot, long long elems) -> bool {
     g->act[slot].bytes = (size_t)elems * 2;
-    return cudaMalloc(&g->act[slot].p, g->act[slot].bytes) == cudaSuccess;
+    return dev_malloc(&g->act[slot].p, g->act[slot].bytes) == cudaSuccess;
   };
   bool ok = alloc(SLOT_X, vox(B, S, 0) * 8);
   long long gmax = vox(B, S, 0) * 8;
@@ -125,9 +125,9 @@ pm_status ensure_shape(pm_guess* g, int B, int S) {
     gmax = std::max(gmax, vox(B, S, l) * c);
   }
   ok = ok && alloc(SLOT_G0, gmax) && alloc(SLOT_G1, gmax) && alloc(SLOT_G2, gmax);
-  ok = ok && cudaMalloc((void**)&g->y, sizeof(float) * need) == cudaSuccess;
-  ok = ok && cudaMalloc((void**)&g->ld, sizeof(float) * need) == cudaSuccess;
-  ok = ok && cudaMalloc((void**)&g->lq, sizeof(float) * need) == cudaSuccess;
+  ok = ok && dev_malloc((void**)&g->y, sizeof(float) * need) == cudaSuccess;
+  ok = ok && dev_malloc((void**)&g->ld, sizeof(float) * need) == cudaSuccess;
+  ok = ok && dev_malloc((void**)&g->lq, sizeof(float) * need) == cudaSuccess;
   if (!ok) return gfail(g, PM_ENOMEM, "guess: activation allocation failed");
   g->cap_vox = need;
   return PM_OK;
@@ -147,11 +147,8 @@ void pack_all(pm_guess* g) {
 void pack_bwd(pm_guess* g) {
   for (auto& c : g->conv) {
     if (c.fast_tt && !c.wft &&
-        cudaMalloc(&c.wft, (size_t)c.nt * conv_fast_kf(round_up(c.cout, 8)) * 2) != cudaSuccess) {
-      cudaGetLastError();
-      c.wft = nullptr;
+        dev_malloc(&c.wft, (size_t)c.nt * conv_fast_kf(round_up(c.cout, 8)) * 2) != cudaSuccess)
       c.fast_tt = 0;
-    }
     if (c.fast_tt) launch_pack_wf(g->st, g->w + c.w_off, c.cin, c.cout, c.nt, true, c.wft);
   }
   g->packed_t = true;
@@ -380,29 +377,29 @@ pm_status pm_guess_create(int32_t levels, void* stream, pm_guess** out) {
   add(8, 8, 0);
   bool ok = true;
   for (auto& c : g->conv) {
-    ok = ok && cudaMalloc(&c.wp, (size_t)c.n * c.kp * 2) == cudaSuccess;
-    ok = ok && cudaMalloc(&c.wt, (size_t)c.nt * c.kpt * 2) == cudaSuccess;
+    ok = ok && dev_malloc(&c.wp, (size_t)c.n * c.kp * 2) == cudaSuccess;
+    ok = ok && dev_malloc(&c.wt, (size_t)c.nt * c.kpt * 2) == cudaSuccess;
     // the staged-input kernel wherever its block and weights fit (forward at
     // 256^3: 8.7 ms against 12.4 ms with every layer on the gathered tile);
     // PM_NN_GATHER keeps the gathered tile everywhere
     c.fast_t = getenv("PM_NN_GATHER") ? 0 : conv_fast_side(c.cin, c.cout);
     if (c.fast_t)
-      ok = ok && cudaMalloc(&c.wf, (size_t)c.n * conv_fast_kf(c.cin) * 2) == cudaSuccess;
+      ok = ok && dev_malloc(&c.wf, (size_t)c.n * conv_fast_kf(c.cin) * 2) == cudaSuccess;
     // the input gradient likewise (the five of a 4-level net at 96^3 that
     // fit: 490 us on the gathered tile, 286 staged)
     c.fast_tt = getenv("PM_NN_GATHER") ? 0 : conv_fast_side(round_up(c.cout, 8), c.cin);
   }
   size_t pb = sizeof(float) * g->n_params;
-  ok = ok && cudaMalloc((void**)&g->w, pb) == cudaSuccess &&
-       cudaMalloc((void**)&g->g, pb) == cudaSuccess &&
-       cudaMalloc((void**)&g->m, pb) == cudaSuccess &&
-       cudaMalloc((void**)&g->v, pb) == cudaSuccess &&
-       cudaMalloc((void**)&g->scale_in, sizeof(float) * 4096) == cudaSuccess &&
-       cudaMalloc((void**)&g->scale_out, sizeof(float) * 4096) == cudaSuccess &&
-       cudaMalloc((void**)&g->tscale, sizeof(float) * 4096) == cudaSuccess &&
-       cudaMalloc((void**)&g->rms_part, sizeof(double) * 4096 * RMS_BLOCKS) == cudaSuccess &&
-       cudaMalloc((void**)&g->loss, sizeof(double)) == cudaSuccess &&
-       cudaMalloc((void**)&g->err, sizeof(int)) == cudaSuccess;
+  ok = ok && dev_malloc((void**)&g->w, pb) == cudaSuccess &&
+       dev_malloc((void**)&g->g, pb) == cudaSuccess &&
+       dev_malloc((void**)&g->m, pb) == cudaSuccess &&
+       dev_malloc((void**)&g->v, pb) == cudaSuccess &&
+       dev_malloc((void**)&g->scale_in, sizeof(float) * 4096) == cudaSuccess &&
+       dev_malloc((void**)&g->scale_out, sizeof(float) * 4096) == cudaSuccess &&
+       dev_malloc((void**)&g->tscale, sizeof(float) * 4096) == cudaSuccess &&
+       dev_malloc((void**)&g->rms_part, sizeof(double) * 4096 * RMS_BLOCKS) == cudaSuccess &&
+       dev_malloc((void**)&g->loss, sizeof(double)) == cudaSuccess &&
+       dev_malloc((void**)&g->err, sizeof(int)) == cudaSuccess;
   if (!ok) {
     pm_guess_destroy(g);
     return PM_ENOMEM;

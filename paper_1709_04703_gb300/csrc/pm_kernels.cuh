@@ -8,6 +8,10 @@ namespace pm {
 // Counts kernel launches made by the library (pm_launch_count).
 void note_launch();
 
+// cudaMalloc for the library's objects; refused, it is tried again after the
+// library's idle work space has gone back (api.cu).  *p is NULL on an error.
+cudaError_t dev_malloc(void** p, size_t bytes);
+
 // Launch with the programmatic-stream-serialization attribute (the kernel
 // starts with pdl_wait); a normal launch when PM_NO_PDL is set.
 bool pdl_enabled();

@@ -412,6 +412,12 @@ def sort_particles(pos4_dev, mom4_dev, n_mesh):
     return po, mo
 
 
+def release_work():
+    """Give the device memory back that sort_particles and the spectra keep
+    between calls (pm_release_work)."""
+    L.check(L.load().pm_release_work(), None)
+
+
 def power_spectrum(pos4_dev, box, n_mesh, n_bins, subtract_shot=True):
     """P(k) of device float4 particles (positions in cells of n_mesh)."""
     lib = L.load()

@@ -62,3 +62,113 @@ def test_plans_and_work_space_across_sizes_streams_and_threads():
     for t in ts:
         t.join()
     assert not bad, bad[0]
+
+
+# --- the idle work space goes back ---------------------------------------
+
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _hold(points):
+    """Let the pool keep a 256^3 spectrum's arrays; the bytes it holds at
+    least (counts, contrast and modes)."""
+    from paper_1709_04703_gb300.sim import power_spectrum
+    power_spectrum(points, 100.0, 256, 4)
+    return 256**3 * (8 + 4 + 4)
+
+
+def _box():
+    return ics.random_particles(4096, 32, 7)
+
+
+def _sim():
+    from paper_1709_04703_gb300.sim import Sim
+    return Sim(*_box(), 32, 500.0, 0.1, 1.0, 10)
+
+
+def _batch():
+    from paper_1709_04703_gb300.sim import Batch
+    return Batch([dict(zip(("pos", "mom", "ids"), _box()), n_mesh=32, box=500.0)], 0.1, 1.0, 10)
+
+
+def _net():
+    from paper_1709_04703_gb300.guess import GuessNet
+    return GuessNet(levels=3, seed=3)
+
+
+def _field():
+    return torch.randn((1, 16, 16, 16), generator=torch.Generator().manual_seed(1)).cuda()
+
+
+def _stepped(run):
+    run.step(1)
+    p = run.particles(0) if hasattr(run, "R") else run.particles()
+    return [p[0], p[1]]
+
+
+# what is made before the refusals begin, and the call that meets them
+CALLS = {
+    "context": (lambda: None, lambda _: _stepped(_sim())),
+    "step": (_sim, _stepped),
+    "batch": (lambda: None, lambda _: _stepped(_batch())),
+    "batch_step": (_batch, _stepped),
+    "network": (lambda: None, lambda _: [_net().forward(_field(), 1).cpu().numpy()]),
+    "forward": (_net, lambda net: [net.forward(_field(), 1).cpu().numpy()]),
+    "gradient": (_net, lambda net: [net.loss_grad(_field(), 2 * _field(), 1, 0), net.grad()]),
+    "spectrum": (lambda: _points(24, 500, 2), lambda p: _spectrum(p[0])),
+    "order": (lambda: _points(24, 500, 2), lambda p: _order(*p)),
+    "deposit": (lambda: _points(24, 500, 2), lambda p: _deposit(p[0])),
+}
+
+
+def _spectrum(p4):
+    from paper_1709_04703_gb300.sim import power_spectrum
+    return list(power_spectrum(p4, 100.0, 24, 12))
+
+
+def _order(p4, m4):
+    from paper_1709_04703_gb300.sim import sort_particles
+    return [t.view(torch.int32).cpu().numpy() for t in sort_particles(p4, m4, 24)]
+
+
+def _deposit(p4):
+    from paper_1709_04703_gb300.sim import deposit
+    return [deposit(p4, 24)[0].cpu().numpy()]
+
+
+@pytest.mark.parametrize("call", list(CALLS))
+def test_refused_allocations_get_the_idle_work_space(call, monkeypatch):
+    """PM_FAULT_FULL=1 refuses the first attempt of every device allocation
+    as a full device would.  Each call that allocates then has the pool's idle
+    memory given back, right after the call that left it there, tries again,
+    and gives the results of a call that met no refusal."""
+    make, act = CALLS[call]
+    want = act(make())
+    points, _ = _points(256, 1000, 1)
+    state = make()
+    held = _hold(points)
+    before = _free()
+    _hold(points)  # (the frees of this call are still queued behind it)
+    monkeypatch.setenv("PM_FAULT_FULL", "1")
+    got = act(state)
+    monkeypatch.delenv("PM_FAULT_FULL")
+    # (what the call keeps itself is a few MB)
+    assert _free() - before > held // 2
+    for a, b in zip(got, want):
+        np.testing.assert_allclose(a, b, rtol=1e-4 if call == "gradient" else 1e-6,
+                                   atol=1e-6 * np.abs(b).max() if call == "gradient" else 0)
+
+
+def test_release_work_gives_the_memory_back():
+    from paper_1709_04703_gb300.sim import power_spectrum, release_work
+    points, _ = _points(256, 1000, 1)
+    ref = power_spectrum(points, 100.0, 256, 4)
+    held = _hold(points)
+    before = _free()
+    release_work()
+    assert _free() - before >= held
+    release_work()  # (nothing left: fine)
+    for a, b in zip(power_spectrum(points, 100.0, 256, 4), ref):
+        np.testing.assert_allclose(a, b, rtol=1e-12)
