@@ -2871,6 +2871,31 @@ int slot_bottom(int maxLc) { return 5 * maxLc; }
 int slot_up(int maxLc, int l, int k) { return 5 * maxLc + 1 + 5 * l + k; }  // k: 0 prolong, 1..4 sweeps
 int n_slots(int maxLc) { return 10 * maxLc + 1; }
 
+// The V-cycle's tables, all or (on an error) none: a step that finds them
+// made takes every one as allocated.
+pm_status alloc_vcycle_tables(pm_batch* B) {
+  // the first configuration fixes the V-cycle depth (cubes only shrink)
+  int M = 0;
+  for (pm_ctx* c : B->ctx) M = std::max(M, first_small_level(c));
+  B->maxLc = M;
+  B->t_vc.resize(n_slots(M));
+  B->t_leg.resize(2 * M);
+  pm_status st = PM_OK;
+  for (auto& t : B->t_vc) {
+    size_t sz = std::max(std::max(sizeof(RbgsDesc), sizeof(RestrictDesc)),
+                         std::max(sizeof(ProlongDesc), sizeof(CmgDesc)));
+    if (st == PM_OK) st = tab_alloc(B, t, sz);
+  }
+  for (auto& t : B->t_leg)
+    if (st == PM_OK) st = tab_alloc(B, t, sizeof(TileDesc));
+  if (st == PM_OK) return PM_OK;
+  for (auto* v : {&B->t_vc, &B->t_leg}) {
+    for (auto& t : *v) tab_free(t);
+    v->clear();
+  }
+  return st;
+}
+
 // Upload the descriptor table of the bottom (every realisation's first level
 // small enough for one CTA or cluster).
 void upload_bottom_table(pm_batch* B) {
@@ -3444,22 +3469,8 @@ pm_status pm_batch_step(pm_batch* B, int32_t n_steps) {
       if (changed) B->tables_stale = true;
     }
     if (B->t_vc.empty()) {
-      // the first configuration fixes the V-cycle depth (cubes only shrink)
-      int M = 0;
-      for (int r = 0; r < R; ++r) M = std::max(M, first_small_level(B->ctx[r]));
-      B->maxLc = M;
-      B->t_vc.resize(n_slots(M));
-      for (auto& t : B->t_vc) {
-        size_t sz = std::max(std::max(sizeof(RbgsDesc), sizeof(RestrictDesc)),
-                             std::max(sizeof(ProlongDesc), sizeof(CmgDesc)));
-        pm_status st = tab_alloc(B, t, sz);
-        if (st != PM_OK) return st;
-      }
-      B->t_leg.resize(2 * M);
-      for (auto& t : B->t_leg) {
-        pm_status st = tab_alloc(B, t, sizeof(TileDesc));
-        if (st != PM_OK) return st;
-      }
+      pm_status st = alloc_vcycle_tables(B);
+      if (st != PM_OK) return st;
     }
     // 1-2. half drift + deposit
     {

@@ -77,3 +77,30 @@ def test_solve_without_enough_vcycles_reports_noconv(lib):
     assert st["resid_last"] > 1e-13 and st["vcycles_last"] == 1
     sim.close()
     _deposit_ok()
+
+
+def test_batch_step_after_refused_tables_starts_over(monkeypatch):
+    """The first batched step allocates its V-cycle tables.  Where the device
+    is full (PM_FAULT_FULL=2) it fails with PM_ENOMEM; the next step makes the
+    tables anew (all of them: none is left half made) and gives the bits of a
+    batch that met no failure."""
+    from paper_1709_04703_gb300 import _lib as L
+    from paper_1709_04703_gb300 import ics
+    from paper_1709_04703_gb300.sim import Batch
+    x, p, ids = ics.random_particles(3000, 64, 11)
+
+    def batch():
+        return Batch([dict(pos=x, mom=p, ids=ids, n_mesh=64, box=900.0)], 0.1, 1.0, 20)
+    ok, bad = batch(), batch()
+    monkeypatch.setenv("PM_FAULT_FULL", "2")
+    for _ in range(2):
+        with pytest.raises(L.PmError) as e:
+            bad.step(1)
+        assert e.value.code == L.PM_ENOMEM
+    monkeypatch.delenv("PM_FAULT_FULL")
+    bad.step(2)
+    ok.step(2)
+    for a, b in zip(bad.particles(0), ok.particles(0)):
+        np.testing.assert_array_equal(a, b)
+    bad.close()
+    ok.close()
