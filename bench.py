@@ -165,9 +165,8 @@ ARITHMETIC = {
 # ncu dram__bytes_read.sum + dram__bytes_write.sum over the algorithmic bytes
 # of the kernel class's launches at 256^3 on the current kernels
 TRAFFIC_RATIO = {
-    # the smoother's algorithmic bytes are 12 B per cell and sweep and 9 for
-    # the residual and restriction in the leg down: 57 B per pair of legs
-    "smooth0": ((71951616 + 31623424 + 152123904 + 36274176) / (57.0 * 256**3),
+    # the fused leg down must move 8.5 B per cell, the two-sweep pass up 12
+    "smooth0": ((71951616 + 31623424 + 152123904 + 36274176) / (20.5 * 256**3),
                 "k_tile down + k_rbgs2 at 256^3, profiles/kernels_pm256.md"),
     "defect": ((273779712 + 50797824 + 347053312 + 169682688) / (335.5e6 + 536.9e6),
                "k_defect<0> + k_defect<1> at 256^3, profiles/kernels_pm256.md"),
@@ -691,7 +690,7 @@ def run_ours(args):
     # headline comes from the uninstrumented run above), and per step the
     # active particles N, cells C and V-cycles k for the whole-step count
     sim = _new_sim(pos, mom, ids, cfg, rtol, args.precision)
-    prof, per_step = None, []
+    prof, seen = None, 0
     p0 = time.perf_counter()
     lib = L.load()
     for k0, cnt in windows:
@@ -702,10 +701,8 @@ def run_ours(args):
         torch.cuda.synchronize()
         l_start = lib.pm_launch_count()
         for _ in range(cnt):
-            n_act = sim.stats()["n_active"]
             sim.step(1)
-            s1 = sim.stats()
-            per_step.append((n_act, s1["cube_side"] ** 3, s1["vcycles_last"]))
+            seen += sim.stats()["vcycles_last"]
         # the library's kernel launches of this window (for a launch list
         # of exactly these steps: ncu -k regex:^k_ -s <start> -c <count>)
         print(f"instrumented window from step {k0}: library launches {l_start} .. "
@@ -716,13 +713,12 @@ def run_ours(args):
             c: {f: prof[c][f] + part[c][f] for f in ("ms", "groups", "bytes")} for c in prof}
     torch.cuda.synchronize()
     prof_wall_ms = (time.perf_counter() - p0) * 1e3
-    if sum(v for _, _, v in per_step) != vstats["vcycles_total"]:
+    if seen != vstats["vcycles_total"]:
         raise RuntimeError("the instrumented repeat took a different number of V-cycles")
     sim.close()
-    # whole-step algorithmic bytes (N active particles, C active cells, k
-    # V-cycles, o = k outer defect-correction iterations in the mixed forms)
-    o_of = (lambda v: v) if args.precision != "fp32" else (lambda v: 0)
-    step_bytes = sum(64.0 * N + (24.0 + 74.0 * v + 40.0 * o_of(v)) * Cc for N, Cc, v in per_step)
+    # whole-step bytes: what every launch of these steps must move, as the
+    # library books it per class (pm_profile_read)
+    step_bytes = sum(v["bytes"] for v in prof.values())
 
     # the same windows with plain FP32 V-cycles at the same tolerance, the
     # mixed path at 1e-7 (below the plain floor), FP64 forms, the other
@@ -856,9 +852,8 @@ def run_ours(args):
                           "achieved": round(step_bytes / (ms * 1e-3) / 1e9, 1),
                           "peak": peak, "unit": "GB/s",
                           "frac": round(step_bytes / (ms * 1e-3) / 1e9 / peak, 4),
-                          "count": "sum over the timed steps of 64 N + (24 + 74 k + 40 o) C: N "
-                                   "active particles, C active cells, k V-cycles, o = k outer "
-                                   "iterations (0 in plain FP32)"},
+                          "count": "bytes that each launch of the timed steps must move, summed "
+                                   "over the kernel classes"},
         "kernels": kernels,
         "kernels_timing": "CUDA events around each kernel class on the context stream, in an "
                           f"instrumented repeat of the same {K} steps ({prof_wall_ms / K:.3f} "

@@ -390,8 +390,10 @@ enum {
   PM_PROF_DEPOSIT = 0,  /* half drift + CIC deposit                         */
   PM_PROF_SOURCE,       /* counts -> double-float source (+ moments)        */
   PM_PROF_BOUNDARY,     /* open-boundary ghost layer                        */
-  PM_PROF_SMOOTH0,      /* red-black sweeps on the finest level             */
-  PM_PROF_TRANSFER0,    /* finest-level residual+restriction, prolongation  */
+  PM_PROF_SMOOTH0,      /* red-black sweeps on the finest level, with the
+                           transfer of a fused leg (pm_step)                */
+  PM_PROF_TRANSFER0,    /* finest-level residual+restriction, prolongation
+                           where they are launches of their own             */
   PM_PROF_COARSE,       /* everything on levels >= 1                        */
   PM_PROF_DEFECT,       /* double-float residual + norm                     */
   PM_PROF_CORRECT,      /* Phi += e                                         */

@@ -826,13 +826,20 @@ pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
     U[l] = masked(ctx, compact_view(ctx->lu[l], ctx->ls[l]), l);
     B[l] = masked(ctx, compact_view(ctx->lb[l], ctx->ls[l]), l);
   }
-  const double c0 = (double)ctx->s * ctx->s * ctx->s;
-  // algorithmic bytes per fine cell: a red-black SOR sweep reads u
-  // and b and writes u, 12 B per sweep (two sweeps per smoothing: 24; the
-  // fused pass moves 8 from a zero start and 12 otherwise, since its two
-  // sweeps share one read and one write); residual + restriction reads u
-  // and b and writes the coarse b and u (9); prolongation reads u and the
-  // coarse u and writes u + P uc (8.5)
+  // What each launch must move, in bytes per cell of its level: a fused leg
+  // down reads b and writes w and the coarse b (8.5), a fused leg up reads w,
+  // b and the coarse u and writes u (12.5); the two-sweep pass reads b and,
+  // unless it starts from zero, u, and writes u (8 or 12), two sweeps of
+  // one-colour passes 12 each; residual + restriction reads u and b and writes
+  // the coarse b and u (9); prolongation reads u and the coarse u and writes
+  // u + P uc (8.5); the bottom reads b and writes u (8).  Levels below the
+  // finest are booked together.
+  double coarse_bytes = 0.0;
+  auto cells_of = [&](int l) { return (double)ctx->ls[l] * ctx->ls[l] * ctx->ls[l]; };
+  auto book = [&](int l, int cls, int e, double per_cell) {
+    if (l == 0) prof_end(ctx, cls, e, per_cell * cells_of(0));
+    else coarse_bytes += per_cell * cells_of(l);
+  };
   float h2 = 1.0f;
   int ec = -1;
   // open-boundary ghost factor of level l (spacing H = 2^l), see k_mg.cu
@@ -865,10 +872,8 @@ pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
       int e = l == 0 ? prof_begin(ctx) : -1;
       Upre[l] = compact_view(ctx->lu2[l], ctx->ls[l]);
       launch_tile(ctx->st, tile_args(l), false, tile_small(ctx->ls[l]));
-      if (l == 0) {
-        prof_end(ctx, PM_PROF_SMOOTH0, e, (24.0 + 9.0) * c0);
-        ec = prof_begin(ctx);
-      }
+      book(l, PM_PROF_SMOOTH0, e, 8.5);
+      if (l == 0) ec = prof_begin(ctx);
       h2 *= 4.0f;
       continue;
     }
@@ -886,31 +891,28 @@ pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
       launch_rbgs2(ctx->st, U[l], Upre[l], B[l], h2, per, gam(l), zs, f2_zc, d0, f2_ty);
     else
       smooth2(ctx, U[l], B[l], h2, per, gam(l), zs, d0, l > 0 ? LEVEL_SWEEPS : 2);
-    if (l == 0) {
-      prof_end(ctx, PM_PROF_SMOOTH0, e, 24.0 * c0);
-      e = prof_begin(ctx);
-    }
+    book(l, PM_PROF_SMOOTH0, e, !fused ? 24.0 : (zs ? 8.0 : 12.0));
+    if (l == 0) e = prof_begin(ctx);
     launch_resid_restrict(ctx->st, Upre[l], B[l], 1.0f / h2, U[l + 1], B[l + 1], per, gam(l),
                           d0);
-    if (l == 0) {
-      prof_end(ctx, PM_PROF_TRANSFER0, e, 9.0 * c0);
-      ec = prof_begin(ctx);
-    }
+    book(l, PM_PROF_TRANSFER0, e, 9.0);
+    if (l == 0) ec = prof_begin(ctx);
     h2 *= 4.0f;
   }
   if (Lc == 0) ec = prof_begin(ctx);
   launch_cmg(ctx->st, U[Lc], B[Lc], Lc, per, COARSE_SWEEPS, Lc == 0 ? zero0 : true,
                    ctx->sig);
+  coarse_bytes += 8.0 * cells_of(Lc);
   for (int l = Lc - 1; l >= 0; --l) {
     h2 *= 0.25f;
     int e = -1;
     if (l == 0) {
-      prof_end(ctx, PM_PROF_COARSE, ec, (Lc > 0 ? 8.0 / 7.0 * 81.0 * c0 / 8.0 : 0.0));
+      prof_end(ctx, PM_PROF_COARSE, ec, coarse_bytes);
       e = prof_begin(ctx);
     }
     if (tiled(l) && ctx->ls[l] < FUSED_MIN) {
       launch_tile(ctx->st, tile_args(l), true, tile_small(ctx->ls[l]));
-      if (l == 0) prof_end(ctx, PM_PROF_SMOOTH0, e, (24.0 + 8.5) * c0);
+      book(l, PM_PROF_SMOOTH0, e, 12.5);
       continue;
     }
     const bool fused = ctx->ls[l] >= FUSED_MIN && (!ball || l == 0);
@@ -920,19 +922,17 @@ pm_status vcycle(pm_ctx* ctx, Grid u0, Grid b0, bool zero0) {
       launch_prolong_to(ctx->st, U[l + 1], Upre[l], W, per, gam(l + 1));
     else
       launch_prolong(ctx->st, U[l + 1], U[l], per, gam(l + 1));
-    if (l == 0) {
-      prof_end(ctx, PM_PROF_TRANSFER0, e, 8.5 * c0);
-      e = prof_begin(ctx);
-    }
+    book(l, PM_PROF_TRANSFER0, e, 8.5);
+    if (l == 0) e = prof_begin(ctx);
     int f2_ty = 16, f2_zc = 0;
     f2_choice(ctx, ctx->ls[l], &f2_ty, &f2_zc);
     if (fused)
       launch_rbgs2(ctx->st, W, U[l], B[l], h2, per, gam(l), false, f2_zc, d0, f2_ty);
     else
       smooth2(ctx, U[l], B[l], h2, per, gam(l), false, d0, l > 0 ? LEVEL_SWEEPS : 2);
-    if (l == 0) prof_end(ctx, PM_PROF_SMOOTH0, e, 24.0 * c0);
+    book(l, PM_PROF_SMOOTH0, e, fused ? 12.0 : 24.0);
   }
-  if (Lc == 0) prof_end(ctx, PM_PROF_COARSE, ec, 0.0);
+  if (Lc == 0) prof_end(ctx, PM_PROF_COARSE, ec, coarse_bytes);
   CKL();
   return PM_OK;
 }
@@ -1723,15 +1723,16 @@ pm_status pm_step(pm_ctx* ctx, int32_t n_steps) {
     if (st != PM_OK) return st;
     const long long N = ctx->n_active;
     if (ctx->cfg.sort_every > 0 && k % ctx->cfg.sort_every == 0 && N > 1) {
-      // particle order by cell: keys (read x 16 B, write key + index 8 B),
-      // per pass a histogram (4 B) and a scatter (read and write key + index,
-      // 16 B), then the permutation (4 B) and both records (read and write,
-      // 64 B)
+      // particle order by cell: keys (read x 16 B, write the key 4 B), per
+      // pass a histogram (4 B; the first pass's with the keys) and a scatter
+      // (read and write key + index, 16 B; the first reads no index, the last
+      // writes no key: 8 + 20 passes in all), then the permutation (4 B) and
+      // both records (read and write, 64 B)
       NvtxRange nvtx_sort("pm sort");
       int es = prof_begin(ctx);
       CK(launch_sort_particles(ctx->st, ctx->pos, ctx->mom, N, n, ctx->sortw, ctx->pos2,
                                ctx->mom2));
-      prof_end(ctx, PM_PROF_SORT, es, (24.0 + 20.0 * sort_passes(n) + 68.0) * N);
+      prof_end(ctx, PM_PROF_SORT, es, (8.0 + 20.0 * sort_passes(n) + 68.0) * N);
       std::swap(ctx->pos, ctx->pos2);
       std::swap(ctx->mom, ctx->mom2);
     }
