@@ -456,6 +456,12 @@ pm_status pm_batch_get_forces(pm_batch* b, int32_t r, float* f4, int32_t host_me
  * cannot be resident. */
 pm_status pm_batch_set_solve(pm_batch* b, int32_t persistent, double wait_seconds,
                              int32_t extra_arrivals);
+/* The tiles of the default solve's V-cycle legs: side[l] = 8 (8 x 8 x 8
+ * cells) or 16 (16 x 16 x 8) on level l, a function of the realisations'
+ * first cubes.  *count (required) = the levels so smoothed (0 before the
+ * first step); at most cap entries are written.  PM_EINVAL on bad
+ * arguments. */
+pm_status pm_batch_leg_tiles(pm_batch* b, int32_t* side, int32_t cap, int32_t* count);
 const char* pm_batch_last_error(const pm_batch* b);
 void pm_batch_destroy(pm_batch* b);
 

@@ -2764,7 +2764,7 @@ struct pm_batch {
   cudaGraphExec_t sgraph = nullptr;
   cudaStream_t st2 = nullptr;  // captures the loop's body
   long long loop_kernels = 0;  // kernels of one pass of the loop body
-  std::vector<char> leg_small;  // per level: its fused legs take the small tiles (autotuned)
+  std::vector<char> leg_small;  // per level: its fused legs take the small tiles (pick_legs)
   // the persistent solve: one cooperative launch per solve
   bool persistent = false;
   double wait_s = 2.0;         // longest wait at one grid barrier
@@ -3060,41 +3060,19 @@ void launch_vcycle_legs(pm_batch* B, cudaStream_t st) {
   for (int l = M - 1; l >= 0; --l) launch_leg(B, st, l, true, B->d_active);
 }
 
-// Autotuner of the fused legs: before the V-cycle graph is captured, each
-// level's down leg runs with both tile shapes on the batch's own grids (it
-// writes only the level's scratch grid and the coarse right-hand side, which
-// every V-cycle rewrites) and the faster shape is kept.  Both compute the
-// same cells with the same arithmetic: the choice changes the time, not the
-// bits.
-pm_status tune_legs(pm_batch* B) {
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
-    return bfail(B, PM_ECUDA, "pm_batch: event creation failed");
-  const int M = B->maxLc;
-  std::vector<float> tot[2];
-  for (int q = 0; q < 2; ++q) {
-    B->leg_small.assign(M, (char)q);
-    for (auto& t : B->t_leg) t.grid_max = 0;
-    upload_leg_tables(B);
-    tot[q].assign(M, 0.0f);
-    for (int l = 0; l < M; ++l)
-      for (int rep = 0; rep < 3; ++rep) {  // the first pass warms up
-        cudaEventRecord(e0, B->st);
-        launch_leg(B, B->st, l, false, nullptr);
-        cudaEventRecord(e1, B->st);
-        cudaEventSynchronize(e1);
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (rep > 0) tot[q][l] += ms;
-      }
+// The tile shape of each level's legs, by the tiles of the realisations that
+// have the level (tile_small), before the V-cycle graph is captured.  Both
+// shapes compute the same cells with the same arithmetic: the choice changes
+// the time, not the bits.
+void pick_legs(pm_batch* B) {
+  B->leg_small.assign(B->maxLc, 0);
+  for (int l = 0; l < B->maxLc; ++l) {
+    long long n[2] = {0, 0};
+    for (pm_ctx* c : B->ctx)
+      if (l < first_small_level(c))
+        for (int q = 0; q < 2; ++q) n[q] += nblocks(tile_grid(c->ls[l], q != 0));
+    B->leg_small[l] = tile_small(n[1], n[0]);
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  for (int l = 0; l < M; ++l) B->leg_small[l] = tot[1][l] < tot[0][l];
-  for (auto& t : B->t_leg) t.grid_max = 0;
-  upload_leg_tables(B);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? PM_OK : bfail(B, PM_ECUDA, cudaGetErrorString(e));
 }
 
 // Capture the graph solve once (grids at their largest: the first cubes,
@@ -3301,12 +3279,8 @@ pm_status batch_solve_persistent(pm_batch* B) {
 
 // One launch of the solve graph (captured at the first solve).
 pm_status batch_solve_graph(pm_batch* B) {
-  if (B->leg_small.empty() && B->maxLc > 0) {
-    pm_status st = tune_legs(B);
-    if (st != PM_OK) return st;
-  } else if (B->tables_stale) {
-    upload_leg_tables(B);
-  }
+  if (B->leg_small.empty()) pick_legs(B);
+  if (B->tables_stale) upload_leg_tables(B);
   B->tables_stale = false;
   upload_defect_table(B, B->d_res->iters);
   upload_grad_table(B, B->d_res->iters);
@@ -3752,6 +3726,14 @@ pm_status pm_batch_set_solve(pm_batch* B, int32_t persistent, double wait_second
   }
   B->wait_s = wait_seconds;
   B->extra = extra_arrivals;
+  return PM_OK;
+}
+
+pm_status pm_batch_leg_tiles(pm_batch* B, int32_t* side, int32_t cap, int32_t* count) {
+  if (!B || !count || cap < 0 || (cap > 0 && !side))
+    return bfail(B, PM_EINVAL, "pm_batch_leg_tiles: bad argument");
+  *count = (int32_t)B->leg_small.size();
+  for (int l = 0; l < std::min(cap, *count); ++l) side[l] = B->leg_small[l] ? 8 : 16;
   return PM_OK;
 }
 

@@ -9,15 +9,20 @@
 // launches and five sweeps over L2.  A tile recomputes its halo instead: 24 x
 // 24 x 16 cells for a 16 x 16 x 8 tile, 4.5 times the updates, but one pass.
 //
-// Microseconds per leg inside a graph, separate passes -> fused (8^3 tiles up
-// to side 48, 16 x 16 x 8 above; periodic, and open on a coarse level):
+// Microseconds per leg inside a graph, separate passes -> fused (the tiles of
+// tile_small below; periodic, and open on a coarse level):
 //   side   down           up             down, open     up, open
-//     32   8.2 ->  3.0    8.8 ->  5.0    8.8 ->  4.2    9.1 ->  7.1
-//     64  11.0 ->  4.0   14.0 ->  6.3   11.8 ->  5.1   13.7 -> 10.5
-//    128  27.0 -> 16.6   35.1 -> 27.2   28.0 -> 20.2   35.7 -> 35.9
+//     32   8.3 ->  3.1    9.1 ->  5.0    8.9 ->  4.3    9.0 ->  7.2
+//     48   9.5 ->  3.6   11.3 ->  5.8   10.3 ->  4.4   10.9 ->  7.6
+//     64  11.2 ->  4.0   13.8 ->  6.3   11.9 ->  5.1   13.7 -> 10.6
+//     96  16.9 ->  8.2   20.2 -> 13.5   17.3 -> 11.2   20.3 -> 19.3
+//    128  27.1 -> 16.6   35.2 -> 27.2   28.0 -> 20.3   35.7 -> 35.9
 // Above, the leg down still gains on the z-marching pass and a restriction
-// (192: 55.9 -> 52.1, 256: 149 -> 124), the leg up does not (192: 67.7 against
-// 87.3, 256: 165 against 202), since that pass updates less halo.
+// (its best of nine tile shapes; 160 open: 39.2 -> 33.6, 192: 55.9 -> 52.0,
+// 256: 149 -> 124).  The leg up loses to the prolongation and that pass, which
+// updates less halo (192: 63.4 against 87.4, 256: 152 against 202; so it would
+// at 160 in its best shape, 44.3 against 58.5, but only levels of side 192 and
+// up are timed for one, and in its default shape it takes 54.6).
 #include "mg_arith.cuh"
 #include "pm_kernels.cuh"
 
@@ -414,7 +419,33 @@ void launch_t(cudaStream_t st, const TileArgs& a) {
 
 }  // namespace
 
-bool tile_small(int s) { return s <= TILE_SMALL_MAX; }
+// A launch takes as long as its busiest SM: a leg down with 1, 2, 3, 4, 5, 7
+// small tiles on an SM 3.7, 4.3, 5.1, 6.1, 8.4, 10.5 us, with 1, 2, 3 large
+// ones (four times the cells) 4.9, 6.5, 9.8 us.  So the small shape is taken
+// while it puts at most twice the large one's tiles on an SM.  us per leg,
+// small / large (periodic, boxes of one side in one launch; 152 SMs):
+//   boxes   side  tiles       per SM  down          up
+//     1      48   216 /  54   2 / 1   3.6 /  3.9    5.8 /  6.2
+//     1      64   512 / 128   4 / 1   6.0 /  5.0    9.3 /  7.3
+//     2      48   432 / 108   3 / 1   5.2 /  5.0    7.8 /  7.2
+//     4      40   500 / 180   4 / 2   5.8 /  6.4    8.9 /  9.5
+//     2      56   686 / 224   5 / 2   8.4 /  6.4   13.0 /  9.5
+//    16      24   432 / 192   3 / 2   5.2 /  6.4    7.9 /  9.1
+//    16      32  1024 / 256   7 / 2  10.8 /  6.6   16.8 /  9.6
+// Over 210 such launches (1 to 32 boxes of side 20 to 128, mixed ones, both
+// boundaries) it is 0.2 % from the better shape in the mean, 10 % at worst.
+// For one box it draws the line between the sides 48 and 56.
+bool tile_small(long long small_tiles, long long large_tiles) {
+  constexpr long long SMS = 152;
+  return (small_tiles + SMS - 1) / SMS <= 2 * ((large_tiles + SMS - 1) / SMS);
+}
+bool tile_small(int s) {
+  auto count = [&](bool small) {
+    const dim3 g = tile_grid(s, small);
+    return (long long)g.x * g.y * g.z;
+  };
+  return tile_small(count(true), count(false));
+}
 
 dim3 tile_grid(int s, bool small) { return small ? grid_of<TileS>(s) : grid_of<TileL>(s); }
 

@@ -262,8 +262,9 @@ struct TileDesc {
   TileArgs a;
   int r, gx, gy, gz;
 };
-// levels up to this side take 8^3 tiles, larger ones 16 x 16 x 8
-constexpr int TILE_SMALL_MAX = 48;
+// 8^3 tiles, or 16 x 16 x 8, for a launch over boxes that together have so
+// many of each (the rule's reasons: k_tile.cu); for one box of side s
+bool tile_small(long long small_tiles, long long large_tiles);
 bool tile_small(int s);
 dim3 tile_grid(int s, bool small);
 void launch_tile(cudaStream_t st, const TileArgs& a, bool up, bool small);

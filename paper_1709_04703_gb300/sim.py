@@ -136,6 +136,13 @@ class Batch:
         self._check(self._lib.pm_batch_set_solve(self._b, int(bool(persistent)),
                                                  float(wait_seconds), int(extra_arrivals)))
 
+    def leg_tiles(self):
+        """Tile side (8 or 16 cells) of the default solve's legs, finest
+        level first ([] before the first step)."""
+        cnt, side = C.c_int32(0), (C.c_int32 * 16)()
+        self._check(self._lib.pm_batch_leg_tiles(self._b, side, 16, C.byref(cnt)))
+        return list(side[:cnt.value])
+
     def stats(self, r):
         s = L.PmStats()
         self._check(self._lib.pm_batch_stats(self._b, int(r), C.byref(s)))

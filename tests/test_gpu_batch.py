@@ -262,3 +262,33 @@ def test_persistent_barrier_wait_runs_out():
     b.step(2)
     _compare(b, 1, _single(reals[1], a0, a1, steps, rtol, 2))
     b.close()
+
+
+@pytest.mark.parametrize("sizes", [[32], [48], [64], [48, 48], [64, 24, 24, 24], [96, 48, 32],
+                                   [32] * 16, [24] * 16,
+                                   [32, 48, 64, 96, 128, 32, 64, 128, 48, 96, 64, 32]])
+def test_leg_tiles_by_the_tiles_per_sm(sizes):
+    """A batch's tile shapes follow from its boxes alone (small tiles while
+    they put at most twice the large ones' number on an SM), not from a timing
+    in the process: two batches of the same boxes take the same."""
+    from paper_1709_04703_gb300 import _lib as L
+    from paper_1709_04703_gb300.sim import Batch
+    top = {1: 16, 8: 32, 16: 64}[L.load().pm_mg_cluster_size()]
+
+    def up(a, b):
+        return -(-a // b)
+    want = []
+    for l in range(8):
+        s = [n >> l for n in sizes if n >> l > top]
+        if not s:
+            break
+        small = sum(up(v, 8) ** 3 for v in s)
+        large = sum(up(v, 16) ** 2 * up(v, 8) for v in s)
+        want.append(8 if up(small, 152) <= 2 * up(large, 152) else 16)
+    for _ in range(2):
+        reals = [_realisation(n, 8.0 * n, 900 + r, 0.05) for r, n in enumerate(sizes)]
+        batch = Batch(reals, 0.05, 1.0, 200)
+        assert batch.leg_tiles() == []
+        batch.step(1)
+        assert batch.leg_tiles() == want
+        batch.close()
