@@ -553,6 +553,20 @@ pm_status pm_mg_restrict(const float* u, const float* b, int32_t s, int32_t peri
 pm_status pm_mg_prolong(const float* uc, float* u, int32_t s, int32_t periodic, float gam_c,
                         void* stream);
 
+/* One leg of a V-cycle level, on arrays as above, with the solver's fused
+ * kernel in tiles of 8 x 8 x 8 (tile = 8) or 16 x 16 x 8 cells (tile = 16), or
+ * as the separate passes that it stands for (tile = 0): the same bits.
+ * up = 0: w = two sweeps of pm_mg_smooth from zero on A w = b and bc = the
+ * restriction of its residual, with the diagonal d0 (6, or more for a shifted
+ * operator) in place of 6; tile = 0 zeroes uc, as pm_mg_restrict does.
+ * up = 1: u = two sweeps on A u = b from w + P uc (pm_mg_prolong with gam_c).
+ * Only interiors are written; the ghost layers of u, w and uc must hold zeros.
+ * All arrays distinct; s even, 20 <= s <= 1024, d0 >= 6.  Errors: PM_EINVAL,
+ * PM_ECUDA.  Synchronises stream. */
+pm_status pm_mg_leg(int32_t up, float* u, const float* b, float* w, float* uc, float* bc,
+                    int32_t s, int32_t periodic, float h2, float gam, float gam_c, float d0,
+                    int32_t tile, void* stream);
+
 /* C[M x N] (FP32, row-major) = A[M x K] B[N x K]^T with A, B row-major BF16
  * device matrices; M % 128 == 0, K % 64 == 0, N in {16, 32, 64, 128}.  The
  * tile engine under every convolution of the learned guess.  PM_ETIMEOUT if

@@ -38,6 +38,7 @@ EXPORTED = [
     "pm_guess_get_params", "pm_guess_forward", "pm_guess_loss_grad", "pm_guess_adam",
     "pm_guess_last_error", "pm_guess_destroy", "pm_set_guess", "pm_capture",
     "pm_mg_cluster_size", "pm_smoother_tiles", "pm_release_work", "pm_batch_leg_tiles",
+    "pm_mg_leg",
 ]
 PROF_CLASSES = ["deposit", "source", "boundary", "smooth0", "transfer0", "coarse",
                 "defect", "correct", "gather", "compact", "guess", "ade", "sort"]
@@ -132,6 +133,7 @@ def load():
         "pm_selftest_wait": (I32, [I32, I64, P]),
         "pm_mg_restrict": (I32, [P, P, I32, I32, F, F, P, P, P]),
         "pm_mg_prolong": (I32, [P, P, I32, I32, F, P]),
+        "pm_mg_leg": (I32, [I32, P, P, P, P, P, I32, I32, F, F, F, F, I32, P]),
         "pm_nn_gemm_bf16": (I32, [P, P, P, I32, I32, I32, P]),
         "pm_mg_smooth": (I32, [P, P, P, I32, I32, C.c_float, C.c_float, I32, I32, I32, P]),
         "pm_guess_create": (I32, [I32, P, C.POINTER(P)]),

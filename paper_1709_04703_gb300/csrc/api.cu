@@ -3798,6 +3798,42 @@ extern "C" pm_status pm_mg_prolong(const float* uc, float* u, int32_t s, int32_t
   return finish_test_call(st);
 }
 
+extern "C" pm_status pm_mg_leg(int32_t up, float* u, const float* b, float* w, float* uc,
+                               float* bc, int32_t s, int32_t periodic, float h2, float gam,
+                               float gam_c, float d0, int32_t tile, void* stream) {
+  if (!u || !b || !w || !uc || !bc || u == w || s < 20 || (s & 1) || s > 1024 || !(h2 > 0) ||
+      !(d0 >= 6) || (up != 0 && up != 1) || (tile != 0 && tile != 8 && tile != 16))
+    return fail(nullptr, PM_EINVAL, "pm_mg_leg: bad argument");
+  cudaStream_t st = (cudaStream_t)stream;
+  TileArgs a;
+  a.u = padded_view(u, s);
+  a.b = padded_view(b, s);
+  a.w = padded_view(w, s);
+  a.uc = padded_view(uc, s / 2);
+  a.bc = padded_view(bc, s / 2);
+  a.h2 = h2;
+  a.inv_h2 = 1.0f / h2;
+  a.gam = gam;
+  a.gam_c = gam_c;
+  a.d0 = d0;
+  a.periodic = periodic != 0;
+  if (tile) {
+    launch_tile(st, a, up != 0, tile == 8);
+    return finish_test_call(st);
+  }
+  const Grid g = up ? a.u : a.w;
+  if (up) {
+    const size_t bytes = sizeof(float) * (size_t)(s + 2) * (s + 2) * (s + 2);
+    if (cudaMemcpyAsync(u, w, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+      return fail(nullptr, PM_ECUDA, "pm_mg_leg: copy");
+    launch_prolong(st, a.uc, g, a.periodic, gam_c);
+  }
+  for (int q = 0; q < 4; ++q)
+    launch_rbgs(st, g, a.b, h2, q & 1, a.periodic, gam, up || q > 1 ? 0 : q + 1, d0);
+  if (!up) launch_resid_restrict(st, g, a.b, a.inv_h2, a.uc, a.bc, a.periodic, gam, d0);
+  return finish_test_call(st);
+}
+
 extern "C" pm_status pm_mg_smooth(const float* u_in, float* u_out, const float* b, int32_t s,
                                   int32_t periodic, float h2, float gam, int32_t zero_start,
                                   int32_t fused, int32_t zchunk, void* stream) {

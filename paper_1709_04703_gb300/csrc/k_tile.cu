@@ -432,7 +432,7 @@ void launch_t(cudaStream_t st, const TileArgs& a) {
 //     2      56   686 / 224   5 / 2   8.4 /  6.4   13.0 /  9.5
 //    16      24   432 / 192   3 / 2   5.2 /  6.4    7.9 /  9.1
 //    16      32  1024 / 256   7 / 2  10.8 /  6.6   16.8 /  9.6
-// Over 210 such launches (1 to 32 boxes of side 20 to 128, mixed ones, both
+// Over 224 such launches (1 to 32 boxes of side 20 to 128, mixed ones, both
 // boundaries) it is 0.2 % from the better shape in the mean, 10 % at worst.
 // For one box it draws the line between the sides 48 and 56.
 bool tile_small(long long small_tiles, long long large_tiles) {
