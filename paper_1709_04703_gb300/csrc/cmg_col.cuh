@@ -10,9 +10,12 @@
 // colour) on two planes, every index is an offset computed once per level,
 // the two colours live in separate padded arrays (conflict-free reads), and
 // each level is a named barrier over the warps it needs.  The bottom itself
-// (side <= 4 or odd) belongs to one warp; its lexicographic sweep on odd
-// periodic sides runs the diagonal fronts in parallel.  The operations and
-// their order are those of cmg_fast.cuh, through mg_arith.cuh: the same bits.
+// (side <= 4 or odd) belongs to one warp, where it is open and of side 5 or 7
+// to a thread per cell of a colour (one warp took 11 trips a pass for the 343
+// cells: inside open steps a top of 14 37.4 us, of 10 20.7; so 14.4 and 13.0);
+// its lexicographic sweep on odd periodic sides runs the diagonal fronts in
+// parallel.  The operations and their order are those of cmg_fast.cuh, through
+// mg_arith.cuh: the same bits.
 #pragma once
 #include "cmg_fast.cuh"
 
@@ -41,6 +44,14 @@ constexpr int CL_SMEM = cl_floats(16);
 
 __device__ __forceinline__ void cl_bar(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// threads that work on the bottom of side S
+__host__ __device__ constexpr bool cl_wide(int S, int periodic) {
+  return !periodic && (S == 5 || S == 7);
+}
+__host__ __device__ constexpr int cl_bottom_threads(int S, int periodic) {
+  return cl_wide(S, periodic) ? (S * S * S / 2 + 1 + 31) / 32 * 32 : 32;
 }
 
 // the cells lane, lane + 32, ... of an S^3 level in x order, by their
@@ -144,6 +155,46 @@ __device__ __noinline__ void cl_bottom(float* u, const FcLev& L, int sweeps, flo
   }
 }
 
+// an open bottom of odd side: colour c holds the cells c, c + 2, ... in x
+// order, thread e the e-th of each, with their values in registers.  The
+// barrier is the bottom's own (3).
+__device__ __noinline__ void cl_bottom_wide(int S, float* u, const FcLev& L, int sweeps) {
+  const int P = S + 2, P2 = P * P, N = S * S * S, n = cl_bottom_threads(S, 0);
+  float *b = u + P * P2, *lin = b + N;
+  int at[2];
+  bool on[2];
+  float v[2], f[2], r[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int t = 2 * (int)threadIdx.x + c;
+    on[c] = t < N;
+    const int q = on[c] ? t : 0, i = q % S, j = q / S % S, k = q / (S * S);
+    at[c] = ((k + 1) * P + j + 1) * P + i + 1;
+    v[c] = u[at[c]];
+    f[c] = b[q];
+    r[c] = L.simple ? 1.0f / 6.0f : __frcp_rn(mg_diag(i, j, k, S, 0, L.gam, L.d0));
+  }
+  const float omega = 2.0f / (1.0f + sinf(3.14159265f / (float)(S + 1)));
+  cl_bar(3, n);  // every value read
+#pragma unroll 1
+  for (int w = 0; w < sweeps; ++w) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (on[c]) {
+        const float* p = u + at[c];
+        const float gs = gs_scaled(nb6(p[-1], p[1], p[-P], p[P], p[-P2], p[P2]), f[c], L.h2, r[c]);
+        v[c] = omega == 1.0f ? gs : __fmaf_rn(omega, __fsub_rn(gs, v[c]), v[c]);
+        u[at[c]] = v[c];
+      }
+      cl_bar(3, n);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+    if (on[c]) lin[2 * threadIdx.x + c] = v[c];
+}
+
+// (by cl_bottom_threads(S, periodic) threads)
 __device__ void cl_bottom_s(int S, int periodic, float* u, const FcLev& L, int sweeps,
                             float sig0) {
   if (periodic) {
@@ -155,8 +206,7 @@ __device__ void cl_bottom_s(int S, int periodic, float* u, const FcLev& L, int s
   } else {
     if (S == 4) cl_bottom<4, false>(u, L, sweeps, sig0);
     else if (S == 3) cl_bottom<3, false>(u, L, sweeps, sig0);
-    else if (S == 5) cl_bottom<5, false>(u, L, sweeps, sig0);
-    else if (S == 7) cl_bottom<7, false>(u, L, sweeps, sig0);
+    else if (cl_wide(S, 0)) cl_bottom_wide(S, u, L, sweeps);
     else cl_bottom<2, false>(u, L, sweeps, sig0);
   }
 }
@@ -171,23 +221,25 @@ __device__ __forceinline__ FcLev cl_lev(int level, int periodic, float sig0) {
   return L;
 }
 
-// a top that is a bottom itself (side 2 to 5 or 7), by one warp
+// a top that is a bottom itself (side 2 to 5 or 7), by its bottom's threads
 __device__ __noinline__ void cl_only_bottom(float* sm, const Grid& gu, const Grid& gb, int level,
                                             int periodic, int sweeps, int zero_top,
                                             float sig0) {
-  const int S = gu.s, P = S + 2, N = S * S * S, lane = (int)threadIdx.x;
+  const int S = gu.s, P = S + 2, N = S * S * S, t0 = (int)threadIdx.x;
+  const int n = cl_bottom_threads(S, periodic);
   float *b = sm + P * P * P, *lin = b + N;
-  for (int t = lane; t < P * P * P; t += 32) {
+  for (int t = t0; t < P * P * P; t += n) {
     const int i = t % P - 1, j = (t / P) % P - 1, k = t / (P * P) - 1;
     const int out = (i < 0 || i >= S) + (j < 0 || j >= S) + (k < 0 || k >= S);
     const bool rd = out == 0 ? !zero_top : (out == 1 && !periodic);
     sm[t] = rd ? gu.base[gidx(gu, i, j, k)] : 0.0f;
   }
-  for (int t = lane; t < N; t += 32)
+  for (int t = t0; t < N; t += n)
     b[t] = gb.base[gidx(gb, t % S, (t / S) % S, t / (S * S))];
-  __syncwarp();
+  cl_bar(3, n);
   cl_bottom_s(S, periodic, sm, cl_lev(level, periodic, sig0), sweeps, sig0);
-  for (int t = lane; t < N; t += 32)  // (lin[t] is this lane's own store)
+  cl_bar(3, n);
+  for (int t = t0; t < N; t += n)
     gu.base[gidx(gu, t % S, (t / S) % S, t / (S * S))] = lin[t];
 }
 
@@ -380,7 +432,7 @@ __device__ __forceinline__ void cl_vcycle(float* sm, const Grid& gu, const Grid&
     if (q + 1 == nl || t >= cl_threads(C0)) break;
     place(++q);
   }
-  if (q + 1 == nl && t < 32) {
+  if (q + 1 == nl && t < cl_bottom_threads(Sb, periodic)) {
     cl_bottom_s(Sb, periodic, bot, cl_lev(level + nl, periodic, sig0), sweeps, sig0);
   }
   // up: the level below has left its result in x order

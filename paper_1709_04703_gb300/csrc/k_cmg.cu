@@ -84,7 +84,7 @@ __device__ __forceinline__ void cmg_one(float* sm, const Grid& u, const Grid& b,
                                         int periodic, int sweeps, int zero_top, float sig0) {
   if (cl_supported(u.s))
     cl_vcycle(sm, u, b, level, periodic, sweeps, zero_top, sig0);
-  else if (threadIdx.x < 32)
+  else if ((int)threadIdx.x < cl_bottom_threads(u.s, periodic))
     cl_only_bottom(sm, u, b, level, periodic, sweeps, zero_top, sig0);
 }
 __global__ void __launch_bounds__(CL_NT) k_cmg_col(Grid u, Grid b, int level, int periodic,
@@ -223,7 +223,8 @@ void launch_cmg(cudaStream_t st, Grid u, Grid b, int level, int periodic, int sw
       break;
     default:
       if (!u.mbase && g_cmg_fast && fc_supported(u.s))
-        launch_pdl(k_cmg_col, dim3(1), dim3(cl_supported(u.s) ? cl_threads(u.s) : 32),
+        launch_pdl(k_cmg_col, dim3(1), dim3(cl_supported(u.s) ? cl_threads(u.s)
+                                                        : cl_bottom_threads(u.s, periodic)),
                    sizeof(float) * CL_SMEM, st, u, b, level, periodic, sweeps, z, sig0);
       else
         cmg_launch<1>(k_cmg<1>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0);

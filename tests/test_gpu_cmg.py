@@ -157,3 +157,32 @@ def test_constant_side_coarse_form_run_is_bitwise():
     b = _with_cluster(False, lambda: _with_generic(True, run))
     for u, v in zip(a, b):
         np.testing.assert_array_equal(u, v)
+
+
+def test_an_odd_bottom_is_no_slower_than_a_larger_even_one():
+    """The V-cycle's bottom runs on every open cube of side 5 * 2^j or 7 * 2^j
+    from tops of 10 and 14 (odd bottoms 5 and 7).  Its device time there
+    stays below 1.25 times that of the larger top 16, whose chain of passes is
+    longer by a level (one warp on the odd bottom: 1.8 and 1.1 times)."""
+    from paper_1709_04703_gb300.sim import Sim
+
+    def bottom(side):
+        # a 16^3 mesh in its open phase: the whole V-cycle is the bottom
+        n, R = 16, {16: 6.5, 14: 5.6, 10: 3.6}[side]
+        pos, mom, ids = ics.random_particles(500, n, 3, 6.0, 10.0, 1e-4)
+        from oracle import cosmology as cz
+        box = float(cz.chi(0.5, 0.3, 0.7)) * n / (R - 1.0)
+        sim = Sim(pos, mom, ids, n, box, 0.5, 1.0, 10000, rtol=1e-6, guess="zero")
+        best = 1e9
+        for _ in range(6):
+            sim.profile(True)
+            sim.step(5)
+            p = sim.profile_read()["coarse"]
+            best = min(best, p["ms"] / p["groups"])
+        s = sim.stats()
+        assert s["cube_side"] == side and not s["periodic"]
+        sim.close()
+        return best
+    ref = bottom(16)
+    for side in (14, 10):
+        assert bottom(side) < 1.25 * ref, (side, ref)
