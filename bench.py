@@ -162,8 +162,8 @@ ARITHMETIC = {
                "particles, int64 density",
 }
 
-# ncu dram__bytes_read.sum + dram__bytes_write.sum over the algorithmic bytes
-# of the kernel class's launches at 256^3 on the current kernels
+# ncu dram__bytes_read.sum + dram__bytes_write.sum over the bytes that the
+# class's launches must move (pm_profile_read) at 256^3
 TRAFFIC_RATIO = {
     # the fused leg down must move 8.5 B per cell, the two-sweep pass up 12
     "smooth0": ((71951616 + 31623424 + 152123904 + 36274176) / (20.5 * 256**3),
@@ -171,8 +171,8 @@ TRAFFIC_RATIO = {
     "defect": ((273779712 + 50797824 + 347053312 + 169682688) / (335.5e6 + 536.9e6),
                "k_defect<0> + k_defect<1> at 256^3, profiles/kernels_pm256.md"),
     "deposit": (1127.9e6 / 1073.7e6, "k_drift_deposit at 256^3, profiles/kernels_pm256.md"),
-    "gather": (1294.6e6 / 1342.2e6, "k_gather_kick_drift at 256^3, "
-               "profiles/defect_gather_deposit_pm256.md"),
+    "gather": ((139764480 + 214919168 + 808541440 + 482791680) / (104.0 * 256**3),
+               "k_grad + k_gather_kick_drift at 256^3, profiles/kernels_pm256.md"),
 }
 
 
@@ -687,8 +687,7 @@ def run_ours(args):
     # the same windows again, one step at a time, with CUDA events around
     # every kernel class on the context's stream: per-class device time and
     # algorithmic bytes (the events cost a few % of the step, so the
-    # headline comes from the uninstrumented run above), and per step the
-    # active particles N, cells C and V-cycles k for the whole-step count
+    # headline comes from the uninstrumented run above)
     sim = _new_sim(pos, mom, ids, cfg, rtol, args.precision)
     prof, seen = None, 0
     p0 = time.perf_counter()

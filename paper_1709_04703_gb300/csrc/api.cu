@@ -1283,10 +1283,9 @@ pm_status solve(pm_ctx* ctx) {
     // one is expected to take it too: where that is one more than have run,
     // the V-cycle and its defect are queued before the residuals are read,
     // both in one read (a host round trip leaves the GPU idle for 15 to 20
-    // us).
-    // They write the correction, r and the other potential buffer, none of
-    // which is used if the solve turns out to have converged before: the same
-    // V-cycles, the same bits.
+    // us).  They write the correction, r and the other potential buffer, none
+    // of which is used if the solve turns out to have converged before: the
+    // same V-cycles, the same bits.
     const bool ahead = mixed && !net_todo && !capture && ctx->vc_same >= VC_SAME &&
                        it + 1 == ctx->vc_prev && it < ctx->cfg.max_vcycles;
     if (ahead) {

@@ -299,14 +299,18 @@ long long cf_blocks(const CfShape& s, int B, int S) {
          ((S + s.tz - 1) / s.tz);
 }
 
-// The block for B samples of side S.  An MMA of 128 rows takes 64 cycles
-// whatever its columns, and an M tile's rows on the halo are lost: 8^3 blocks
-// (57 % of the rows are outputs) against 16 x 16 x 2 or 20 x 10 x 2 (80 %).
-// So of the blocks that fit, the one whose busiest SM takes the fewest
-// cycles, counting MMAs, staged 16-byte pieces and a start per block, the two
-// overlapped where several blocks share an SM.  Every block gives a voxel the
-// same MMAs in the same order: the same bits.  160^3 forward, layers of 16
-// columns: 1283 us with 8^3 blocks, 996 so.
+// The block for B samples of side S.  An MMA of 128 rows hardly depends on its
+// columns (39, 40, 44, 48 cycles an SM for 16, 32, 48, 64 in chains of several
+// CTAs, 50 in one CTA alone), and an M tile's rows on the halo are lost: 8^3
+// blocks (57 % of the rows are outputs) against 16 x 16 x 2 or 20 x 10 x 2
+// (80 %).  So of the blocks that fit, the one whose busiest SM takes the
+// fewest cycles by a model of MMAs, staged 16-byte pieces and a start per
+// block, the two overlapped where several blocks share an SM.  Its weights
+// (64, 1.2, 2000, 0.25) are chosen by whole passes and matter little: from 39
+// to 64, 0.8 to 1.8, 1000 to 4000 and 0 to 1 a forward or backward pass at ten
+// sides of 32 to 192 moved by 5 % at most.  Every block gives a voxel the same
+// MMAs in the same order: the same bits.  160^3 forward, layers of 16 columns:
+// 1283 us with 8^3 blocks, 996 so.
 CfShape cf_choose(int B, int S, int cin, int n, int T) {
   struct Entry {
     int B, S, cin, n;

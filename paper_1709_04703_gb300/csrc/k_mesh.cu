@@ -320,8 +320,13 @@ __device__ __forceinline__ void tsc_axis(float u, int& i, unsigned int w[3]) {
 // later lane adds the earlier ones' parts to its own (from their weights, 16
 // shuffles in all, not from the 27 products).  A chain of such lanes issues
 // one atomic per row and lane, and the last lane's two outer nodes: 9.6 per
-// particle instead of 27 on a lattice (2.1 million particles, 128^3: 82 -> 52
-// us).  Integer sums: any order gives the same counts.
+// particle instead of 27 on a lattice.  Where nothing links, the shuffles hide
+// behind the atomics.  Integer sums: any order gives the same counts.  us per
+// deposit without -> with (lattice; clustered particles in lattice, cell and
+// random order):
+//   2.1 million, 128^3    77 ->  47   127 -> 105    156 ->  144    244 ->  242
+//   6.3 million, 192^3                365 -> 298    452 ->  414    725 ->  716
+//   16.8 million, 256^3  570 -> 369   960 -> 779   1195 -> 1095   3478 -> 3494
 template <bool DRIFT>
 __global__ void __launch_bounds__(256) k_drift_deposit_tsc(
     float4* __restrict__ pos, const float4* __restrict__ mom, long long N, float c0, int n,

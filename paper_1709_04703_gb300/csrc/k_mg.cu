@@ -625,26 +625,6 @@ void launch_defect(cudaStream_t st, Grid ph, Grid pl, const Grid* e, Grid qh, Gr
   note_launch();
 }
 
-// Phi (hi, lo) += e.
-__global__ void __launch_bounds__(256) k_correct(Grid ph, Grid pl, Grid e) {
-  pdl_wait();
-  pdl_release();
-  const int s = ph.s;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  int k = blockIdx.z;
-  if (i >= s || j >= s) return;
-  int c = gidx(ph, i, j, k);
-  df v = df_add(df{ph.base[c], pl.base[c]}, df{e.base[gidx(e, i, j, k)], 0.0f});
-  ph.base[c] = v.hi;
-  pl.base[c] = v.lo;
-}
-
-void launch_correct(cudaStream_t st, Grid ph, Grid pl, Grid e) {
-  launch_pdl(k_correct, grid_full(ph.s), dim3(32, 8), 0, st, ph, pl, e);
-  note_launch();
-}
-
 // Dense [z][y][x] FP32 arrays of side s <-> grid interiors (the learned
 // guess and training-pair capture).  to_dense: d (=|+=) g; from_dense:
 // g (=|+=) d.

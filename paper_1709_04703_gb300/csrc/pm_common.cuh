@@ -327,9 +327,10 @@ struct BTable {
   int off[MAX_MEMBERS + 1];    // cumulative block counts
 };
 
-// Planes per block of the batched mesh passes (colour pass, restriction,
-// prolongation, warm-start prediction, gradient field): a block's table lookup is shared by
-// BZ planes of its (x, y) tile.
+// Planes per block of the batched mesh passes (warm-start prediction and
+// gradient field, and in the persistent solve the colour passes and
+// transfers): a block's table lookup is shared by BZ planes of its (x, y)
+// tile.
 constexpr int BZ = 4;
 template <class F>
 __device__ __forceinline__ void each_plane(const BI& bi, int nz, F&& f) {

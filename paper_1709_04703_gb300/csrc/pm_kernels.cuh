@@ -141,7 +141,6 @@ void launch_defect(cudaStream_t st, Grid ph, Grid pl, const Grid* e, Grid qh, Gr
                    Grid fh, Grid fl, Grid rb, int periodic, bool write_r, double* partial,
                    unsigned int* counter, double* out, double d0 = 6.0);
 int defect_blocks(int s);
-void launch_correct(cudaStream_t st, Grid ph, Grid pl, Grid e);
 void launch_to_dense(cudaStream_t st, Grid g, float* d, bool add);
 void launch_from_dense(cudaStream_t st, const float* d, Grid g, bool add);
 void launch_predict(cudaStream_t st, Grid ph, Grid pl, Grid qh, Grid ql, float w, bool pair);
