@@ -288,10 +288,12 @@ __global__ void k_pack_wf(const float* __restrict__ w, int cin, int cout, int n,
 
 constexpr int CF_SMEM_MAX = 200 * 1024;
 
+// the most that any launch takes, not this one's: another thread may set it
+// between the setting and the launch
 template <int N>
-bool cf_set_attr(int smem) {
+bool cf_set_attr() {
   return cudaFuncSetAttribute(k_conv_fast<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              smem) == cudaSuccess;
+                              CF_SMEM_MAX) == cudaSuccess;
 }
 
 long long cf_blocks(const CfShape& s, int B, int S) {
@@ -381,7 +383,7 @@ bool launch_conv_fast(cudaStream_t st, const void* in, int B, int S, int per, in
   const CfShape sh = cf_choose(B, S, cin, n, T);
   const dim3 grid((unsigned)cf_blocks(sh, B, S));
 #define PM_CF(NN)                                                                       \
-  if (!cf_set_attr<NN>(sh.smem)) return false;                                          \
+  if (!cf_set_attr<NN>()) return false;                                                 \
   k_conv_fast<NN><<<grid, CF_NT, sh.smem, st>>>((const bf16*)in, B, S, per, cin,          \
                                                  (const bf16*)wf, sh, bias, cout, relu,    \
                                                  (bf16*)out_bf, out_f, err,                \

@@ -146,6 +146,7 @@ __device__ __forceinline__ df df_shfl_down(df a, int o) {
 }
 
 constexpr int PK_NT = 256, PK_WARPS = PK_NT / 32;
+constexpr size_t PK_SMEM = 200 * 1024;  // at most; one warp's part of 2048 bins is 66 KB
 // shared floats of a warp: per bin the count, sum |k| (three floats), sum P
 // (and sum C1/C2) as pairs; with aliases each lane's x factors
 __host__ __device__ constexpr int pk_warp_floats(int n_bins, int m) {
@@ -324,10 +325,12 @@ template <int m>
 static cudaError_t pk_launch(cudaStream_t st, const float2* dk, int n, double box, double shot,
                              int n_bins, const void* tab, const double* nu, double* acc) {
   const size_t per = sizeof(float) * pk_warp_floats(n_bins, m);
-  const int nw = (int)std::max<size_t>(1, std::min<size_t>(PK_WARPS, (size_t)200 * 1024 / per));
+  const int nw = (int)std::max<size_t>(1, std::min<size_t>(PK_WARPS, PK_SMEM / per));
   if (per * nw > 48 * 1024) {
+    // (the most that any launch takes, not this one's: another thread may set
+    // it between the setting and the launch)
     const cudaError_t e = cudaFuncSetAttribute(
-        k_pk_modes<m>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per * nw));
+        k_pk_modes<m>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PK_SMEM);
     if (e != cudaSuccess) return e;
   }
   const long long rows = (long long)(n / 2 + 1) * (n / 2 + 1);

@@ -199,8 +199,11 @@ template <int NT>
 cudaError_t wg_launch(cudaStream_t st, const void* in, int B, int S, int per, int cin, int cgp,
                       const void* dy, int cout, float* dw, float* db) {
   const int smem = (cgp + NT) * WG_ROWS * 16 + 256;
-  const cudaError_t e = cudaFuncSetAttribute(
-      k_wgrad<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // (the most that any launch takes, not this one's: another thread may set it
+  // between the setting and the launch)
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_wgrad<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (WG_CG + NT) * WG_ROWS * 16 + 256);
   if (e != cudaSuccess) return e;
   const long long t = (S + WG_T - 1) / WG_T, nblk = t * t * t * B;
   const int gy = cin / 8 / cgp, gz = cout / 8 / NT;

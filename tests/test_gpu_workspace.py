@@ -172,3 +172,71 @@ def test_release_work_gives_the_memory_back():
     release_work()  # (nothing left: fine)
     for a, b in zip(power_spectrum(points, 100.0, 256, 4), ref):
         np.testing.assert_allclose(a, b, rtol=1e-12)
+
+
+def _in_threads(jobs):
+    bad = []
+
+    def work(job):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                job()
+        except Exception as e:  # noqa: BLE001 - reported below
+            bad.append(e)
+    ts = [threading.Thread(target=work, args=(j,)) for j in jobs]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad, bad[0]
+
+
+def test_spectra_of_many_bins_in_threads():
+    """Spectra whose binning takes different amounts of shared memory (57 to
+    196 KB a block) from eight threads: a launch must not be refused because
+    another thread has asked for less in between (it happened in about one of
+    50 launches that met)."""
+    import ctypes as C
+    from paper_1709_04703_gb300 import _lib as L
+    from paper_1709_04703_gb300.sim import power_spectrum
+    lib = L.load()
+    p4, _ = _points(8, 500, 3)
+    ref = power_spectrum(p4, 100.0, 8, 300)
+
+    def job(bins):
+        def run():
+            out = [np.zeros(bins) for _ in range(3)]
+            args = (C.c_void_p(p4.data_ptr()), 500, 100.0, 8, bins, 1,
+                    *(C.c_void_p(o.ctypes.data) for o in out),
+                    C.c_void_p(torch.cuda.current_stream().cuda_stream))
+            codes = [lib.pm_power_spectrum(*args) for _ in range(2000)]
+            assert codes.count(L.PM_OK) == len(codes), codes.count(L.PM_OK)
+            np.testing.assert_array_equal(out[2][:300], ref[2])
+            has = ref[2] > 0
+            np.testing.assert_allclose(out[1][:300][has], ref[1][has], rtol=1e-12)
+        return run
+    _in_threads([job(b) for b in (300, 700, 1000, 2048) * 2])
+
+
+def test_networks_in_threads():
+    """Four networks forward and backward at once, each in its own thread:
+    their layers' staged blocks differ in size."""
+    from paper_1709_04703_gb300.guess import GuessNet
+    f = _field()
+    nets = [GuessNet(levels=3, seed=3) for _ in range(4)]
+    want = [nets[0].forward(f, 1).cpu().numpy(), nets[0].loss_grad(f, 2 * f, 1, 0), nets[0].grad()]
+    g2 = 2 * f
+    torch.cuda.synchronize()
+
+    def job(net):
+        def run():
+            for _ in range(60):
+                loss = net.loss_grad(f, g2, 1, 0)
+                assert loss == pytest.approx(want[1], rel=1e-6)
+            grad = net.grad()  # FP32 sums by atomics
+            np.testing.assert_allclose(grad, want[2], rtol=1e-4, atol=1e-6 * np.abs(want[2]).max())
+            out = net.forward(f, 1)
+            net.stream.synchronize()
+            np.testing.assert_array_equal(out.cpu().numpy(), want[0])
+        return run
+    _in_threads([job(n) for n in nets])
