@@ -12,7 +12,7 @@
 // each level is a named barrier over the warps it needs.  The bottom itself
 // (side <= 4 or odd) belongs to one warp, where it is open and of side 5 or 7
 // to a thread per cell of a colour (one warp took 11 trips a pass for the 343
-// cells: inside open steps a top of 14 37.4 us, of 10 20.7; so 14.4 and 13.0);
+// cells: inside open steps a top of 14 37.4 us, of 10 20.7; so 14.1 and 13.0);
 // its lexicographic sweep on odd periodic sides runs the diagonal fronts in
 // parallel.  The operations and their order are those of cmg_fast.cuh, through
 // mg_arith.cuh: the same bits.
@@ -46,12 +46,13 @@ __device__ __forceinline__ void cl_bar(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// threads that work on the bottom of side S
+// whether a thread per cell of a colour works on the bottom under a top of side
+// S (open, the bottom's side 5 or 7; else one warp), and its threads then
 __host__ __device__ constexpr bool cl_wide(int S, int periodic) {
-  return !periodic && (S == 5 || S == 7);
+  return !periodic && (S == 5 || S == 7 || S == 10 || S == 14);
 }
-__host__ __device__ constexpr int cl_bottom_threads(int S, int periodic) {
-  return cl_wide(S, periodic) ? (S * S * S / 2 + 1 + 31) / 32 * 32 : 32;
+__host__ __device__ constexpr int cl_wide_threads(int S) {
+  return (S * S * S / 2 + 1 + 31) / 32 * 32;
 }
 
 // the cells lane, lane + 32, ... of an S^3 level in x order, by their
@@ -159,7 +160,7 @@ __device__ __noinline__ void cl_bottom(float* u, const FcLev& L, int sweeps, flo
 // order, thread e the e-th of each, with their values in registers.  The
 // barrier is the bottom's own (3).
 __device__ __noinline__ void cl_bottom_wide(int S, float* u, const FcLev& L, int sweeps) {
-  const int P = S + 2, P2 = P * P, N = S * S * S, n = cl_bottom_threads(S, 0);
+  const int P = S + 2, P2 = P * P, N = S * S * S, n = cl_wide_threads(S);
   float *b = u + P * P2, *lin = b + N;
   int at[2];
   bool on[2];
@@ -194,7 +195,6 @@ __device__ __noinline__ void cl_bottom_wide(int S, float* u, const FcLev& L, int
     if (on[c]) lin[2 * threadIdx.x + c] = v[c];
 }
 
-// (by cl_bottom_threads(S, periodic) threads)
 __device__ void cl_bottom_s(int S, int periodic, float* u, const FcLev& L, int sweeps,
                             float sig0) {
   if (periodic) {
@@ -206,7 +206,6 @@ __device__ void cl_bottom_s(int S, int periodic, float* u, const FcLev& L, int s
   } else {
     if (S == 4) cl_bottom<4, false>(u, L, sweeps, sig0);
     else if (S == 3) cl_bottom<3, false>(u, L, sweeps, sig0);
-    else if (cl_wide(S, 0)) cl_bottom_wide(S, u, L, sweeps);
     else cl_bottom<2, false>(u, L, sweeps, sig0);
   }
 }
@@ -221,12 +220,14 @@ __device__ __forceinline__ FcLev cl_lev(int level, int periodic, float sig0) {
   return L;
 }
 
-// a top that is a bottom itself (side 2 to 5 or 7), by its bottom's threads
+// a top that is a bottom itself (side 2 to 5 or 7): one warp, or WIDE
+// cl_wide_threads
+template <bool WIDE>
 __device__ __noinline__ void cl_only_bottom(float* sm, const Grid& gu, const Grid& gb, int level,
                                             int periodic, int sweeps, int zero_top,
                                             float sig0) {
   const int S = gu.s, P = S + 2, N = S * S * S, t0 = (int)threadIdx.x;
-  const int n = cl_bottom_threads(S, periodic);
+  const int n = WIDE ? cl_wide_threads(S) : 32;
   float *b = sm + P * P * P, *lin = b + N;
   for (int t = t0; t < P * P * P; t += n) {
     const int i = t % P - 1, j = (t / P) % P - 1, k = t / (P * P) - 1;
@@ -237,14 +238,18 @@ __device__ __noinline__ void cl_only_bottom(float* sm, const Grid& gu, const Gri
   for (int t = t0; t < N; t += n)
     b[t] = gb.base[gidx(gb, t % S, (t / S) % S, t / (S * S))];
   cl_bar(3, n);
-  cl_bottom_s(S, periodic, sm, cl_lev(level, periodic, sig0), sweeps, sig0);
+  if (WIDE) cl_bottom_wide(S, sm, cl_lev(level, periodic, sig0), sweeps);
+  else cl_bottom_s(S, periodic, sm, cl_lev(level, periodic, sig0), sweeps, sig0);
   cl_bar(3, n);
   for (int t = t0; t < N; t += n)
     gu.base[gidx(gu, t % S, (t / S) % S, t / (S * S))] = lin[t];
 }
 
 // the V-cycle from an unmasked even top of side S0 (cl_supported) in one CTA
-// of at least cl_threads(S0) threads; sm holds cl_floats(S0) floats
+// of at least cl_threads(S0) threads; sm holds cl_floats(S0) floats.  WIDE as
+// cl_wide(S0): a form of its own, since the test in the other one's code cost
+// every V-cycle 0.8 us.
+template <bool WIDE>
 __device__ __forceinline__ void cl_vcycle(float* sm, const Grid& gu, const Grid& gb, int level,
                                           int periodic, int sweeps, int zero_top, float sig0) {
   const int t = (int)threadIdx.x;
@@ -432,7 +437,10 @@ __device__ __forceinline__ void cl_vcycle(float* sm, const Grid& gu, const Grid&
     if (q + 1 == nl || t >= cl_threads(C0)) break;
     place(++q);
   }
-  if (q + 1 == nl && t < cl_bottom_threads(Sb, periodic)) {
+  if (WIDE) {
+    if (q + 1 == nl && t < cl_wide_threads(Sb))
+      cl_bottom_wide(Sb, bot, cl_lev(level + nl, periodic, sig0), sweeps);
+  } else if (q + 1 == nl && t < 32) {
     cl_bottom_s(Sb, periodic, bot, cl_lev(level + nl, periodic, sig0), sweeps, sig0);
   }
   // up: the level below has left its result in x order

@@ -80,19 +80,21 @@ __global__ void __launch_bounds__(CC_NT, 1) kb_cmg(const CmgDesc* d, int n_desc,
 
 // one CTA from an unmasked top <= 16 (cmg_col.cuh), and its batched form:
 // CTA c takes table entry c
+template <bool WIDE>
 __device__ __forceinline__ void cmg_one(float* sm, const Grid& u, const Grid& b, int level,
                                         int periodic, int sweeps, int zero_top, float sig0) {
   if (cl_supported(u.s))
-    cl_vcycle(sm, u, b, level, periodic, sweeps, zero_top, sig0);
-  else if ((int)threadIdx.x < cl_bottom_threads(u.s, periodic))
-    cl_only_bottom(sm, u, b, level, periodic, sweeps, zero_top, sig0);
+    cl_vcycle<WIDE>(sm, u, b, level, periodic, sweeps, zero_top, sig0);
+  else if ((int)threadIdx.x < (WIDE ? cl_wide_threads(u.s) : 32))
+    cl_only_bottom<WIDE>(sm, u, b, level, periodic, sweeps, zero_top, sig0);
 }
+template <bool WIDE>
 __global__ void __launch_bounds__(CL_NT) k_cmg_col(Grid u, Grid b, int level, int periodic,
                                                    int sweeps, int zero_top, float sig0) {
   extern __shared__ float cc_sm[];
   pdl_wait();
   pdl_release();
-  cmg_one(cc_sm, u, b, level, periodic, sweeps, zero_top, sig0);
+  cmg_one<WIDE>(cc_sm, u, b, level, periodic, sweeps, zero_top, sig0);
 }
 __global__ void __launch_bounds__(CL_NT) kb_cmg_col(const CmgDesc* d, int n_desc,
                                                     const int* active) {
@@ -101,7 +103,11 @@ __global__ void __launch_bounds__(CL_NT) kb_cmg_col(const CmgDesc* d, int n_desc
   if (q >= n_desc) return;
   const CmgDesc& e = d[q];
   if (active && !active[e.r]) return;
-  cmg_one(cc_sm, in_global(e.u), in_global(e.b), e.level, e.periodic, e.sweeps, e.zero_top, 0.0f);
+  const Grid u = in_global(e.u), b = in_global(e.b);
+  if (cl_wide(u.s, e.periodic))
+    cmg_one<true>(cc_sm, u, b, e.level, e.periodic, e.sweeps, e.zero_top, 0.0f);
+  else
+    cmg_one<false>(cc_sm, u, b, e.level, e.periodic, e.sweeps, e.zero_top, 0.0f);
 }
 
 int g_cmg_cl = 1;  // CTAs per cluster of this process's launches (set by cmg_prepare)
@@ -184,7 +190,9 @@ cudaError_t cmg_prepare() {
   cudaError_t e = cmg_attrs<1>();
   const int col = (int)sizeof(float) * CL_SMEM;
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cmg_col, cudaFuncAttributeMaxDynamicSharedMemorySize, col);
+    e = cudaFuncSetAttribute(k_cmg_col<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, col);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_cmg_col<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, col);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kb_cmg_col, cudaFuncAttributeMaxDynamicSharedMemorySize, col);
   if (e != cudaSuccess) return e;
@@ -222,12 +230,14 @@ void launch_cmg(cudaStream_t st, Grid u, Grid b, int level, int periodic, int sw
       cmg_launch<8>(k_cmg<8>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0);
       break;
     default:
-      if (!u.mbase && g_cmg_fast && fc_supported(u.s))
-        launch_pdl(k_cmg_col, dim3(1), dim3(cl_supported(u.s) ? cl_threads(u.s)
-                                                        : cl_bottom_threads(u.s, periodic)),
+      if (!u.mbase && g_cmg_fast && fc_supported(u.s)) {
+        const bool wide = cl_wide(u.s, periodic);
+        launch_pdl(wide ? k_cmg_col<true> : k_cmg_col<false>, dim3(1),
+                   dim3(cl_supported(u.s) ? cl_threads(u.s) : (wide ? cl_wide_threads(u.s) : 32)),
                    sizeof(float) * CL_SMEM, st, u, b, level, periodic, sweeps, z, sig0);
-      else
+      } else {
         cmg_launch<1>(k_cmg<1>, 1, u.s, st, u, b, level, periodic, sweeps, z, sig0);
+      }
       break;
   }
   note_launch();
